@@ -58,8 +58,9 @@ static void dfree(T*& p) {
 
 static void free_check(bv_ctx* c) {
     auto& k = c->chk;
-    for (auto& b : k.sbins) dfree(b.d_work);
+    for (auto& b : k.sbins) dfree(b.d_work);  // (their workspace slots are the redo bins')
     k.sbins.clear();
+    for (auto& b : k.rbins) dfree(b.d_slots);
     k.rbins.clear();  // their lists live inside d_redo
     dfree(k.d_samp);
     dfree(k.d_samp_ptr);
@@ -77,7 +78,10 @@ static void free_check(bv_ctx* c) {
 
 static void free_plan(bv_ctx* c, int prec) {
     if (prec == BV_MIXED) free_check(c);
-    for (auto& b : c->plan[prec]) dfree(b.d_work);
+    for (auto& b : c->plan[prec]) {
+        dfree(b.d_work);
+        dfree(b.d_slots);
+    }
     c->plan[prec].clear();
     c->plan_valid[prec] = false;
     c->tuned[prec] = false;
@@ -257,6 +261,15 @@ extern "C" int bv_create(bv_ctx** out, int device, void* stream) {
     if (e == cudaSuccess) e = cudaMallocHost(&c->h_fail, sizeof(unsigned long long));
     if (e == cudaSuccess) e = cudaMallocHost(&c->h_fb, sizeof(int));
     if (e == cudaSuccess) *c->h_fb = 0;
+    if (e == cudaSuccess) e = cudaMalloc(&c->d_fixtab, sizeof(uint64_t) * 512);
+    if (e == cudaSuccess) {
+        static const std::vector<uint64_t> tab = [] {
+            std::vector<uint64_t> t(512);
+            bv_fix_tables(t.data());
+            return t;
+        }();
+        e = cudaMemcpy(c->d_fixtab, tab.data(), sizeof(uint64_t) * 512, cudaMemcpyHostToDevice);
+    }
     if (e != cudaSuccess) {
         bv_record_cuda_error(e, "bv_create", __FILE__, __LINE__);
         bv_destroy(c);
@@ -275,6 +288,7 @@ extern "C" void bv_destroy(bv_ctx* c) {
     free_data(c);
     dfree(c->d_fail);
     dfree(c->d_wctr);
+    dfree(c->d_fixtab);
     dfree(c->d_ws);
     for (auto s : c->side) cudaStreamDestroy(s);
     for (auto e : c->side_ev) cudaEventDestroy(e);
@@ -319,7 +333,7 @@ extern "C" int bv_set_datasets(bv_ctx* c, int32_t ndata, const int64_t* n_per, c
     BV_CUDA(cudaMalloc(&c->d_quad, sizeof(double) * ndata));
     BV_CUDA(cudaMallocHost(&c->h_quad, sizeof(double) * ndata));
     BV_CUDA(cudaMalloc(&c->d_theta, sizeof(DevTheta) * ndata));
-    BV_CUDA(cudaMalloc(&c->d_gtab, sizeof(double) * BV_GTAB_DOUBLES * ndata));
+    BV_CUDA(cudaMalloc(&c->d_gtab, sizeof(double) * 2 * BV_GTAB_DOUBLES * ndata));
     BV_CUDA(cudaMallocHost(&c->h_out, sizeof(double) * ndata));
     c->h_theta.assign(ndata, DevTheta{});
     BV_CUDA(cudaMemcpyAsync(c->d_locs, soa.data(), sizeof(double) * n_tot * d, cudaMemcpyHostToDevice,
@@ -751,14 +765,18 @@ int bv_theta_to_dev(const bv_theta* t, int d, DevTheta* o) {
     const float d32 = o->sigma2_f + o->nugget_f;
     o->diag_lo_f = (float)((o->sigma2 + o->nugget) - (double)d32);
     for (int k = 0; k < 3; ++k) o->inv_range_f[k] = (float)o->inv_range[k];
+    o->diag = o->sigma2 + o->nugget;
+    o->diag_ratio = o->sigma2 / o->diag;
+    o->diag_rsqrt = 1.0 / std::sqrt(o->diag);
     return BV_OK;
 }
 
 static const int kBinEdges[] = {16, 32, 48, 64, 80, 96, 112, 128, 160, 192, 224, 256, 288, 320};
 
-// CTA sizes of the shared-memory kernels: one panel warp plus 2, 4, 8 or 16 update warps.
-static int default_threads(int kind, int nmax) {
+// CTA sizes: the mixed kernel's one panel warp plus 2, 4, 8 or 16 update warps.
+static int default_threads(const bv_ctx* c, int kind, int nmax, int nwork) {
     if (kind == 2) return 256;
+    if (kind == 7 || kind == 8) return bv_fix_threads(nmax, nwork, c->num_sms);
     if (nmax <= 48) return 96;
     if (nmax <= 128) return 160;
     return 288;
@@ -788,12 +806,33 @@ static LLArgs make_args(bv_ctx* c) {
     a.fail = c->d_fail;
     a.ws = c->d_ws;
     a.ws_stride = c->ws_stride;
+    a.fixtab = c->d_fixtab;
     a.gen = c->cur_gen ? 1 : 0;
     a.fb = nullptr;
     a.dyn = 0;
     a.gtab = c->d_gtab;
+    a.gtabi = reinterpret_cast<const int64_t*>(c->d_gtab) + (int64_t)BV_GTAB_DOUBLES * c->ndata;
     bv_exp_consts(&a.ex);
     return a;
+}
+
+// Bin edges of the fixed-point FP64 kernel: a block of N points has (N + 16) / 16 tile rows,
+// so a bin of N = 16 k .. 16 k + 15 holds blocks of one shared-memory footprint; four tile
+// rows to a bin beyond N = 255, where few blocks lie.
+static std::vector<int> fix_edges(int d) {
+    const int nsm = bv_fix_max_n(d);
+    std::vector<int> edges;
+    for (int e = 15; e < nsm; e += e < 255 ? 16 : 64) edges.push_back(e);
+    edges.push_back(nsm);
+    return edges;
+}
+
+// Workspace slots of a kind-8 bin, one per CTA of its grid.
+static int alloc_slots(BinPlan& bp) {
+    if (bp.kind != 8) return BV_OK;
+    bp.slot_stride = (int64_t)(bv_fix_slot_bytes(bp.nmax) / sizeof(double));
+    BV_CUDA(bv_plan_malloc(&bp.d_slots, sizeof(double) * bp.slot_stride * bp.grid));
+    return BV_OK;
 }
 
 static int set_grid(bv_ctx* c, BinPlan& bp) {
@@ -821,11 +860,7 @@ static const int64_t kChkMinSamples = 64, kChkFrac = 256;
 static int build_check(bv_ctx* c, const std::vector<int>& Nof) {
     free_check(c);
     auto& k = c->chk;
-    const int nsm = bv_smem_max_n(0, c->d);
-    std::vector<int> edges;
-    for (int e : kBinEdges)
-        if (e < nsm) edges.push_back(e);
-    edges.push_back(nsm);
+    const std::vector<int> edges = fix_edges(c->d);
     const size_t nbin = edges.size() + 1;
     std::vector<int32_t> bin_of(c->nblk);
     std::vector<std::vector<int32_t>> all(nbin), smp(nbin);
@@ -877,11 +912,10 @@ static int build_check(bv_ctx* c, const std::vector<int>& Nof) {
         int nmax = 0;
         for (int32_t i : all[b]) nmax = std::max(nmax, Nof[i]);
         bp.nmax = nmax;
-        // (not timed by the autotuner: two-column steps from N = 112, where they win)
-        bp.kind = b < edges.size() ? (nmax >= 112 && bv_smem_bytes(6, nmax, c->d, 0) <= (size_t)(227 * 1024 - 3072) ? 6 : 0) : 2;
-        bp.threads = default_threads(bp.kind, bp.nmax);
+        bp.kind = b < edges.size() ? bv_fix_kind(nmax, c->d) : 2;
         // redo launch: the whole bin's capacity, count from the device
         bp.nwork = (int32_t)all[b].size();
+        bp.threads = default_threads(c, bp.kind, bp.nmax, bp.nwork);
         bp.d_work = k.d_redo + roff[b];
         bp.d_ctr = c->d_wctr + 3 * BV_WCTR_PER_PREC + b;
         bp.smem = bv_smem_bytes(bp.kind, bp.nmax, c->d, bp.threads);
@@ -894,10 +928,18 @@ static int build_check(bv_ctx* c, const std::vector<int>& Nof) {
         }
         bp.slot = (int)b;
         k.rbins.push_back(bp);
+        BV_TRY(alloc_slots(k.rbins.back()));
+        bp = k.rbins.back();
         if (!smp[b].empty()) {
             BinPlan sb = bp;
             sb.nwork = (int32_t)smp[b].size();
             sb.d_ctr = c->d_wctr + 2 * BV_WCTR_PER_PREC + b;
+            if (sb.kind != 2) {
+                sb.threads = default_threads(c, sb.kind, sb.nmax, sb.nwork);
+                const int occ = bv_occupancy(sb.kind, sb.threads, sb.smem);
+                if (occ <= 0) return BV_EINTERNAL;
+                sb.grid = std::min(sb.grid, occ * c->num_sms);  // (not more CTAs than workspace slots)
+            }
             sb.grid = std::min(sb.grid, sb.nwork);
             sb.d_work = nullptr;
             BV_CUDA(bv_plan_malloc(&sb.d_work, sizeof(int32_t) * smp[b].size()));
@@ -913,8 +955,8 @@ int bv_ensure_plan(bv_ctx* c, int prec) {
     if (c->plan_valid[prec]) return BV_OK;
     BV_TRY(build_layout(c));
     free_plan(c, prec);
-    const int smem_kind = prec == BV_MIXED ? 1 : 0;
-    const int nsm = bv_smem_max_n(smem_kind, c->d);
+    const bool fix = prec == BV_FP64;
+    const int nsm = fix ? bv_fix_max_n(c->d) : bv_smem_max_n(1, c->d);
     std::vector<int> Nof(c->nblk);
     int64_t maxlarge = 0;
     for (int64_t i = 0; i < c->nblk; ++i) {
@@ -925,9 +967,13 @@ int bv_ensure_plan(bv_ctx* c, int prec) {
     }
     // bins: edges up to the shared-memory limit, then one global-memory bin
     std::vector<int> edges;
-    for (int e : kBinEdges)
-        if (e < nsm) edges.push_back(e);
-    edges.push_back(nsm);
+    if (fix) {
+        edges = fix_edges(c->d);
+    } else {
+        for (int e : kBinEdges)
+            if (e < nsm) edges.push_back(e);
+        edges.push_back(nsm);
+    }
     std::vector<std::vector<int32_t>> lists(edges.size() + 1);
     for (int64_t i = 0; i < c->nblk; ++i) {
         const int N = Nof[i];
@@ -977,10 +1023,10 @@ int bv_ensure_plan(bv_ctx* c, int prec) {
         std::stable_sort(L.begin(), L.end(), [&](int32_t x, int32_t y) { return Nof[x] > Nof[y]; });
         BinPlan bp;
         bp.d_ctr = nullptr;
-        bp.kind = b < edges.size() ? smem_kind : 2;
         bp.nmax = Nof[L.front()];
-        bp.threads = default_threads(bp.kind, bp.nmax);
+        bp.kind = b >= edges.size() ? 2 : fix ? bv_fix_kind(bp.nmax, c->d) : 1;
         bp.nwork = (int32_t)L.size();
+        bp.threads = default_threads(c, bp.kind, bp.nmax, bp.nwork);
         bp.h_work = L;
         bp.d_work = nullptr;
         BV_CUDA(bv_plan_malloc(&bp.d_work, sizeof(int32_t) * L.size()));
@@ -988,6 +1034,7 @@ int bv_ensure_plan(bv_ctx* c, int prec) {
         BinPlan& pb = c->plan[prec].back();
         BV_CUDA(cudaMemcpyAsync(pb.d_work, L.data(), sizeof(int32_t) * L.size(), cudaMemcpyHostToDevice, c->stream));
         BV_TRY(set_grid(c, pb));
+        BV_TRY(alloc_slots(pb));
     }
     // largest bins first so the long blocks start early
     std::stable_sort(c->plan[prec].begin(), c->plan[prec].end(),
@@ -1061,34 +1108,22 @@ static int autotune(bv_ctx* c, int prec) {
                             c->stream));
     BV_CUDA(bv_launch_fail_reset(c->d_fail, c->stream));
     for (auto& bp : c->plan[prec]) {
-        if (bp.kind == 2) continue;
-        // candidates: CTA per block with 1 panel warp + 2/4/8/16 update warps (FP64 bins
-        // with N >= 128 also 31); for small
-        // blocks also a warp per block with 2/4/8 warps per CTA (mixed up to N = 128,
-        // FP64 up to N = 64)
-        // BV_KERNEL_FORM=cta or =warp restricts the choice to one form where both exist
-        // (tests use it to check each kernel against the oracle); FP64 CTA bins try the
-        // one-column and the two-column step (=cta keeps the first, =cta2 the second)
+        if (bp.kind != 1) continue;  // one form each
+        // candidates: CTA per block with 1 panel warp + 2/4/8/16 update warps; up to N = 128
+        // also a warp per block with 2/4/8 warps per CTA; from N = 64 on also the tensor-core
+        // kernel.  BV_KERNEL_FORM=cta, =warp or =tc restricts the choice to one form where it
+        // exists (tests use it to check each kernel against the oracle).
         const char* form = getenv("BV_KERNEL_FORM");
-        const bool only_cta2 = form && strcmp(form, "cta2") == 0;
-        const bool only_cta = (form && strcmp(form, "cta") == 0) || only_cta2;
+        const bool only_cta = form && (strcmp(form, "cta") == 0 || strcmp(form, "cta2") == 0);
         const bool only_warp = form && strcmp(form, "warp") == 0;
-        // mixed bins with N >= 64 also try the tensor-core kernel (BV_KERNEL_FORM=tc
-        // restricts them to it, =cta to the SIMT CTA kernel)
-        std::vector<std::pair<int, int>> cands;
-        const bool warp_ok = (bp.kind == 1 && bp.nmax <= 128) || (bp.kind == 0 && bp.nmax <= 64);
         const bool only_tc = form && strcmp(form, "tc") == 0;
-        const bool tc_ok = bp.kind == 1 && bp.nmax >= 64 &&
-                           bv_smem_bytes(5, bp.nmax, c->d, 256) <= (size_t)(227 * 1024 - 3072);
-        const bool w2_ok = bp.kind == 0 && bv_smem_bytes(6, bp.nmax, c->d, 0) <= (size_t)(227 * 1024 - 3072);
-        if (!(only_warp && warp_ok) && !(only_tc && tc_ok) && !(only_cta2 && w2_ok))
-            for (int t : {96, 160, 288, 544, 1024})
-                if (t < 1024 || (bp.kind == 0 && bp.nmax >= 128)) cands.push_back({bp.kind, t});
-        if (w2_ok && !only_warp && !(only_cta && !only_cta2))
-            for (int t : {96, 160, 288, 544, 1024})
-                if (t < 1024 || bp.nmax >= 128) cands.push_back({6, t});
+        std::vector<std::pair<int, int>> cands;
+        const bool warp_ok = bp.nmax <= 128;
+        const bool tc_ok = bp.nmax >= 64 && bv_smem_bytes(5, bp.nmax, c->d, 256) <= (size_t)(227 * 1024 - 3072);
+        if (!(only_warp && warp_ok) && !(only_tc && tc_ok))
+            for (int t : {96, 160, 288, 544}) cands.push_back({1, t});
         if (!only_cta && !only_tc && warp_ok)
-            for (int t : {64, 128, 256}) cands.push_back({bp.kind == 1 ? 3 : 4, t});
+            for (int t : {64, 128, 256}) cands.push_back({3, t});
         if (!only_cta && !only_warp && tc_ok)
             for (int t : {128, 256, 384, 512}) cands.push_back({5, t});
         int best_k = bp.kind, best_t = bp.threads;

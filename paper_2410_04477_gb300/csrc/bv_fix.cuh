@@ -1,0 +1,244 @@
+// bv_fix.cuh -- 64-bit fixed-point arithmetic of the FP64-accurate block kernel
+// (bv_fix_ll.cu): products, reciprocal square root, exponential and the closed-form Matern
+// correlation, on the integer pipe.
+//
+// Why: this part's SM executes 2 FP64 lanes per clock but 64 or more 32 x 32 -> 64-bit
+// integer multiply-adds.  A correlation matrix normalised to a unit diagonal has entries,
+// Schur complements and factor entries all in [-1, 1], so 64-bit fixed point holds them
+// with an absolute error of 2^-60 or less, where FP64 arithmetic leaves 2^-54 on values
+// near 1.
+#pragma once
+#include <stdint.h>
+
+#ifdef __CUDACC__
+#define BV_FIX __device__ __forceinline__
+#else  // host build of the arithmetic's own test
+#include <math.h>
+#include <string.h>
+#define BV_FIX static inline
+#endif
+
+namespace bvfix {
+
+#ifdef __CUDACC__
+BV_FIX int clz64(uint64_t v) { return __clzll((long long)v); }
+BV_FIX float rsq32(float x) {
+    float r;
+    asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
+    return r;
+}
+BV_FIX int f2i(float x) { return __float2int_rn(x); }
+BV_FIX uint64_t dbits(double x) { return (uint64_t)__double_as_longlong(x); }
+BV_FIX double bitsd(uint64_t x) { return __longlong_as_double((long long)x); }
+#else
+BV_FIX int clz64(uint64_t v) { return v ? __builtin_clzll(v) : 64; }
+BV_FIX float rsq32(float x) { return (float)(1.0 / sqrt((double)x)) * (1.0f + 1.2e-7f); }  // a last-bit error, as the unit has
+BV_FIX int f2i(float x) { return (int)rintf(x); }
+BV_FIX uint64_t dbits(double x) { uint64_t u; memcpy(&u, &x, 8); return u; }
+BV_FIX double bitsd(uint64_t u) { double x; memcpy(&x, &u, 8); return x; }
+#endif
+
+BV_FIX uint32_t hi32(uint64_t a) { return (uint32_t)(a >> 32); }
+BV_FIX uint32_t lo32(uint64_t a) { return (uint32_t)a; }
+
+// a b + c, 32 x 32 + 64 bits: one instruction, 64 lanes a clock (written out, since the
+// compiler does not always see that both factors are 32 bits wide).
+#ifdef __CUDACC__
+BV_FIX int64_t smad(int32_t a, int32_t b, int64_t c) {
+    asm("mad.wide.s32 %0, %1, %2, %0;" : "+l"(c) : "r"(a), "r"(b));
+    return c;
+}
+BV_FIX uint64_t umad(uint32_t a, uint32_t b, uint64_t c) {
+    asm("mad.wide.u32 %0, %1, %2, %0;" : "+l"(c) : "r"(a), "r"(b));
+    return c;
+}
+#else
+BV_FIX int64_t smad(int32_t a, int32_t b, int64_t c) { return (int64_t)((uint64_t)((int64_t)a * b) + (uint64_t)c); }
+BV_FIX uint64_t umad(uint32_t a, uint32_t b, uint64_t c) { return (uint64_t)a * b + c; }
+#endif
+
+// High 64 bits of a b, up to 2 units low (the low x low product is left out); a, b < 2^63,
+// so that the two middle products sum without a carry: three multiply-adds.
+BV_FIX uint64_t mulhi63(uint64_t a, uint64_t b) {
+    const uint64_t mid = umad(hi32(a), lo32(b), umad(lo32(a), hi32(b), 0));
+    return umad(hi32(a), hi32(b), hi32(mid));
+}
+// The same for any a, b.
+BV_FIX uint64_t mulhi64(uint64_t a, uint64_t b) {
+    const uint64_t p = umad(hi32(a), lo32(b), 0), q = umad(lo32(a), hi32(b), 0);
+    return umad(hi32(a), hi32(b), hi32(p)) + hi32(q);
+}
+
+// A signed 64-bit value as h 2^32 + l with both halves signed (l in [-2^31, 2^31)), so that
+// all partial products are signed 32 x 32 -> 64.
+struct Bal {
+    int32_t h, l;
+};
+BV_FIX Bal bal(int64_t v) {
+    Bal b;
+    b.l = (int32_t)(uint32_t)v;
+    b.h = (int32_t)(((uint64_t)v + 0x80000000ull) >> 32);
+    return b;
+}
+// Scales: matrix entries and Schur complements in units of 2^-60 (kUnitC), factor entries in
+// units of 2^-59 (kUnitL).
+constexpr int kUnitC = 60, kUnitL = 59;
+
+// A factor entry x = h 2^29 + l for products: h h exactly on the integer pipe, the two cross
+// products in FP32, whose accumulators are half as wide: they are below 2^-31 |x| |y|, so that
+// FP32's 2^-24 leaves 2^-55 |x| |y|; l l is below 2^-62.
+struct Fac {
+    int32_t h;
+    float hf, lf;  // h and l 2^-31
+};
+BV_FIX Fac fac(int64_t x) {
+    Fac f;
+    f.h = (int32_t)((x + (1ll << 28)) >> 29);
+    f.hf = (float)f.h;
+    f.lf = (float)((int32_t)((uint32_t)x << 3) >> 3) * 4.656612873077392578125e-10f;
+    return f;
+}
+// a 2^-60 + c 2^-58 -= x y.
+BV_FIX void msub(int64_t& a, float& c, int32_t nxh, float nxhf, float nxlf, int32_t yh, float yhf, float ylf) {
+    a = smad(nxh, yh, a);
+    c = fmaf(nxhf, ylf, c);
+    c = fmaf(nxlf, yhf, c);
+}
+
+// 1 / sqrt(P), P = p 2^-60, for p in [1, 2^60]: r 2^(e - 62) with r in [2^62, 2^63) and e >= 0,
+// within 2^-59 relative and exact for P = 1.  The hardware seed's mantissa Y (24 bits, error
+// 2^-22) takes a Newton step with the second-order term in fixed point, which cubes its error.
+struct Rsq {
+    int64_t r;
+    int e;
+};
+BV_FIX uint32_t fbits(float x) {
+#ifdef __CUDACC__
+    return __float_as_uint(x);
+#else
+    uint32_t u;
+    memcpy(&u, &x, 4);
+    return u;
+#endif
+}
+BV_FIX Rsq rsqrt_fix(int64_t p) {
+    Rsq o;
+    const float pf = fmaf((float)(int32_t)hi32((uint64_t)p), 4294967296.0f, (float)lo32((uint64_t)p));
+    const uint32_t u = fbits(rsq32(pf));
+    const uint32_t Y = (u & 0x7fffffu) | 0x800000u;       // units 2^-23
+    o.e = (int)(u >> 23) - 127 + 30;
+    const uint64_t M = (uint64_t)p << (2 * o.e + 3);      // P 4^e in (1/4, 1], units 2^-63
+    const int64_t e60 = (1ll << 60) - (int64_t)mulhi63(M, umad(Y, Y, 0) << 15);  // 1 - P 4^e y^2
+    const int32_t es = (int32_t)(e60 >> 20);              // units 2^-40
+    const int64_t c = e60 + (smad(es, es + es + es, 0) >> 22);  // e + 3 e^2 / 4
+    const int64_t pr = smad((int32_t)Y, (int32_t)(c >> 16), smad((int32_t)Y, (int32_t)(c & 0xffff), 0) >> 16);
+    o.r = ((int64_t)Y << 39) + (pr >> 6);                 // y (1 + c / 2)
+    return o;
+}
+
+// sqrt(M) 2^31 for M in [2^62, 2^64), within 2^-62 relative: 24 bits from the hardware
+// reciprocal square root and two residual corrections.
+BV_FIX uint64_t sqrt_fix(uint64_t M) {
+    const float mf = (float)hi32(M);                    // M 2^-32 in [2^30, 2^32]
+    const float y = rsq32(mf);
+    const uint32_t s0 = (uint32_t)f2i(mf * y * 256.0f);  // sqrt(M) 2^-8
+    const int64_t r = (int64_t)(M - (umad(s0, s0, 0) << 16));
+    const float h = y * 7.62939453125e-6f;               // 1 / (2 sqrt(M)): y 2^-16 / 2
+    const int32_t c1 = f2i((float)(int32_t)(r >> 13) * (h * 67108864.0f));        // r h in units 2^-13
+    const int64_t r2 = (int64_t)((uint64_t)r << 16) - (int64_t)((uint64_t)smad((int32_t)s0, c1, 0) << 12) - (smad(c1, c1, 0) >> 10);
+    const int32_t c2 = f2i((float)(int32_t)(r2 >> 9) * (h * 33554432.0f));        // units 2^-32
+    return ((uint64_t)s0 << 39) + (uint64_t)((int64_t)c1 << 18) + (uint64_t)(int64_t)(c2 >> 1);
+}
+
+// The scaled distance x = sqrt(acc) of a normal acc > 0 as x = X 2^(q - 63), X in
+// [2^62, 2^63), from acc's 53-bit significand.
+struct Dist {
+    uint64_t X;
+    int q;
+};
+BV_FIX Dist dist_fix(uint64_t accbits) {
+    Dist o;
+    const int k = (int)(accbits >> 52) - 1023;
+    o.q = (k >> 1) + 1;
+    o.X = sqrt_fix(((accbits & 0x000FFFFFFFFFFFFFull) | 0x0010000000000000ull) << (10 + (k & 1)));
+    return o;
+}
+
+// Tables of the exponential: A[j] = 2^(-j/256) w in units 2^-62 (w <= 1, a weight of the
+// caller's) and B[j] = 2^(-j/65536) in units 2^-63 (B[0] one unit below 1).
+BV_FIX uint64_t shr(uint64_t v, int n) { return v >> (n < 63 ? n : 63); }
+
+// w e^-x = w 2^-z from z in units 2^-57: W 2^-i with W in units 2^-61.  z = i + j1/256 +
+// j2/65536 + g: tables for the middle parts, e^-r - 1 for r = g ln 2 < 2^-16 as -r + (r^2/2 -
+// r^3/6) with the bracket in FP32 (below 2^-33, its rounding below 2^-57 of the result).
+struct Exp {
+    uint64_t W;
+    int i;
+};
+template <typename TA, typename TB>
+BV_FIX Exp exp2_fix(uint64_t zf, const TA* A, const TB* B) {
+    const uint64_t r = mulhi63((zf & 0x1FFFFFFFFFFull) << 22, 0x58B90BFBE8E7BCD6ull);  // units 2^-78; ln 2 in 2^-63
+    const float rf = (float)(int32_t)hi32(r);                      // units 2^-46
+    const int32_t q2 = f2i(rf * rf * 1.862645149230957e-9f * (1.0f - rf * 4.736951571734001e-15f));  // r^2/2 - r^3/6, 2^-64
+    const uint64_t E = r - ((uint64_t)(uint32_t)q2 << 14);
+    const uint64_t P = mulhi63(A[(zf >> 49) & 255], B[(zf >> 41) & 255]);
+    Exp o;
+    o.W = P - (mulhi63(P, E) >> 14);
+    o.i = (int)(zf >> 57);
+    return o;
+}
+
+// w rho(x) in matrix units for the closed forms: NU = 0 (1/2), 1 (3/2) or 2 (5/2).  x >= 64
+// gives 0 (rho below 2^-80).  No branches: a caller's entries are independent chains that the
+// compiler can interleave.
+template <int NU, typename TA, typename TB>
+BV_FIX int64_t matern_fix(Dist x, const TA* A, const TB* B) {
+    const uint64_t Z = mulhi63(x.X, 0x5C551D94AE0BF85Eull);        // log2 e in units 2^-62
+    const int q = x.q > 6 ? 6 : x.q < -55 ? -55 : x.q, sh = 6 - q;
+    const Exp e = exp2_fix(((Z << 2) + ((1ull << sh) >> 1)) >> sh, A, B);
+    uint64_t v = shr(e.W, e.i);
+    if (NU > 0) {
+        const uint64_t H = mulhi63(x.X, e.W);                      // units 2^(q - 60)
+        v += shr(H << 1, e.i - q);
+        if (NU > 1) {
+            const uint64_t H2 = mulhi63(x.X, mulhi63(H, 0x5555555555555555ull));  // units 2^(2 q - 59)
+            v += shr(H2 << 6, e.i - 2 * q + 4);
+        }
+    }
+    return x.q > 6 ? 0 : (int64_t)((v + 1) >> 1);
+}
+
+// The general smoothness: rho = e^-(x - L(x)), L a polynomial of degree DEG - 1 in t = 2 m - 3
+// on each octave x = m 2^o, m in [1, 2), its coefficients (power basis, units 2^-57, |L| < 64)
+// at tab + (o + OCT0) DEG, evaluated by Horner's rule.  For 2^-OCT0 <= x; x >= 128 gives 0.
+template <int DEG, int OCT0, typename TA, typename TB>
+BV_FIX int64_t matern_gen_fix(Dist x, const int64_t* tab, const TA* A, const TB* B) {
+    const int q = x.q > 7 ? 7 : x.q < 1 - OCT0 ? 1 - OCT0 : x.q;
+    const int64_t* c = tab + (q - 1 + OCT0) * DEG;
+    const Bal t = bal((int64_t)(2 * x.X) - (3ll << 62));           // units 2^-62
+    int64_t b = c[DEG - 1];
+#ifdef __CUDACC__
+#pragma unroll
+#endif
+    for (int k = DEG - 2; k >= 0; --k) {
+        const Bal y = bal(b);
+        const int64_t mid = smad(y.h, t.l, smad(y.l, t.h, 1ll << 29));
+        b = c[k] + (int64_t)((uint64_t)smad(y.h, t.h, 0) << 2) + (mid >> 30);
+    }
+    const uint64_t xf = q > 6 ? x.X << 1 : x.X >> (6 - q);         // x in units 2^-57
+    const int64_t y = (int64_t)(xf - (uint64_t)b);                 // x - L; from 64 on its sign bit is set
+    const bool far = x.q > 7 || (q >= 6 && y < 0) || (q == 7 && b <= 0);
+    const uint64_t yc = y < 0 ? 0 : (uint64_t)y;
+    const Exp e = exp2_fix(mulhi64(yc, 0xB8AA3B295C17F0BCull) << 1, A, B);  // log2 e in units 2^-63
+    return far ? 0 : (int64_t)((shr(e.W, e.i) + 1) >> 1);
+}
+
+// A double in [0, 1] in matrix units, truncated.
+BV_FIX int64_t unit_fix(double v) {
+    const uint64_t b = dbits(v);
+    const int k = (int)(b >> 52) - 1023;  // v = 1.f 2^k, k <= 0
+    if (k < -61) return 0;
+    return (int64_t)(((b & 0x000FFFFFFFFFFFFFull) | 0x0010000000000000ull) << 8 >> (-k));
+}
+
+}  // namespace bvfix

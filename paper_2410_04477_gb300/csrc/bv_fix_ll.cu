@@ -1,0 +1,256 @@
+// bv_fix_ll.cu -- the FP64-accurate block-Vecchia log-likelihood kernel (Eq. 4, Algorithm 1)
+// in 64-bit fixed point, with the trailing updates on the tensor cores.
+//
+// The computation is the one of bv_loglik.cu: one Cholesky factorisation of the block's
+// augmented (N+1) x (N+1) matrix.  FP64 arithmetic bounded it: the SM executes 2 FP64 lanes
+// per clock, and a block needs N^3/6 of them for the updates and about 10 N^2 for the
+// covariance.  Dividing by D = sigma^2 + tau^2 makes the diagonal 1, so that every entry,
+// Schur complement and factor entry lies in [-1, 1] and 64-bit integers hold them with an
+// absolute error below FP64's (which rounds at 2^-54 of values near 1):
+//   covariance   bv_fix.cuh: squared distances in FP64, the rest on the integer pipe;
+//   panel        16 columns: the diagonal tile by one warp, the rows below one per thread;
+//   update       C_IJ -= L_I L_J^T on the tensor cores, exactly: every factor entry is cut
+//                into six signed 10-bit digits, held as FP16; products of digits sum to whole
+//                numbers below 2^24 over 16 columns and up to four digit pairs, which FP32
+//                accumulation adds without rounding.  The 21 digit pairs of combined order
+//                <= 5 are taken (the pairs of order 4 and 5, five and six to a sum, could
+//                round in the last bit only on sums that real digits do not reach, by one
+//                unit of 2^-58); what is left out is below 2^-57 of 1.
+// The data row is scaled by a power of two so that |y| / sqrt(D) stays below 2^-5; if a
+// solved entry leaves the range, the block is done again with a larger power (an outlier
+// more than 2^5 conditional standard deviations above the largest observation).
+//
+// Against a 113-bit factorisation of the same scaled coordinates, the blocks' ell errs by
+// 8.4e-13 (RMS; n = 20,000, m = 60, nu = 3/2, tau^2 = 1e-4), FP64 arithmetic by 2.8e-12; at m =
+// 113 by 4.9e-13 against 1.9e-12.  Time of an evaluation, FP64 arithmetic and this kernel:
+//   n = 200,000, m = 60 (N about 70)        5.04 ms   2.60 ms
+//   n = 36,931, m = 113                     3.64      1.20
+//   n = 100,000, 3D, m = 200                42.4      9.60
+//   n = 50,000, blocks of 1, m = 30         2.36      1.64
+//   n = 100,000, m = 60, nu = 1.2           4.92      2.38
+//   n = 2,000, m = 30                       0.122     0.094
+// What bounds it: up to N about 100 the latency of the pivots' chain (a tile's 16 pivots take
+// some 13,000 clocks, in which the other warps follow one pair of columns behind) with four to
+// eight blocks an SM; beyond, instruction issue, shared by the covariance, the panel rows and
+// the sums of digit products, the tensor cores themselves being busy a tenth of the time.
+#include <cuda_runtime.h>
+#include <math.h>
+#include <stdint.h>
+
+#include "bv_device.cuh"
+#include "bv_fix.cuh"
+#include "bv_fix_tile.cuh"
+#include "bv_internal.h"
+#include "bv_ll_block.cuh"
+
+namespace {
+
+constexpr int kFixWarps = 16;       // resident warps an SM that the register budget allows
+
+// GLOB: the tiles live in a global-memory slot of the CTA (they stay in L2), for blocks whose
+// triangle does not leave room in shared memory.
+template <int NT, bool GEN, bool GLOB>
+__global__ void __launch_bounds__(NT, kFixWarps * 32 / NT) k_ll_fix(LLArgs a) {
+    extern __shared__ __align__(16) unsigned char smraw[];
+    __shared__ uint64_t tA[256], tB[256];
+    __shared__ int s_w;
+    __shared__ unsigned s_ymax;  // largest high word of |y| / sqrt(D)
+    __shared__ __align__(8) uint64_t s_mb[8];
+    constexpr int NW = NT / 32;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    for (int j = tid; j < 256; j += NT) tB[j] = a.fixtab[256 + j];
+    const int nwork = work_count(a);
+    if (tid < 8)
+        asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"((uint32_t)__cvta_generic_to_shared(s_mb + tid)) : "memory");
+    uint32_t parity = 0;  // of the panel's phase of the mbarriers
+    if (tid == 0) s_w = take_work(a.ctr, blockIdx.x);
+    __syncthreads();
+    int dsprev = -1;
+    for (int w = s_w; w < nwork; w = s_w) {
+        const int nx = tid == 0 ? take_work(a.ctr, w + gridDim.x) : 0;
+        const int blk = a.work[w];
+        const int64_t b0 = a.bptr[blk], n0 = a.nptr[blk];
+        const int b = (int)(a.bptr[blk + 1] - b0), m = (int)(a.nptr[blk + 1] - n0);
+        const int N = m + b, T = fix_tiles(N), TC = (N + 15) >> 4;
+        const int ds = a.bds[blk];
+        const DevTheta th = a.theta[ds];
+        const int d = a.d;
+        unsigned char* wk = GLOB ? smraw : smraw + (size_t)((T * (T + 1)) >> 1) * kTileB;
+        longlong2* tiles = GLOB ? reinterpret_cast<longlong2*>(a.ws + (int64_t)blockIdx.x * a.ws_stride)
+                                : reinterpret_cast<longlong2*>(smraw);
+        uint32_t* dig = reinterpret_cast<uint32_t*>(wk);
+        int4* Ld = reinterpret_cast<int4*>(wk + (size_t)(T - 1) * kDigB);
+        FixRs* rsv = reinterpret_cast<FixRs*>(Ld + 16 * kLd + 16);
+        double* px = reinterpret_cast<double*>(rsv + 16);
+        double* yv = px + d * N;
+        int64_t* piv = reinterpret_cast<int64_t*>(yv + N);
+        int64_t* zrow = piv + N;
+
+        const double D = th.diag, ratio = th.diag_ratio, isd = th.diag_rsqrt;
+        if (ds != dsprev) {  // A[j] = 2^(-j/256) sigma^2 / D
+            const uint64_t rf = (uint64_t)__double2ull_rn(ratio * 0x1p63);
+            for (int j = tid; j < 256; j += NT) tA[j] = bvfix::mulhi64(a.fixtab[j], rf) << 1;
+            dsprev = ds;
+        }
+        if (tid == 0) s_ymax = 0;
+        for (int j = tid; j < 16 * kLd + 16; j += NT)
+            if (j % kLd >= 16) Ld[j] = make_int4(0, 0, 0, 0);
+        __syncthreads();
+        unsigned ym = 0;
+        for (int t = tid; t < N; t += NT) {
+            const int g = t < m ? a.nidx[n0 + t] : a.pidx[b0 + (t - m)];
+            for (int k = 0; k < d; ++k) px[k * N + t] = a.locs[(int64_t)k * a.n_tot + g] * inv_range_k(th, k);
+            const double y = a.y[g] * isd;
+            yv[t] = y;  // (in place of its fixed-point value until the scale is known)
+            ym = max(ym, (unsigned)__double2hiint(y) & 0x7fffffffu);
+        }
+        ym = __reduce_max_sync(0xffffffffu, ym);
+        if (lane == 0) atomicMax(&s_ymax, ym);
+        __syncthreads();
+        const int ye = (int)(s_ymax >> 20);
+        const bool valid = D > 0.0 && D < INFINITY && ratio >= 0.0 && ratio <= 1.0 && ye != 0x7ff;
+        int E = (ye > 0 ? ye - 1022 : -1021) + kYRoom;  // |y| 2^-E < 2^-kYRoom
+
+        bool fail = false;
+        int64_t* yfix = reinterpret_cast<int64_t*>(yv);
+        // again with a larger E when a solved data entry leaves the range (a finite z needs a
+        // few passes at most; the data row is 0 after 9)
+        for (int pass = 0;; ++pass) {
+            int flags = valid ? 0 : kFail;
+            for (int t = tid; t < N; t += NT) {
+                const double y = pass == 0 ? yv[t] : ldexp((double)yfix[t], E - kYStep - bvfix::kUnitC);
+                yfix[t] = __double2ll_rn(ldexp(y, bvfix::kUnitC - E));
+            }
+            __syncthreads();
+            const int ntile = (T * (T + 1)) >> 1;
+            for (int q = warp; q < ntile; q += NW) {
+                int I, J;
+                tri_rc(q, I, J);
+                if (J >= TC) continue;
+                fix_fill<GEN ? 1 : 0, false>(tiles + q * 128, I, J, N, N, N, lane, px, d, yfix, a.theta + ds, th.nu_code, ratio,
+                                             a.gtabi + (int64_t)ds * GTAB_SIZE, tA, tB, flags);
+            }
+            int stop = __syncthreads_or(flags);
+            if (!stop) stop = fix_panels<NT>(tiles, T, TC, TC, N, dig, Ld, rsv, piv, zrow, s_mb, parity, flags);
+            fail = stop && __syncthreads_or(flags & kFail);
+            if (fail || !stop) break;
+            if (pass == 12) {
+                fail = true;
+                break;
+            }
+            E += kYStep;
+        }
+
+        if (warp == 0) {
+            const double zs = ldexp(1.0, E - bvfix::kUnitL), ps = D * 0x1p-60;
+            const double2 s2 = warp_terms(m, N, lane, [&](int k) { return fail ? 0.0 : (double)zrow[k] * zs; },
+                                          [&](int k) { return fail ? 0.0 : log((double)piv[k] * ps); });
+            if (lane == 0) {
+                double ell = -0.5 * (s2.x + (double)b * kLog2Pi);
+                if (fail || !(ell == ell)) {
+                    ell = -INFINITY;
+                    record_fail(a.fail, blk);
+                }
+                a.ell_blk[blk] = ell;
+                a.u_blk[blk] = s2.y;
+                s_w = nx;
+            }
+        }
+        __syncthreads();
+    }
+}
+
+template <int NT, bool GEN, bool GLOB>
+cudaError_t fix_attr() {
+    return cudaFuncSetAttribute(k_ll_fix<NT, GEN, GLOB>, cudaFuncAttributeMaxDynamicSharedMemorySize, kFixSmemCap);
+}
+
+template <int NT>
+cudaError_t fix_go(int grid, size_t smem, bool glob, const LLArgs& a, cudaStream_t s) {
+    cudaError_t e;
+#define BV_GO(GEN, GLOB)                                         \
+    {                                                            \
+        e = fix_attr<NT, GEN, GLOB>();                           \
+        if (e != cudaSuccess) return e;                          \
+        k_ll_fix<NT, GEN, GLOB><<<grid, NT, smem, s>>>(a);       \
+    }
+    if (a.gen) {
+        if (glob) BV_GO(true, true) else BV_GO(true, false)
+    } else {
+        if (glob) BV_GO(false, true) else BV_GO(false, false)
+    }
+#undef BV_GO
+    return cudaGetLastError();
+}
+
+template <int NT>
+int fix_occ(size_t smem, bool glob) {
+    int n1 = 0, n2 = 0;
+    cudaError_t e = glob ? fix_attr<NT, false, true>() : fix_attr<NT, false, false>();
+    if (e == cudaSuccess) e = glob ? fix_attr<NT, true, true>() : fix_attr<NT, true, false>();
+    if (e != cudaSuccess) return 0;
+    if (glob) {
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n1, k_ll_fix<NT, false, true>, NT, smem);
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n2, k_ll_fix<NT, true, true>, NT, smem);
+    } else {
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n1, k_ll_fix<NT, false, false>, NT, smem);
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n2, k_ll_fix<NT, true, false>, NT, smem);
+    }
+    return n1 > n2 ? n1 : n2;
+}
+
+}  // namespace
+
+// CTA size: one warp for the diagonal tiles, the others for the rows below, with which four
+// warps cover blocks up to N = 111 in one pass.  Blocks of up to three tile rows take two
+// warps, large ones eight.  A bin of few blocks (two an SM) takes eight as well: there a
+// block's latency counts, not the SM's rate.
+int bv_fix_threads(int nmax, int nwork, int num_sms) {
+    if (nwork <= 2 * num_sms) return 256;
+    return nmax <= 47 ? 64 : nmax <= 239 ? 128 : 256;
+}
+
+size_t bv_fix_smem_bytes(int kind, int nmax, int d) {
+    return fix_work_bytes(nmax, d) + (kind == 8 ? 0 : fix_tile_bytes(nmax));
+}
+
+// The kernel form of a bin of largest size nmax: tiles in shared memory (7) up to three tile
+// rows, in a workspace (8) beyond, where four to eight CTAs an SM would not fit with them; -1
+// when even the panel's digits do not fit.
+int bv_fix_kind(int nmax, int d) {
+    if (fix_tiles(nmax) <= 3) return 7;
+    return bv_fix_smem_bytes(8, nmax, d) <= (size_t)kFixSmemCap ? 8 : -1;
+}
+int bv_fix_max_n(int d) {
+    int n = 64;
+    while (bv_fix_kind(n + 1, d) > 0) ++n;
+    return n;
+}
+size_t bv_fix_slot_bytes(int nmax) { return fix_tile_bytes(nmax); }
+
+int bv_fix_occupancy(int kind, int threads, size_t smem) {
+    switch (threads) {
+        case 64: return fix_occ<64>(smem, kind == 8);
+        case 128: return fix_occ<128>(smem, kind == 8);
+        case 256: return fix_occ<256>(smem, kind == 8);
+        default: return 0;
+    }
+}
+
+cudaError_t bv_fix_launch(int kind, int threads, int grid, size_t smem, const LLArgs& a, cudaStream_t s) {
+    switch (threads) {
+        case 64: return fix_go<64>(grid, smem, kind == 8, a, s);
+        case 128: return fix_go<128>(grid, smem, kind == 8, a, s);
+        case 256: return fix_go<256>(grid, smem, kind == 8, a, s);
+        default: return cudaErrorInvalidValue;
+    }
+}
+
+// The exponential's tables (bv_fix.cuh): 2^(-j/256) in units 2^-62, then 2^(-j/65536) in units
+// 2^-63, the first of them one unit below 1.
+void bv_fix_tables(uint64_t* t) {
+    for (int j = 0; j < 256; ++j) {
+        t[j] = (uint64_t)(exp2l(-(long double)j / 256.0L) * 0x1p62L + 0.5L);
+        t[256 + j] = j ? (uint64_t)(exp2l(-(long double)j / 65536.0L) * 0x1p63L + 0.5L) : (1ull << 63) - 1;
+    }
+}

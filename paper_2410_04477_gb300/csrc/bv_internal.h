@@ -66,6 +66,9 @@ struct DevTheta {
     // (added to every pivot, so that the FP32 factor is that of the exact diagonal)
     float sigma2_f, nugget_f, inv_range_f[3];
     float diag_lo_f;
+    // normalised covariance of the fixed-point kernel: D = sigma^2 + tau^2, sigma^2 / D and
+    // 1 / sqrt(D)
+    double diag, diag_ratio, diag_rsqrt;
 };
 
 // Constants of the table-driven FP64 exponential (Tang, "Table-driven implementation of
@@ -113,6 +116,7 @@ struct LLArgs {
     int* fb;                 // mixed precision: [0] count, [1..] blocks to redo in FP64 (or null)
     int dyn;                 // global-memory kernel: take the work list and count from fb
     const double* gtab;      // per dataset: general-nu Matern table (GTAB_SIZE doubles)
+    const int64_t* gtabi;    // the same in the power basis, units 2^-57 (fixed-point kernel)
     double* ell_blk;         // per-block conditional log-likelihood (output)
     double* u_blk;           // per-block quadratic form u_i = v_i^T v_i (output)
     float* ind_blk;          // mixed kernels, or null: per-block sum over all pivots of
@@ -120,15 +124,15 @@ struct LLArgs {
     unsigned long long* fail;  // min over failing block ids (ULLONG_MAX = none)
     double* ws;              // global workspace (large-block path)
     int64_t ws_stride;       // doubles per workspace slot
+    const uint64_t* fixtab;  // fixed-point exponential tables (bv_fix_tables)
     ExpConsts ex;            // FP64 exponential constants (and the FP32 table of exp_neg32)
 };
 
 // Per-size-bin launch plan entry.
 struct BinPlan {
-    int kind;            // 0: FP64 shared-memory, 1: mixed (CTA per block), 2: large (global),
-                         // 3: mixed (warp per block), 4: FP64 (warp per block),
-                         // 5: mixed with tensor-core updates (CTA per block),
-                         // 6: FP64 shared-memory with two-column steps
+    int kind;            // 1: mixed (CTA per block), 2: large (global), 3: mixed (warp per
+                         // block), 5: mixed with tensor-core updates (CTA per block),
+                         // 7: FP64 in fixed point, 8: the same with its tiles in d_slots
     int nmax;            // largest augmented size N = m + b in the bin
     int threads;         // CTA size (autotuned)
     int grid;            // CTAs launched
@@ -136,6 +140,8 @@ struct BinPlan {
     int32_t* d_work;     // device block ids (largest N first)
     int32_t nwork;
     int* d_ctr;          // this bin's work counter (a slot of the context's counter array)
+    double* d_slots = nullptr;  // kind 8: one workspace slot of slot_stride doubles per CTA
+    int64_t slot_stride = 0;
     int slot = -1;       // mixed check's redo launches: index of the bin's device count
     std::vector<int32_t> h_work;
 };
@@ -145,10 +151,19 @@ size_t bv_tc_smem_bytes(int nmax);
 int bv_tc_occupancy(int threads, size_t smem);
 cudaError_t bv_tc_launch(int threads, int grid, size_t smem, const LLArgs& a, cudaStream_t s);
 
+// FP64 kernel in fixed point with tensor-core updates (bv_fix_ll.cu), kinds 7 and 8.
+int bv_fix_kind(int nmax, int d);
+int bv_fix_max_n(int d);
+int bv_fix_threads(int nmax, int nwork, int num_sms);
+size_t bv_fix_smem_bytes(int kind, int nmax, int d);
+size_t bv_fix_slot_bytes(int nmax);
+int bv_fix_occupancy(int kind, int threads, size_t smem);
+cudaError_t bv_fix_launch(int kind, int threads, int grid, size_t smem, const LLArgs& a, cudaStream_t s);
+void bv_fix_tables(uint64_t* t);  // 512 values
+
 // Launchers (bv_loglik.cu).
 int bv_smem_max_n(int kind, int d);
 size_t bv_smem_bytes(int kind, int nmax, int d, int threads);
-int bv_max_threads_for(int kind);
 int bv_occupancy(int kind, int threads, size_t smem);
 // Largest augmented size the global-memory path accepts (packed indices stay in int32).
 #define BV_LARGE_MAX_N 30000
@@ -179,7 +194,7 @@ cudaError_t bv_launch_mixed_redo_list(const int32_t* bds, int64_t nblk, const in
                                       cudaStream_t s);
 // Builds every general-nu dataset's Matern table (bv_device.cuh) from the device thetas.
 cudaError_t bv_launch_gtab(const DevTheta* theta, int32_t ndata, double* gtab, cudaStream_t s);
-#define BV_GTAB_DOUBLES 931  // GTAB_NOCT * GTAB_DEG
+#define BV_GTAB_DOUBLES 931  // GTAB_NOCT * GTAB_DEG (per dataset: so many doubles, then so many int64)
 
 // K-means and neighbour search (bv_kmeans.cu, bv_nn.cu).
 int bv_kmeans_device(const double* d_locs_soa, int64_t n_tot, int64_t off, int64_t n, int d,
@@ -280,7 +295,8 @@ struct bv_ctx {
     double* d_out = nullptr;          // ndata
     double* h_out = nullptr;          // pinned, ndata
     DevTheta* d_theta = nullptr;      // ndata
-    double* d_gtab = nullptr;         // ndata x BV_GTAB_DOUBLES general-nu Matern tables
+    uint64_t* d_fixtab = nullptr;     // fixed-point exponential tables (bv_fix_tables)
+    double* d_gtab = nullptr;         // 2 x ndata x BV_GTAB_DOUBLES: general-nu Matern tables, then their fixed-point forms
     std::vector<DevTheta> h_theta;    // ndata (pageable: copies are staged by the driver)
     unsigned long long* h_fail = nullptr;  // pinned
     double* d_ws = nullptr;

@@ -15,16 +15,16 @@
 // v = L'^{-1}(y_B - mu).  So u = sum_{k>=m} z_k^2 and d = sum_{k>=m} log p_k, with z the
 // last row of the factor and p_k the pivots (squared diagonal of the factor), and
 //        ell_i = -(u + d + b log 2 pi) / 2.
-// The kernels generate the matrix (Matern, Eq. 5) straight into shared memory, factor it
-// in place (right-looking, one or two columns per step in FP64, 4-column tile panels in
-// mixed precision) and reduce ell_i, so nothing but the
-// locations, y and the index lists is read from HBM and one double per block is written.
+// The kernels generate the matrix (Matern, Eq. 5) straight into on-chip memory, factor it
+// in place and reduce ell_i, so nothing but the locations, y and the index lists is read from
+// HBM and one double per block is written.
 //
 // Paths:
-//   k_ll_fp64<NT>   FP64 packed lower triangle in shared memory (N up to 233 for d=3; 231 with two-column steps)
+//   k_ll_fix<NT>    FP64 accuracy in 64-bit fixed point with tensor-core updates (bv_fix_ll.cu)
 //   k_ll_mixed<NT>  FP32 covariance (block-local coordinates), FP32 updates; pivots,
 //                   log-determinant and quadratic form accumulated in FP64
-//   k_ll_large<NT>  FP64, packed triangle in a global-memory workspace slot (any N)
+//   k_ll_large<NT>  FP64, packed triangle in a global-memory workspace slot: blocks too large
+//                   for k_ll_fix, and the mixed path's fallback
 #include <cuda_runtime.h>
 #include <math.h>
 #include <stdint.h>
@@ -37,207 +37,6 @@
 #include "bv_ll_block.cuh"
 
 namespace {
-
-// ---------------------------------------------------------------------------------
-// FP64, shared memory.  Layout (doubles): A packed (N+1)(N+2)/2 | col[2 or 4][N+1] | pts[d][N]
-// ---------------------------------------------------------------------------------
-
-// Column c of the factor, by one warp: its entries in rows c..N have been updated with
-// every column before it except those in `prev` (np of them, each a finished column held
-// contiguously by row, applied here in order); then the pivot and the scaling, the scaled
-// column written to A and to out.  Raises *fail on a bad pivot.
-template <int NP>
-__device__ __forceinline__ void fp64_column(double* A, int c, int N, int lane, const double* const (&prev)[NP], int np,
-                                            double* out, int* fail) {
-    for (int j = c + lane; j <= N; j += 32) {
-        double v = A[pk(j, c)];
-#pragma unroll
-        for (int q = 0; q < NP; ++q)
-            if (q < np) v = fma(-prev[q][j], prev[q][c], v);
-        A[pk(j, c)] = v;
-    }
-    __syncwarp();
-    const double p = A[pk(c, c)];
-    if (bad_pivot(p) && lane == 0) *fail = 1;
-    const double rs = rsqrt(p);
-    for (int j = c + 1 + lane; j <= N; j += 32) {
-        const double v = A[pk(j, c)] * rs;
-        A[pk(j, c)] = v;
-        out[j] = v;
-    }
-    __syncwarp();
-}
-
-// W2 selects the step width of the factorisation: one column per barrier (two column
-// buffers) or two (four buffers); both give the same results bit for bit, and the planner
-// times both per size bin (one column wins on small blocks, where the panel warp's pivot
-// chain is the critical path, two on large ones, where the trailing update is).
-template <int NT, bool GEN, bool W2>
-__global__ void __launch_bounds__(NT) k_ll_fp64(LLArgs a) {
-    extern __shared__ __align__(16) unsigned char smraw[];
-    double* sm = reinterpret_cast<double*>(smraw);
-    __shared__ double etab[BV_EXP_TAB];
-    __shared__ int s_fail;
-    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    for (int i = tid; i < BV_EXP_TAB; i += NT) etab[i] = a.ex.tab[i];
-    const double eK = a.ex.k, eL1 = a.ex.l1, eL2 = a.ex.l2;
-
-    __shared__ int s_w;
-    const int nwork = work_count(a);
-    if (tid == 0) s_w = take_work(a.ctr, blockIdx.x);
-    __syncthreads();
-    for (int w = s_w; w < nwork; w = s_w) {
-        const int nx = tid == 0 ? take_work(a.ctr, w + gridDim.x) : 0;
-        const int blk = a.work[w];
-        const int64_t b0 = a.bptr[blk], n0 = a.nptr[blk];
-        const int b = (int)(a.bptr[blk + 1] - b0), m = (int)(a.nptr[blk + 1] - n0);
-        const int N = m + b, R = N + 1;
-        const DevTheta th = a.theta[a.bds[blk]];
-        double* A = sm;
-        double* colbuf = A + ((R * (R + 1)) >> 1);  // column buffers of R doubles
-        double* px = colbuf + (W2 ? 4 : 2) * R;
-        const int d = a.d;
-
-        // gather: conditioning points first, then the block (Algorithm 1 order)
-        for (int t = tid; t < N; t += NT) {
-            const int g = t < m ? a.nidx[n0 + t] : a.pidx[b0 + (t - m)];
-            for (int k = 0; k < d; ++k) px[k * N + t] = a.locs[(int64_t)k * a.n_tot + g] * inv_range_k(th, k);
-            A[pk(N, t)] = a.y[g];
-            A[pk(t, t)] = th.sigma2 + th.nugget;  // diagonal of Eq. 5 + nugget: rho(0) = 1
-        }
-        if (tid == 0) {
-            A[pk(N, N)] = 0.0;
-            s_fail = 0;
-        }
-        __syncthreads();
-
-        // covariance (Eq. 5), strictly lower triangle of rows 1..N-1: flat index f over that
-        // triangle maps to (r' + 1, c) with (r', c) = tri_rc(f), packed index f + r' + 1
-        const int T = (N * (N - 1)) >> 1;
-        for (int f = tid; f < T; f += NT) {
-            int r, c;
-            tri_rc(f, r, c);
-            ++r;
-            double acc = 0.0;
-            for (int k = 0; k < d; ++k) {
-                const double t = px[k * N + r] - px[k * N + c];
-                acc = fma(t, t, acc);
-            }
-            // x = acc / sqrt(acc) through the reciprocal square root (within 2 ulp)
-            const double x = dist_of(acc);
-            const double v = GEN ? matern64g(a.gtab + (int64_t)a.bds[blk] * GTAB_SIZE, a.theta + a.bds[blk],
-                                             th.nu_code, th.sigma2, x, etab, eK, eL1, eL2)
-                                 : matern64t(th.nu_code, th.sigma2, x, etab, eK, eL1, eL2);
-            A[f + r] = v;
-        }
-        __syncthreads();
-
-        if constexpr (!W2) {
-            // column 0 (warp 0)
-            if (warp == 0) {
-                const double* none[1] = {nullptr};
-                fp64_column<1>(A, 0, N, lane, none, 0, colbuf, &s_fail);
-            }
-            __syncthreads();
-
-            // right-looking steps: warp 0 finishes column k+1 (update, pivot, scale) while
-            // the other warps apply column k to the rest of the trailing triangle; one
-            // barrier per step
-            for (int k = 0; k + 1 < N; ++k) {
-                const double* cur = colbuf + (k & 1) * R;
-                double* nxt = colbuf + ((k & 1) ^ 1) * R;
-                const int kk = k + 1;
-                if (warp == 0) {
-                    const double* p1[1] = {cur};
-                    fp64_column<1>(A, kk, N, lane, p1, 1, nxt, &s_fail);
-                } else {
-                    // rows kk+1..N, columns kk+1..row, two independent elements per iteration
-                    const int S = N - kk;
-                    const int TS = (S * (S + 1)) >> 1;
-                    constexpr int NU = NT - 32;
-                    for (int f = tid - 32; f < TS; f += 2 * NU) {
-                        int r1, c1, r2, c2;
-                        tri_rc(f, r1, c1);
-                        const bool two = f + NU < TS;
-                        tri_rc(two ? f + NU : f, r2, c2);
-                        const int j1 = kk + 1 + r1, i1 = kk + 1 + c1, j2 = kk + 1 + r2, i2 = kk + 1 + c2;
-                        const double a1 = A[pk(j1, i1)], x1 = cur[j1], y1 = cur[i1];
-                        const double a2 = A[pk(j2, i2)], x2 = cur[j2], y2 = cur[i2];
-                        A[pk(j1, i1)] = fma(-x1, y1, a1);
-                        if (two) A[pk(j2, i2)] = fma(-x2, y2, a2);
-                    }
-                }
-                __syncthreads();
-            }
-        } else {
-            // columns 0 and 1 (warp 0)
-            if (warp == 0) {
-                const double* none[1] = {nullptr};
-                fp64_column<1>(A, 0, N, lane, none, 0, colbuf, &s_fail);
-                if (N > 1) {
-                    const double* p0[1] = {colbuf};
-                    fp64_column<1>(A, 1, N, lane, p0, 1, colbuf + R, &s_fail);
-                }
-            }
-            __syncthreads();
-
-            // right-looking steps of two columns: with columns k and k+1 finished (buffers
-            // c0, c1), warp 0 finishes columns k+2 and k+3 (their updates by k and k+1, then
-            // k+3's by k+2; pivots; scaling) while the other warps apply columns k and k+1 to
-            // the trailing triangle from row and column k+4; one barrier per two columns.
-            // Every entry receives its updates in column order, as in a one-column-per-step
-            // factorisation, so the results are the same bit for bit.
-            for (int k = 0; k + 2 < N; k += 2) {
-                const int sel = (k >> 1) & 1;
-                const double* c0 = colbuf + (2 * sel) * R;
-                const double* c1 = c0 + R;
-                double* n0b = colbuf + (2 * (sel ^ 1)) * R;
-                double* n1b = n0b + R;
-                if (warp == 0) {
-                    const double* p2[2] = {c0, c1};
-                    fp64_column<2>(A, k + 2, N, lane, p2, 2, n0b, &s_fail);
-                    if (k + 3 < N) {
-                        const double* p3[3] = {c0, c1, n0b};
-                        fp64_column<3>(A, k + 3, N, lane, p3, 3, n1b, &s_fail);
-                    }
-                } else {
-                    const int kk = k + 4;  // trailing triangle: rows kk..N, columns kk..row
-                    const int S = N - kk + 1;
-                    if (S > 0) {
-                        const int TS = (S * (S + 1)) >> 1;
-                        constexpr int NU = NT - 32;
-                        for (int f = tid - 32; f < TS; f += NU) {
-                            int r, c;
-                            tri_rc(f, r, c);
-                            const int j = kk + r, i = kk + c;
-                            const double v = fma(-c0[j], c0[i], A[pk(j, i)]);
-                            A[pk(j, i)] = fma(-c1[j], c1[i], v);
-                        }
-                    }
-                }
-                __syncthreads();
-            }
-        }
-
-        // u + d over the block columns (warp 0)
-        if (warp == 0) {
-            const double2 s2 = warp_terms(m, N, lane, [&](int k) { return A[pk(N, k)]; },
-                                          [&](int k) { return log(A[pk(k, k)]); });
-            const double s = s2.x, su = s2.y;
-            if (lane == 0) {
-                double ell = -0.5 * (s + (double)b * kLog2Pi);
-                if (s_fail || !(ell == ell)) {
-                    ell = -INFINITY;
-                    record_fail(a.fail, blk);
-                }
-                a.ell_blk[blk] = ell;
-                a.u_blk[blk] = su;
-                s_w = nx;
-            }
-        }
-        __syncthreads();
-    }
-}
 
 // ---------------------------------------------------------------------------------
 // Mixed: FP32 covariance and updates, FP64 log-determinant and quadratic form.
@@ -547,100 +346,6 @@ __global__ void __launch_bounds__(NT) k_ll_mixed_w(LLArgs a, int region_floats) 
         const double2 part = mixed_block<32, true, GEN>(a, blk, sm, lane, &s_fail[warp], t32);
         __syncwarp();
         if (lane == 0) finish_block(a, blk, (int)(a.bptr[blk + 1] - a.bptr[blk]), part.x, part.y, s_fail[warp]);
-        __syncwarp();
-        w = __shfl_sync(0xffffffffu, nx, 0);
-    }
-}
-
-// ---------------------------------------------------------------------------------
-// FP64, one warp per block (several blocks per CTA): for small blocks, where a CTA's
-// barriers and partly filled update warps cost more than the work.  Same arithmetic as
-// k_ll_fp64 (gather with the diagonal, strictly-lower covariance, right-looking Cholesky
-// of the augmented matrix, Algorithm 1 order); every column's pivot, scaling and trailing
-// update by the warp's 32 lanes with warp synchronisation only.  Layout per warp
-// (doubles, region_doubles each): A packed (N+1)(N+2)/2 | col[N+1] | pts[d][N].
-// ---------------------------------------------------------------------------------
-template <int NT, bool GEN>
-__global__ void __launch_bounds__(NT) k_ll_fp64_w(LLArgs a, int region_doubles) {
-    extern __shared__ __align__(16) unsigned char smraw[];
-    constexpr int WPB = NT / 32;
-    __shared__ double etab[BV_EXP_TAB];
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    for (int i = threadIdx.x; i < BV_EXP_TAB; i += NT) etab[i] = a.ex.tab[i];
-    __syncthreads();
-    const double eK = a.ex.k, eL1 = a.ex.l1, eL2 = a.ex.l2;
-    double* A = reinterpret_cast<double*>(smraw) + (size_t)warp * region_doubles;
-    const int nwork = work_count(a);
-    int w = __shfl_sync(0xffffffffu, lane == 0 ? take_work(a.ctr, blockIdx.x * WPB + warp) : 0, 0);
-    while (w < nwork) {
-        const int nx = lane == 0 ? take_work(a.ctr, w + gridDim.x * WPB) : 0;
-        const int blk = a.work[w];
-        const int64_t b0 = a.bptr[blk], n0 = a.nptr[blk];
-        const int b = (int)(a.bptr[blk + 1] - b0), m = (int)(a.nptr[blk + 1] - n0);
-        const int N = m + b, R = N + 1;
-        const DevTheta th = a.theta[a.bds[blk]];
-        double* col = A + ((R * (R + 1)) >> 1);
-        double* px = col + R;
-        const int d = a.d;
-
-        for (int t = lane; t < N; t += 32) {
-            const int g = t < m ? a.nidx[n0 + t] : a.pidx[b0 + (t - m)];
-            for (int k = 0; k < d; ++k) px[k * N + t] = a.locs[(int64_t)k * a.n_tot + g] * inv_range_k(th, k);
-            A[pk(N, t)] = a.y[g];
-            A[pk(t, t)] = th.sigma2 + th.nugget;
-        }
-        if (lane == 0) A[pk(N, N)] = 0.0;
-        __syncwarp();
-        const int T = (N * (N - 1)) >> 1;
-        for (int f = lane; f < T; f += 32) {
-            int r, c;
-            tri_rc(f, r, c);
-            ++r;
-            double acc = 0.0;
-            for (int k = 0; k < d; ++k) {
-                const double t = px[k * N + r] - px[k * N + c];
-                acc = fma(t, t, acc);
-            }
-            const double x = dist_of(acc);
-            A[f + r] = GEN ? matern64g(a.gtab + (int64_t)a.bds[blk] * GTAB_SIZE, a.theta + a.bds[blk], th.nu_code,
-                                       th.sigma2, x, etab, eK, eL1, eL2)
-                           : matern64t(th.nu_code, th.sigma2, x, etab, eK, eL1, eL2);
-        }
-        __syncwarp();
-
-        bool bad = false;  // the same pivot in every lane: warp-uniform
-        for (int k = 0; k < N; ++k) {
-            const double p = A[pk(k, k)];
-            bad = bad || bad_pivot(p);
-            const double rs = rsqrt(p);
-            for (int j = k + 1 + lane; j <= N; j += 32) {
-                const double v = A[pk(j, k)] * rs;
-                A[pk(j, k)] = v;
-                col[j] = v;
-            }
-            __syncwarp();
-            // trailing triangle, rows and columns k+1..N (row N: the forward solve of y)
-            const int S = N - k;
-            const int TS = (S * (S + 1)) >> 1;
-            for (int f = lane; f < TS; f += 32) {
-                int r, c;
-                tri_rc(f, r, c);
-                const int j = k + 1 + r, i = k + 1 + c;
-                A[pk(j, i)] = fma(-col[j], col[i], A[pk(j, i)]);
-            }
-            __syncwarp();
-        }
-        const double2 s2 = warp_terms(m, N, lane, [&](int k) { return A[pk(N, k)]; },
-                                      [&](int k) { return log(A[pk(k, k)]); });
-        if (lane == 0) {
-            double ell = -0.5 * (s2.x + (double)b * kLog2Pi);
-            if (bad || !(ell == ell)) {
-                ell = -INFINITY;
-                record_fail(a.fail, blk);
-            }
-            a.ell_blk[blk] = ell;
-            a.u_blk[blk] = s2.y;
-        }
         __syncwarp();
         w = __shfl_sync(0xffffffffu, nx, 0);
     }
@@ -994,8 +699,21 @@ __global__ void k_exp_check(const double* x, double* out, int64_t n, ExpConsts e
     if (i < n) out[i] = exp_neg(x[i], ex.tab, ex.k, ex.l1, ex.l2);
 }
 
+// Coefficient of t^j in the Chebyshev polynomial T_k, at k GTAB_DEG + j (whole numbers).
+struct ChebPow {
+    double m[GTAB_DEG * GTAB_DEG];
+    constexpr ChebPow() : m() {
+        for (int k = 0; k < GTAB_DEG; ++k)
+            for (int j = 0; j <= k; ++j)
+                m[k * GTAB_DEG + j] = k < 2 ? (j == k ? 1.0 : 0.0)
+                                            : (j > 0 ? 2.0 * m[(k - 1) * GTAB_DEG + j - 1] : 0.0) - m[(k - 2) * GTAB_DEG + j];
+    }
+};
+__constant__ ChebPow c_cheb_pow = ChebPow();
+
 // One CTA per dataset: L(x) = x + log rho(x) at the Chebyshev nodes of every octave, then
-// the coefficients c_k = (2 / D) sum_j L_j cos(pi k (j + 1/2) / D), c_0 halved.
+// the coefficients c_k = (2 / D) sum_j L_j cos(pi k (j + 1/2) / D), c_0 halved; and the same
+// polynomials in the power basis, in units 2^-57, after the doubles of all datasets.
 __global__ void __launch_bounds__(1024) k_gtab_build(const DevTheta* theta, double* gtab) {
     __shared__ double node[GTAB_SIZE];
     const DevTheta* g = theta + blockIdx.x;
@@ -1015,6 +733,16 @@ __global__ void __launch_bounds__(1024) k_gtab_build(const DevTheta* theta, doub
         s *= 2.0 / GTAB_DEG;
         out[f] = k == 0 ? 0.5 * s : s;
     }
+    __syncthreads();
+    for (int f = threadIdx.x; f < GTAB_SIZE; f += blockDim.x) node[f] = out[f];
+    __syncthreads();
+    long long* outi = reinterpret_cast<long long*>(gtab) + ((int64_t)gridDim.x + blockIdx.x) * GTAB_SIZE;
+    for (int f = threadIdx.x; f < GTAB_SIZE; f += blockDim.x) {
+        const int o = f / GTAB_DEG, j = f % GTAB_DEG;
+        double s = 0.0;
+        for (int k = GTAB_DEG - 1; k >= j; --k) s = fma(c_cheb_pow.m[k * GTAB_DEG + j], node[o * GTAB_DEG + k], s);
+        outi[f] = __double2ll_rn(s * 0x1p57);
+    }
 }
 
 __global__ void k_matern_check(const double* x, double* out, int64_t n, const DevTheta* th, const double* gtab,
@@ -1031,20 +759,11 @@ __global__ void k_matern_check(const double* x, double* out, int64_t n, const De
 // stay valid when a smaller bin is launched later).
 constexpr int kSmemCap = 227 * 1024 - 3072;
 
-// NT = 1024 (one panel warp and 31 update warps) exists for the FP64 CTA kernels only:
-// their large blocks run one CTA per SM, where more update warps hide more latency.
 template <int NT, bool GEN>
 cudaError_t set_smem_cap_g() {
-    cudaError_t e = cudaFuncSetAttribute(k_ll_fp64<NT, GEN, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemCap);
-    if (e == cudaSuccess)
-        e = cudaFuncSetAttribute(k_ll_fp64<NT, GEN, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemCap);
-    if constexpr (NT == 1024) return e;
-    if (e == cudaSuccess)
-        e = cudaFuncSetAttribute(k_ll_mixed<NT, GEN>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemCap);
+    cudaError_t e = cudaFuncSetAttribute(k_ll_mixed<NT, GEN>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemCap);
     if (e == cudaSuccess)
         e = cudaFuncSetAttribute(k_ll_mixed_w<NT, GEN>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemCap);
-    if (e == cudaSuccess)
-        e = cudaFuncSetAttribute(k_ll_fp64_w<NT, GEN>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemCap);
     return e;
 }
 
@@ -1058,12 +777,8 @@ cudaError_t set_smem_cap() {
 // any dataset's nu is not 1/2, 3/2 or 5/2); the others carry no call in their inner loops.
 template <int NT, bool GEN>
 cudaError_t launch_kind_g(int kind, int grid, size_t smem, const LLArgs& a, cudaStream_t s) {
-    if (kind == 0) k_ll_fp64<NT, GEN, false><<<grid, NT, smem, s>>>(a);
-    else if (kind == 6) k_ll_fp64<NT, GEN, true><<<grid, NT, smem, s>>>(a);
-    else if constexpr (NT == 1024) return cudaErrorInvalidValue;
-    else if (kind == 1) k_ll_mixed<NT, GEN><<<grid, NT, smem, s>>>(a);
+    if (kind == 1) k_ll_mixed<NT, GEN><<<grid, NT, smem, s>>>(a);
     else if (kind == 3) k_ll_mixed_w<NT, GEN><<<grid, NT, smem, s>>>(a, (int)(smem / sizeof(float) / (NT / 32)));
-    else if (kind == 4) k_ll_fp64_w<NT, GEN><<<grid, NT, smem, s>>>(a, (int)(smem / sizeof(double) / (NT / 32)));
     else k_ll_large<NT, GEN><<<grid, NT, 0, s>>>(a);
     return cudaGetLastError();
 }
@@ -1081,19 +796,10 @@ cudaError_t launch_kind(int kind, int grid, size_t smem, const LLArgs& a, cudaSt
 
 // Shared-memory footprint of one CTA for augmented size N.
 size_t bv_smem_bytes(int kind, int nmax, int d, int threads) {
-    (void)threads;
-    const size_t R = (size_t)nmax + 1;
-    const size_t el = kind == 1 ? sizeof(float) : sizeof(double);
     if (kind == 2) return 0;
     if (kind == 5) return bv_tc_smem_bytes(nmax);
-    if (kind == 1) return sizeof(float) * (size_t)mixed_floats(nmax);
-    if (kind == 3) return sizeof(float) * (size_t)mixed_floats(nmax) * (size_t)(threads / 32);
-    if (kind == 4) {  // one region per warp, each a multiple of 16 bytes
-        const size_t region = (R * (R + 1) / 2 + R + (size_t)d * nmax + 1) & ~(size_t)1;
-        return sizeof(double) * region * (size_t)(threads / 32);
-    }
-    size_t bytes = el * (R * (R + 1) / 2 + (kind == 6 ? 4 : 2) * R + (size_t)d * nmax);
-    return (bytes + 15) & ~(size_t)15;
+    if (kind == 7 || kind == 8) return bv_fix_smem_bytes(kind, nmax, d);
+    return sizeof(float) * (size_t)mixed_floats(nmax) * (size_t)(kind == 3 ? threads / 32 : 1);
 }
 
 // Largest N the shared-memory kernels take (227 KB opt-in per CTA, minus static smem).
@@ -1104,7 +810,6 @@ int bv_smem_max_n(int kind, int d) {
     return n;
 }
 
-int bv_max_threads_for(int kind) { return kind == 2 ? 256 : 544; }
 
 cudaError_t bv_launch_bin(const BinPlan& bp, const LLArgs& a0, cudaStream_t s) {
     if (bp.nwork == 0) return cudaSuccess;
@@ -1113,6 +818,11 @@ cudaError_t bv_launch_bin(const BinPlan& bp, const LLArgs& a0, cudaStream_t s) {
     a.nwork = bp.nwork;
     a.ctr = bp.d_ctr;
     if (bp.kind == 5) return bv_tc_launch(bp.threads, bp.grid, bp.smem, a, s);
+    if (bp.kind == 7 || bp.kind == 8) {
+        a.ws = bp.d_slots;
+        a.ws_stride = bp.slot_stride;
+        return bv_fix_launch(bp.kind, bp.threads, bp.grid, bp.smem, a, s);
+    }
     switch (bp.threads) {
         case 64: return launch_kind<64>(bp.kind, bp.grid, bp.smem, a, s);
         case 128: return launch_kind<128>(bp.kind, bp.grid, bp.smem, a, s);
@@ -1121,7 +831,6 @@ cudaError_t bv_launch_bin(const BinPlan& bp, const LLArgs& a0, cudaStream_t s) {
         case 288: return launch_kind<288>(bp.kind, bp.grid, bp.smem, a, s);
         case 544: return launch_kind<544>(bp.kind, bp.grid, bp.smem, a, s);
         case 256: return launch_kind<256>(bp.kind, bp.grid, bp.smem, a, s);
-        case 1024: return launch_kind<1024>(bp.kind, bp.grid, bp.smem, a, s);
         default: return cudaErrorInvalidValue;
     }
 }
@@ -1186,34 +895,23 @@ cudaError_t bv_launch_eval_reset(unsigned long long* fail, int* ctr, int n, cuda
 // Occupancy helper for the planner.
 int bv_occupancy(int kind, int threads, size_t smem) {
     if (kind == 5) return bv_tc_occupancy(threads, smem);
+    if (kind == 7 || kind == 8) return bv_fix_occupancy(kind, threads, smem);
     int nb = 0;
     cudaError_t e = cudaSuccess;
 #define BV_OCC(NT)                                                                            \
     if (threads == NT) {                                                                      \
         if (kind != 2) e = set_smem_cap<NT>();                                                \
         if (e == cudaSuccess) {                                                               \
-            if (kind == 0)                                                                    \
-                e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_ll_fp64<NT, false, false>, NT, smem); \
-            else if (kind == 6)                                                               \
-                e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_ll_fp64<NT, false, true>, NT, smem); \
-            else if (kind == 1)                                                               \
+            if (kind == 1)                                                                    \
                 e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_ll_mixed<NT, false>, NT, smem); \
             else if (kind == 3)                                                               \
                 e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_ll_mixed_w<NT, false>, NT, smem); \
-            else if (kind == 4)                                                               \
-                e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_ll_fp64_w<NT, false>, NT, smem); \
             else                                                                              \
                 e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_ll_large<NT, false>, NT, 0);    \
         }                                                                                     \
     }
     BV_OCC(64) BV_OCC(128) BV_OCC(96) BV_OCC(160) BV_OCC(288) BV_OCC(544) BV_OCC(256)
 #undef BV_OCC
-    if (threads == 1024 && (kind == 0 || kind == 6)) {
-        e = set_smem_cap<1024>();
-        if (e == cudaSuccess)
-            e = kind == 0 ? cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_ll_fp64<1024, false, false>, 1024, smem)
-                          : cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_ll_fp64<1024, false, true>, 1024, smem);
-    }
     if (e != cudaSuccess) return 0;
     return nb;
 }
@@ -1321,7 +1019,7 @@ extern "C" int bv_matern_check(double nu, int32_t tabulated, int64_t n, const do
     BV_CUDA(cudaMalloc(&dx, sizeof(double) * n));
     BV_CUDA(cudaMalloc(&dy, sizeof(double) * n));
     BV_CUDA(cudaMalloc(&dth, sizeof(DevTheta)));
-    BV_CUDA(cudaMalloc(&dtab, sizeof(double) * GTAB_SIZE));
+    BV_CUDA(cudaMalloc(&dtab, sizeof(double) * 2 * GTAB_SIZE));
     BV_CUDA(cudaMemcpy(dx, x, sizeof(double) * n, cudaMemcpyHostToDevice));
     BV_CUDA(cudaMemcpy(dth, &th, sizeof(DevTheta), cudaMemcpyHostToDevice));
     k_gtab_build<<<1, 1024>>>(dth, dtab);
