@@ -2,16 +2,19 @@
 // factorisation on the GPU, and the KL divergence of the block-Vecchia approximation
 // (Eq. 7 of Sec. 3.1: KL = ell_0(theta; 0) - ell_a(theta; 0)).
 //
-// The (n+1) x (n+1) augmented matrix [[Sigma, .], [y^T, .]] is padded to a multiple of
-// the tile size T with an identity block and stored as packed lower T x T tiles (tile
-// (i, j), j <= i, at (i(i+1)/2 + j) T^2, row-major inside).  Right-looking tiled
-// Cholesky, three launches per tile column k:
-//   k_potrf   the diagonal tile (one CTA, shared memory)
-//   k_trsm    L_ik = A_ik L_kk^-T for every tile below it (one CTA per tile)
-//   k_update  A_ij -= L_ik L_jk^T for every trailing tile (one CTA per tile, 4 x 4 outputs
-//             per thread from shared-memory operands)
-// The factor's row n is z = L^-1 y, so y^T Sigma^-1 y = |z|^2 and log|Sigma| = 2 sum log
-// L_ii.  The pivot of row n itself is not part of Sigma and is set to 1.
+// The (n+1) x (n+1) augmented matrix [[Sigma, .], [y^T, .]], divided by the diagonal D =
+// sigma^2 + tau^2, in the fixed-point form of bv_fix_tile.cuh: packed lower 16 x 16 tiles of
+// 64-bit entries, products of factor entries on the tensor cores through their digits.  At n =
+// 8,000 26.8 ms; FP64 arithmetic, 2 lanes a clock and SM, took 188.7 ms (n^3 / 3 operations at
+// 72% of its peak).  Right-looking by panels of 64 columns (four tiles), three launches a panel:
+//   k_ex_diag    the 64 x 64 diagonal block, one CTA
+//   k_ex_rows    the rows below it, 32 of them a warp: four solves against the 16 x 16
+//                diagonal tiles with the updates between them, and the rows' digits
+//   k_ex_update  A_IJ -= sum over the panel's four tiles of L_I L_J^T, a CTA per 64 x 64 block,
+//                the sums of a block kept in registers so that it is read and written once
+// The factor's row n is z = L^-1 y, so y^T Sigma^-1 y = |z|^2 and log|Sigma| is the sum of the
+// pivots' logarithms.  The data row is scaled by a power of two; should a solved entry leave
+// the fixed-point range, the factorisation is done again with a larger one.
 #include <cuda_runtime.h>
 #include <math.h>
 #include <stdint.h>
@@ -20,182 +23,233 @@
 #include <vector>
 
 #include "bv_device.cuh"
+#include "bv_fix_tile.cuh"
 #include "bv_internal.h"
 
 namespace {
 
-constexpr int T = 64;          // tile edge
-constexpr int TT = T * T;
-constexpr int kUpdNT = 256;    // 16 x 16 threads, 4 x 4 outputs each
+constexpr int kP = 4;                                     // tiles of a panel
+constexpr int kLdN = 16 * kLd + 16;                       // entries of a tile's factor in memory
 
-__device__ __forceinline__ int64_t tile_off(int64_t i, int64_t j) { return ((i * (i + 1)) / 2 + j) * TT; }
+__device__ __forceinline__ int64_t etile(int64_t I, int64_t J) { return ((I * (I + 1)) / 2 + J) * 128; }
 
-__device__ __forceinline__ double matern_exact(const DevTheta& th, double x) {
-    if (th.nu_code == NU_GENERAL) return th.sigma2 * matern_gen_corr(th, x);
-    const double e = exp(-x);
-    if (th.nu_code == NU_HALF) return th.sigma2 * e;
-    if (th.nu_code == NU_3HALF) return th.sigma2 * ((1.0 + x) * e);
-    return th.sigma2 * ((1.0 + x * (1.0 + x * (1.0 / 3.0))) * e);
-}
-
-struct FillArgs {
+struct ExArgs {
     const double* locs;  // SoA d x n
     const double* y;     // null: y = 0
     int64_t n;
     int d;
-    int64_t nt;
+    int T, TC;           // tile rows of the n + 1 rows, tile columns of the n columns
     DevTheta th;
-    double* A;
+    longlong2* A;        // packed lower tiles
+    uint32_t* dig;       // digits of the panel's rows: tile row I, panel tile s at (I kP + s)
+    int4* Ld;            // the panel's four diagonal factors, their reciprocal roots and the
+    FixRs* rsv;          // digits of the tiles between them (i, s), i > s, at i (i - 1) / 2 + s
+    uint32_t* ddig;
+    int64_t* piv;        // pivots and data row, by column
+    int64_t* zrow;
+    const uint64_t* fixtab;
+    int E;               // data row in units of 2^(E - 60) sqrt(D)
+    int* flags;
 };
 
-// One CTA per lower tile (blockIdx.x = packed tile index).
-__global__ void __launch_bounds__(256) k_fill(FillArgs a) {
-    const int64_t f = blockIdx.x;
-    int64_t ti = (int64_t)((sqrt(8.0 * (double)f + 1.0) - 1.0) * 0.5);
-    while ((ti + 1) * (ti + 2) / 2 <= f) ++ti;
-    while (ti * (ti + 1) / 2 > f) --ti;
-    const int64_t tj = f - ti * (ti + 1) / 2;
-    double* out = a.A + f * TT;
-    for (int e = threadIdx.x; e < TT; e += 256) {
-        const int64_t r = ti * T + e / T, c = tj * T + e % T;
-        double v = 0.0;
-        if (c > r) {
-            v = 0.0;
-        } else if (r < a.n) {
+// One warp per tile.
+template <bool GEN>
+__global__ void __launch_bounds__(256) k_ex_fill(ExArgs a, int64_t ntiles) {
+    __shared__ uint64_t tA[256], tB[256];
+    const uint64_t rf = (uint64_t)__double2ull_rn(a.th.diag_ratio * 0x1p63);
+    tA[threadIdx.x] = bvfix::mulhi64(a.fixtab[threadIdx.x], rf) << 1;
+    tB[threadIdx.x] = a.fixtab[256 + threadIdx.x];
+    __syncthreads();
+    const int lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3;
+    const int64_t f = (int64_t)blockIdx.x * 8 + (threadIdx.x >> 5);
+    if (f >= ntiles) return;
+    int64_t I = (int64_t)((sqrt(8.0 * (double)f + 1.0) - 1.0) * 0.5);
+    while ((I + 1) * (I + 2) / 2 <= f) ++I;
+    while (I * (I + 1) / 2 > f) --I;
+    const int64_t J = f - I * (I + 1) / 2, n = a.n;
+    longlong2* tp = a.A + f * 128;
+#pragma unroll 1
+    for (int s = 0; s < 4; ++s) {
+        const int64_t r = 16 * I + g + 8 * (s & 1), c0 = 16 * J + 8 * (s >> 1) + 2 * t;
+        int64_t v[2];
+#pragma unroll
+        for (int e = 0; e < 2; ++e) {
+            const int64_t c = c0 + e, rr = min(r, n - 1), cc = min(c, n - 1);
             double acc = 0.0;
             for (int k = 0; k < a.d; ++k) {
-                const double t = (a.locs[k * a.n + r] - a.locs[k * a.n + c]) * inv_range_k(a.th, k);
-                acc = fma(t, t, acc);
+                const double dt = (a.locs[k * n + rr] - a.locs[k * n + cc]) * inv_range_k(a.th, k);
+                acc = fma(dt, dt, acc);
             }
-            v = matern_exact(a.th, sqrt(acc));
-            if (r == c) v += a.th.nugget;
-        } else if (r == a.n) {
-            v = c < a.n ? (a.y ? a.y[c] : 0.0) : 1.0;
-        } else {
-            v = (r == c) ? 1.0 : 0.0;
+            const int ex = (int)(bvfix::dbits(acc) >> 52);
+            if (ex == 0x7ff) atomicOr(a.flags, kFail);
+            if (GEN) v[e] = bvfix::unit_fix(fmin(matern_gen_corr(a.th, sqrt(acc)), 1.0) * a.th.diag_ratio);
+            else if (ex == 0) v[e] = (int64_t)(tA[0] >> 2);
+            else if (a.th.nu_code == NU_HALF) v[e] = bvfix::matern_fix<0>(bvfix::dist_fix(bvfix::dbits(acc)), tA, tB);
+            else if (a.th.nu_code == NU_3HALF) v[e] = bvfix::matern_fix<1>(bvfix::dist_fix(bvfix::dbits(acc)), tA, tB);
+            else v[e] = bvfix::matern_fix<2>(bvfix::dist_fix(bvfix::dbits(acc)), tA, tB);
+            if (c >= r || r >= n) v[e] = c == r ? 1ll << bvfix::kUnitC : 0;
+            if (r == n && c < n && a.y) v[e] = __double2ll_rn(ldexp(a.y[c] * a.th.diag_rsqrt, bvfix::kUnitC - a.E));
         }
-        out[e] = v;
+        tp[((s >> 1) * 2 + (s & 1)) * 32 + lane] = make_longlong2(v[0], v[1]);
     }
 }
 
-// Unblocked right-looking Cholesky of diagonal tile k in shared memory.  Row `yrow` (the
-// data row, global index n) gets pivot 1; a non-positive pivot elsewhere sets *fail.
-__global__ void __launch_bounds__(256) k_potrf(double* A, int64_t k, int64_t yrow, unsigned long long* fail) {
-    __shared__ double s[TT];
-    double* t = A + tile_off(k, k);
-    for (int e = threadIdx.x; e < TT; e += 256) s[e] = t[e];
-    __syncthreads();
-    for (int c = 0; c < T; ++c) {
-        const int64_t g = k * T + c;
-        if (threadIdx.x == 0) {
-            double p = s[c * T + c];
-            if (g == yrow) {
-                p = 1.0;
-            } else if (!(p > 0.0)) {
-                atomicMin(fail, (unsigned long long)g);
-                p = 1.0;
-            } else {
-                p = sqrt(p);
-            }
-            s[c * T + c] = p;
-        }
-        __syncthreads();
-        const double rl = 1.0 / s[c * T + c];
-        for (int r = c + 1 + threadIdx.x; r < T; r += 256) s[r * T + c] *= rl;
-        __syncthreads();
-        for (int e = threadIdx.x; e < TT; e += 256) {
-            const int r = e / T, q = e % T;
-            if (q > c && q <= r) s[e] = fma(-s[r * T + c], s[q * T + c], s[e]);
-        }
-        __syncthreads();
-    }
-    for (int e = threadIdx.x; e < TT; e += 256) t[e] = s[e];
+// Largest high word of |y| / sqrt(D).
+__global__ void __launch_bounds__(256) k_ex_ymax(const double* y, int64_t n, double isd, unsigned* out) {
+    unsigned m = 0;
+    for (int64_t i = blockIdx.x * 256ll + threadIdx.x; i < n; i += 256ll * gridDim.x)
+        m = max(m, (unsigned)__double2hiint(y[i] * isd) & 0x7fffffffu);
+    m = __reduce_max_sync(0xffffffffu, m);
+    if ((threadIdx.x & 31) == 0) atomicMax(out, m);
 }
 
-// L_ik = A_ik L_kk^-T for i = k+1 .. nt-1 (blockIdx.x = i - k - 1): row r of L_ik solves
-// x L_kk^T = a, column by column; 64 threads, one row each.
-constexpr size_t kTrsmSmem = sizeof(double) * (TT + T * (T + 1));
-constexpr size_t kUpdSmem = sizeof(double) * 2 * TT;
-
-__global__ void __launch_bounds__(64) k_trsm(double* A, int64_t k) {
-    extern __shared__ __align__(32) double sm[];
-    double* L = sm;
-    double* X = sm + TT;
-    const int64_t i = k + 1 + blockIdx.x;
-    const double* lk = A + tile_off(k, k);
-    double* ai = A + tile_off(i, k);
-    for (int e = threadIdx.x; e < TT; e += 64) {
-        L[e] = lk[e];
-        X[(e / T) * (T + 1) + e % T] = ai[e];
+// The diagonal block of panel P: at most 4 x 4 tiles, factored as a block of its own
+// (bv_fix_ll.cu); the bound is the chain of its 64 pivots.
+__global__ void __launch_bounds__(128) k_ex_diag(ExArgs a, int P) {
+    __shared__ longlong2 tiles[10 * 128];
+    __shared__ __align__(16) uint32_t dig[3 * kDigB / 4];
+    __shared__ int4 Ld[kLdN];
+    __shared__ FixRs rsv[16];
+    __shared__ __align__(8) uint64_t mb[8];
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int I0 = kP * P, tr = min(kP, a.T - I0), tc = min(kP, a.TC - I0);
+    if (tid < 8)
+        asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"((uint32_t)__cvta_generic_to_shared(mb + tid)) : "memory");
+    for (int q = 0; q < ((tr * (tr + 1)) >> 1); ++q) {
+        int i, j;
+        tri_rc(q, i, j);
+        tiles[q * 128 + tid] = a.A[etile(I0 + i, I0 + j) + tid];
     }
+    for (int j = tid; j < kLdN; j += 128) Ld[j] = make_int4(0, 0, 0, 0);
     __syncthreads();
-    const int r = threadIdx.x;
-    double* x = X + r * (T + 1);
-    for (int c = 0; c < T; ++c) {
-        double v = x[c];
-        for (int l = 0; l < c; ++l) v = fma(-x[l], L[c * T + l], v);
-        x[c] = v / L[c * T + c];
+    int flags = 0;
+    for (int p = 0; p < tc; ++p) {
+        const int64_t k0 = 16ll * (I0 + p);
+        const int nc = (int)min((int64_t)16, a.n - k0), rows = (tr - p - 1) << 4, ry = (int)min(a.n - k0, (int64_t)1 << 20);
+        if (warp == 0) {
+            fix_diag(tiles + ftile(p, p) * 128, nc, 0, ry, lane, Ld, rsv, a.piv + k0, a.zrow + k0, mb, flags);
+        } else if (tid - 32 < rows) {
+            const int rw = tid - 32, i = p + 1 + (rw >> 4);
+            fix_row(tiles + ftile(i, p) * 128, Ld, rsv, rw & 15, 16 * (i - p) + (rw & 15) == ry, a.zrow + k0, nc, true, mb,
+                    p & 1, dig + (rw >> 4) * (kDigB / 4), flags);
+        }
+        __syncthreads();
+        for (int j = tid; j < kLdN; j += 128) a.Ld[p * kLdN + j] = Ld[j];
+        if (tid < 16) a.rsv[p * 16 + tid] = rsv[tid];
+        for (int i = p + 1; i < tr; ++i)
+            for (int j = tid; j < kDigB / 16; j += 128)
+                reinterpret_cast<uint4*>(a.ddig + (i * (i - 1) / 2 + p) * (kDigB / 4))[j] =
+                    reinterpret_cast<const uint4*>(dig + (i - p - 1) * (kDigB / 4))[j];
+        const int S = tr - p - 1;
+        for (int q = warp; q < ((S * (S + 1)) >> 1); q += 4) {
+            int ii, jj;
+            tri_rc(q, ii, jj);
+            if (I0 + p + 1 + jj >= a.TC) continue;
+            fix_update(tiles + ftile(p + 1 + ii, p + 1 + jj) * 128, dig + ii * (kDigB / 4), dig + jj * (kDigB / 4), ii == jj,
+                       lane);
+        }
+        __syncthreads();
     }
-    __syncthreads();
-    for (int e = threadIdx.x; e < TT; e += 64) ai[e] = X[(e / T) * (T + 1) + e % T];
+    if (flags) atomicOr(a.flags, flags);
 }
 
-// A_ij -= L_ik L_jk^T for the trailing tiles k < j <= i < nt, blockIdx.x = packed index
-// of (i - k - 1, j - k - 1).  Operands staged transposed in shared memory so that each
-// thread reads its 4 rows and 4 columns of every inner step as two 32-byte loads.
-__global__ void __launch_bounds__(kUpdNT) k_update(double* A, int64_t k) {
-    extern __shared__ __align__(32) double sm[];
-    double* Ls = sm;        // Ls[l * T + r] = L_ik[r][l]
-    double* Rs = sm + TT;   // Rs[l * T + c] = L_jk[c][l]
+// The rows below panel P's diagonal block: 32 rows (two tile rows) a warp.
+constexpr size_t kRowsSmem = kP * kLdN * sizeof(int4) + kP * 16 * sizeof(FixRs) + 6 * kDigB + 4 * 2 * kDigB;
+__global__ void __launch_bounds__(128) k_ex_rows(ExArgs a, int P) {
+    extern __shared__ __align__(16) unsigned char smx[];
+    int4* Ld = reinterpret_cast<int4*>(smx);
+    FixRs* rsv = reinterpret_cast<FixRs*>(Ld + kP * kLdN);
+    uint32_t* dd = reinterpret_cast<uint32_t*>(rsv + kP * 16);
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    uint32_t* dw = dd + 6 * (kDigB / 4) + warp * 2 * (kDigB / 4);
+    const int I0 = kP * P, tc = min(kP, a.TC - I0);
+    for (int j = tid; j < tc * kLdN; j += 128) Ld[j] = a.Ld[j];
+    if (tid < tc * 16) rsv[tid] = a.rsv[tid];
+    for (int j = tid; j < 6 * kDigB / 16; j += 128) reinterpret_cast<uint4*>(dd)[j] = reinterpret_cast<const uint4*>(a.ddig)[j];
+    __syncthreads();
+    const int Iw = I0 + kP + 2 * (blockIdx.x * 4 + warp);  // the warp's first tile row
+    if (Iw >= a.T) return;
+    const int nI = min(2, a.T - Iw), I = Iw + min(lane >> 4, nI - 1);
+    int flags = 0;
+    for (int s = 0; s < tc; ++s) {
+        const int64_t k0 = 16ll * (I0 + s);
+        const int nc = (int)min((int64_t)16, a.n - k0);
+        if ((lane >> 4) < nI)
+            fix_row(a.A + etile(I, I0 + s), Ld + s * kLdN, rsv + s * 16, lane & 15, 16ll * I + (lane & 15) == a.n, a.zrow + k0,
+                    nc, false, nullptr, 0, dw + (lane >> 4) * (kDigB / 4), flags);
+        __syncwarp();
+        for (int i = 0; i < nI; ++i) {
+            uint4* out = reinterpret_cast<uint4*>(a.dig + ((int64_t)(Iw + i) * kP + s) * (kDigB / 4));
+            const uint4* src = reinterpret_cast<const uint4*>(dw + i * (kDigB / 4));
+            for (int j = lane; j < kDigB / 16; j += 32) out[j] = src[j];
+            for (int j = s + 1; j < tc; ++j)
+                fix_update(a.A + etile(Iw + i, I0 + j), dw + i * (kDigB / 4), dd + (j * (j - 1) / 2 + s) * (kDigB / 4), false,
+                           lane);
+        }
+        __syncwarp();
+    }
+    if (flags) atomicOr(a.flags, flags);
+}
+
+// Trailing 64 x 64 block (bi, bj): warp w has tile row w / 2 and two tile columns of it.
+__global__ void __launch_bounds__(256, 2) k_ex_update(ExArgs a, int P) {
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int64_t f = blockIdx.x;
-    int64_t a = (int64_t)((sqrt(8.0 * (double)f + 1.0) - 1.0) * 0.5);
-    while ((a + 1) * (a + 2) / 2 <= f) ++a;
-    while (a * (a + 1) / 2 > f) --a;
-    const int64_t b = f - a * (a + 1) / 2;
-    const int64_t i = k + 1 + a, j = k + 1 + b;
-    const double* li = A + tile_off(i, k);
-    const double* lj = A + tile_off(j, k);
-    for (int e = threadIdx.x; e < TT; e += kUpdNT) {
-        const int r = e / T, l = e % T;
-        Ls[l * T + r] = li[e];
-        Rs[l * T + r] = lj[e];
-    }
-    __syncthreads();
-    const int tr = threadIdx.x / 16, tc = threadIdx.x % 16;
-    double acc[4][4];
+    int64_t x = (int64_t)((sqrt(8.0 * (double)f + 1.0) - 1.0) * 0.5);
+    while ((x + 1) * (x + 2) / 2 <= f) ++x;
+    while (x * (x + 1) / 2 > f) --x;
+    const int bi = P + 1 + (int)x, bj = P + 1 + (int)(f - x * (x + 1) / 2);
+    const int I = kP * bi + (warp >> 1), J0 = kP * bj + 2 * (warp & 1), tc = min(kP, a.TC - kP * P);
+    if (I >= a.T || J0 > I || J0 >= a.TC) return;
+    const bool two = J0 + 1 <= I && J0 + 1 < a.TC;
+    int64_t sum[2][2][4];
 #pragma unroll
-    for (int p = 0; p < 4; ++p)
+    for (int j = 0; j < 2; ++j)
 #pragma unroll
-        for (int q = 0; q < 4; ++q) acc[p][q] = 0.0;
-#pragma unroll 4
-    for (int l = 0; l < T; ++l) {
-        const double4_32a x = *reinterpret_cast<const double4_32a*>(&Ls[l * T + 4 * tr]);
-        const double4_32a w = *reinterpret_cast<const double4_32a*>(&Rs[l * T + 4 * tc]);
-        const double xv[4] = {x.x, x.y, x.z, x.w}, wv[4] = {w.x, w.y, w.z, w.w};
+        for (int h = 0; h < 2; ++h)
 #pragma unroll
-        for (int p = 0; p < 4; ++p)
+            for (int e = 0; e < 4; ++e) sum[j][h][e] = 0;
+#pragma unroll 1
+    for (int s = 0; s < tc; ++s) {
+        uint2 A[kDig][2];
+        load_digits(A, a.dig + ((int64_t)I * kP + s) * (kDigB / 4), lane);
 #pragma unroll
-            for (int q = 0; q < 4; ++q) acc[p][q] = fma(xv[p], wv[q], acc[p][q]);
-    }
-    double* out = A + tile_off(i, j);
+        for (int j = 0; j < 2; ++j) {
+            if (j && !two) break;
+            const uint32_t* dJ = a.dig + ((int64_t)(J0 + j) * kP + s) * (kDigB / 4);
 #pragma unroll
-    for (int p = 0; p < 4; ++p)
+            for (int h = 0; h < 2; ++h) {
+                int64_t o[4];
+                digit_dot(o, A, dJ, h, I == J0 + j, lane);
 #pragma unroll
-        for (int q = 0; q < 4; ++q) {
-            const int r = 4 * tr + p, c = 4 * tc + q;
-            if (i != j || c <= r) out[r * T + c] -= acc[p][q];
+                for (int e = 0; e < 4; ++e) sum[j][h][e] += o[e];
+            }
         }
+    }
+#pragma unroll
+    for (int j = 0; j < 2; ++j) {
+        if (j && !two) break;
+        longlong2* C = a.A + etile(I, J0 + j);
+#pragma unroll
+        for (int h = 0; h < 2; ++h)
+#pragma unroll
+            for (int rr = 0; rr < 2; ++rr) {
+                longlong2 v = C[(2 * h + rr) * 32 + lane];
+                v.x -= sum[j][h][2 * rr];
+                v.y -= sum[j][h][2 * rr + 1];
+                C[(2 * h + rr) * 32 + lane] = v;
+            }
+    }
 }
 
 // log-det and quadratic form from the factor: one CTA, fixed-order sums.
-__global__ void __launch_bounds__(256) k_exact_terms(const double* A, int64_t n, double* out) {
+__global__ void __launch_bounds__(256) k_exact_terms(const int64_t* piv, const int64_t* zrow, int64_t n, double ps, double zs,
+                                                     double* out) {
     __shared__ double s1[256], s2[256];
     double ld = 0.0, q = 0.0;
-    const int64_t yt = n / T, yr = n % T;
     for (int64_t g = threadIdx.x; g < n; g += 256) {
-        const int64_t t = g / T, r = g % T;
-        ld += log(A[tile_off(t, t) + r * T + r]);
-        const double z = A[tile_off(yt, t) + yr * T + r];
+        ld += log((double)piv[g] * ps);
+        const double z = (double)zrow[g] * zs;
         q = fma(z, z, q);
     }
     s1[threadIdx.x] = ld;
@@ -207,10 +261,20 @@ __global__ void __launch_bounds__(256) k_exact_terms(const double* A, int64_t n,
             a += s1[t];
             b += s2[t];
         }
-        out[0] = 2.0 * a;
+        out[0] = a;
         out[1] = b;
     }
 }
+
+// The call's device memory, taken from the stream's pool and given back on every path.
+struct ExBuf {
+    cudaStream_t s;
+    void* p = nullptr;
+    explicit ExBuf(cudaStream_t st) : s(st) {}
+    ~ExBuf() {
+        if (p) cudaFreeAsync(p, s);
+    }
+};
 
 }  // namespace
 
@@ -224,44 +288,80 @@ extern "C" int bv_exact_loglik(bv_ctx* c, const bv_theta* theta, int32_t use_y, 
     DevTheta th;
     BV_TRY(bv_theta_to_dev(theta, c->d, &th));
     BV_CUDA(cudaSetDevice(c->device));
-    const int64_t nt = (n + 1 + T - 1) / T;
-    const int64_t ntiles = nt * (nt + 1) / 2;
-    double* A = nullptr;
-    double* terms = nullptr;
-    unsigned long long* fail = nullptr;
-    BV_CUDA(cudaMallocAsync(&A, sizeof(double) * ntiles * TT, c->stream));
-    BV_CUDA(cudaMallocAsync(&terms, sizeof(double) * 2, c->stream));
-    BV_CUDA(cudaMallocAsync(&fail, sizeof(unsigned long long), c->stream));
-    BV_CUDA(cudaMemsetAsync(fail, 0xff, sizeof(unsigned long long), c->stream));
-    BV_CUDA(cudaFuncSetAttribute(k_trsm, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kTrsmSmem));
-    BV_CUDA(cudaFuncSetAttribute(k_update, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kUpdSmem));
-    FillArgs fa{c->d_locs, use_y ? c->d_y : nullptr, n, c->d, nt, th, A};
-    k_fill<<<(unsigned)ntiles, 256, 0, c->stream>>>(fa);
-    BV_CUDA(cudaGetLastError());
-    for (int64_t k = 0; k < nt; ++k) {
-        k_potrf<<<1, 256, 0, c->stream>>>(A, k, n, fail);
-        const int64_t m = nt - k - 1;
-        if (m > 0) {
-            k_trsm<<<(unsigned)m, 64, kTrsmSmem, c->stream>>>(A, k);
-            k_update<<<(unsigned)(m * (m + 1) / 2), kUpdNT, kUpdSmem, c->stream>>>(A, k);
-        }
+    const cudaStream_t st = c->stream;
+    ExArgs a;
+    a.locs = c->d_locs;
+    a.y = use_y ? c->d_y : nullptr;
+    a.n = n;
+    a.d = c->d;
+    a.T = (int)((n + 16) / 16);
+    a.TC = (int)((n + 15) / 16);
+    a.th = th;
+    a.fixtab = c->d_fixtab;
+    const int64_t ntiles = (int64_t)a.T * (a.T + 1) / 2;
+    // one allocation: tiles | row digits | factors, roots and digits of the diagonal block |
+    // pivots | data row | terms, flags, largest |y|
+    const size_t szA = (size_t)ntiles * kTileB, szD = (size_t)a.T * kP * kDigB, szL = kP * kLdN * sizeof(int4);
+    const size_t szR = kP * 16 * sizeof(FixRs), szE = 6 * kDigB, szN = (size_t)a.TC * 16 * sizeof(int64_t);
+    ExBuf buf(st);
+    BV_CUDA(cudaMallocAsync(&buf.p, szA + szD + szL + szR + szE + 2 * szN + 32, st));
+    unsigned char* q = static_cast<unsigned char*>(buf.p);
+    a.A = reinterpret_cast<longlong2*>(q);
+    a.dig = reinterpret_cast<uint32_t*>(q += szA);
+    a.Ld = reinterpret_cast<int4*>(q += szD);
+    a.rsv = reinterpret_cast<FixRs*>(q += szL);
+    a.ddig = reinterpret_cast<uint32_t*>(q += szR);
+    a.piv = reinterpret_cast<int64_t*>(q += szE);
+    a.zrow = reinterpret_cast<int64_t*>(q += szN);
+    struct {
+        double term[2];
+        int flags;
+        unsigned ymax;
+    } h = {};
+    double* terms = reinterpret_cast<double*>(q += szN);
+    a.flags = reinterpret_cast<int*>(terms + 2);
+    BV_CUDA(cudaMemsetAsync(a.Ld, 0, szL + szR + szE + 2 * szN + 32, st));
+    BV_CUDA(cudaFuncSetAttribute(k_ex_rows, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kRowsSmem));
+    int E = 0;
+    if (use_y) {
+        k_ex_ymax<<<(unsigned)std::min<int64_t>((n + 255) / 256, c->num_sms), 256, 0, st>>>(c->d_y, n, th.diag_rsqrt,
+                                                                                         reinterpret_cast<unsigned*>(a.flags + 1));
+        BV_CUDA(cudaGetLastError());
+        BV_CUDA(cudaMemcpyAsync(&h.ymax, a.flags + 1, sizeof(unsigned), cudaMemcpyDeviceToHost, st));
+        BV_CUDA(cudaStreamSynchronize(st));
+        const int ye = (int)(h.ymax >> 20);
+        E = (ye > 0 ? ye - 1022 : -1021) + kYRoom;
     }
-    BV_CUDA(cudaGetLastError());
-    k_exact_terms<<<1, 256, 0, c->stream>>>(A, n, terms);
-    BV_CUDA(cudaGetLastError());
-    double h[2] = {0.0, 0.0};
-    unsigned long long hf = 0;
-    BV_CUDA(cudaMemcpyAsync(h, terms, sizeof(h), cudaMemcpyDeviceToHost, c->stream));
-    BV_CUDA(cudaMemcpyAsync(&hf, fail, sizeof(hf), cudaMemcpyDeviceToHost, c->stream));
-    BV_CUDA(cudaFreeAsync(A, c->stream));
-    BV_CUDA(cudaFreeAsync(terms, c->stream));
-    BV_CUDA(cudaFreeAsync(fail, c->stream));
-    BV_CUDA(cudaStreamSynchronize(c->stream));
-    if (hf != ~0ull) {
+    const bool valid = th.diag > 0.0 && th.diag < INFINITY && (int)(h.ymax >> 20) != 0x7ff;
+    const int np = (a.TC + kP - 1) / kP, nb = (a.T + kP - 1) / kP;
+    for (int pass = 0; valid; ++pass) {
+        a.E = E;
+        BV_CUDA(cudaMemsetAsync(a.flags, 0, sizeof(int), st));
+        const unsigned fg = (unsigned)((ntiles + 7) / 8);
+        if (th.nu_code == NU_GENERAL) k_ex_fill<true><<<fg, 256, 0, st>>>(a, ntiles);
+        else k_ex_fill<false><<<fg, 256, 0, st>>>(a, ntiles);
+        BV_CUDA(cudaGetLastError());
+        for (int P = 0; P < np; ++P) {
+            k_ex_diag<<<1, 128, 0, st>>>(a, P);
+            const int64_t strips = a.T - (int64_t)kP * (P + 1), m = nb - P - 1;
+            if (strips > 0) {
+                k_ex_rows<<<(unsigned)((strips + 7) / 8), 128, kRowsSmem, st>>>(a, P);
+                k_ex_update<<<(unsigned)(m * (m + 1) / 2), 256, 0, st>>>(a, P);
+            }
+        }
+        BV_CUDA(cudaGetLastError());
+        k_exact_terms<<<1, 256, 0, st>>>(a.piv, a.zrow, n, th.diag * 0x1p-60, ldexp(1.0, E - bvfix::kUnitL), terms);
+        BV_CUDA(cudaGetLastError());
+        BV_CUDA(cudaMemcpyAsync(&h, terms, sizeof(double) * 2 + sizeof(int), cudaMemcpyDeviceToHost, st));
+        BV_CUDA(cudaStreamSynchronize(st));
+        if (!(h.flags & kOver) || (h.flags & kFail) || pass == 12) break;
+        E += kYStep;
+    }
+    if (!valid || h.flags) {
         if (out_loglik) *out_loglik = -INFINITY;
         return BV_ENOTPD;
     }
-    const double logdet = h[0], quad = h[1];
+    const double logdet = h.term[0], quad = h.term[1];
     if (out_logdet) *out_logdet = logdet;
     if (out_quad) *out_quad = quad;
     if (out_loglik) *out_loglik = -0.5 * (quad + logdet + (double)n * 1.8378770664093454835606594728112);

@@ -108,3 +108,19 @@ def test_extreme_scales(bv):
     for s2 in (1e-200, 1e200):
         th = (s2, 0.1, 1.5, 1e-2 * s2)
         _compare(bv, locs, np.sqrt(s2) * z, bp, pi, cen, 45, th)
+
+
+@pytest.mark.parametrize("n", [15, 16, 17, 64, 79, 80, 128, 129, 257, 700])
+def test_exact_tile_edges(bv, n):
+    # the dense factorisation at the edges of its 16-row tiles and 64-column panels, and with a
+    # data row that has to be rescaled (white data: standardised values near 1 / sqrt(tau^2));
+    # tau^2 = 1e-4: pivots within n 2^-53 1e4, 1e-9 of their logarithms' sum
+    locs = synth.locs_uniform(n, 2, 700 + n)
+    y = synth.normal(700 + n, 20, n)
+    for nu in (1.5, 0.8):
+        th = (1.1, 0.3, nu, 1e-4)
+        with bv.Context() as ctx:
+            ctx.set_data(locs, y)
+            ll, quad, ld = ctx.exact_loglik(bv.theta(*th))
+        want = oracle.exact_loglik(oracle.theta(*th), locs, y)
+        assert abs(ll - want) <= 1e-9 * max(1.0, abs(want), quad), (nu, ll, want)
