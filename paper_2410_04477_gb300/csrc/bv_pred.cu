@@ -30,6 +30,7 @@
 #include <vector>
 
 #include "bv_device.cuh"
+#include "bv_fix_tile.cuh"
 #include "bv_internal.h"
 
 struct PredState {
@@ -64,6 +65,8 @@ struct PredState {
     int64_t launch_grid[2] = {0, 0};
     size_t launch_smem = 0;
     int launch_nsm = 0;
+    bool fix = false;             // all blocks go to the fixed-point kernel
+    int64_t max_n = 0;            // its largest padded block, else the largest block
 };
 
 namespace {
@@ -123,6 +126,7 @@ struct PredArgs {
     double* ws;
     int64_t ws_stride;
     int smem_n;            // largest N whose matrix lives in shared memory
+    const uint64_t* fixtab;  // fixed-point exponential tables
     int64_t nblk;
     unsigned long long* fail;
 };
@@ -250,6 +254,127 @@ __global__ void __launch_bounds__(kPredNT) k_pred(PredArgs a) {
                 int r, c;
                 tri_rc(f, r, c);
                 out[f] = failed ? NAN : A[pk(m + r, m + c)];
+            }
+        }
+        if (tid == 0 && failed) atomicMin(a.fail, (unsigned long long)blk);
+        __syncthreads();
+    }
+}
+
+// The same in fixed point (bv_fix_tile.cuh), for blocks whose panel digits fit in shared memory
+// (about 800 points): the m conditioning points are filled up to whole panels with rows of the
+// identity, so that the first panels' elimination leaves the Schur complement in whole tiles.
+// k_pred spends its time on the FP64 pipe (2 lanes a clock and SM); this one uses the integer
+// pipe and the tensor cores: 2,000 blocks of m = 120 and 10 sites in 0.5 ms, before 2.8.  Tiles in a global-memory slot of the CTA.  The mean is left by the
+// elimination at the data row's scale, so a block is done again with a larger one when a solved
+// entry or the sum of their squares (above 16: the mean could leave the range) is too large.
+constexpr int kPredFixNT = 128;
+template <bool GEN>
+__global__ void __launch_bounds__(kPredFixNT, 4) k_pred_fix(PredArgs a) {
+    constexpr int NT = kPredFixNT;
+    extern __shared__ __align__(16) double sm[];
+    __shared__ uint64_t tA[256], tB[256];
+    __shared__ unsigned s_ymax;
+    __shared__ __align__(8) uint64_t s_mb[8];
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const double D = a.th.diag, ratio = a.th.diag_ratio, isd = a.th.diag_rsqrt;
+    const uint64_t rf = (uint64_t)__double2ull_rn(ratio * 0x1p63);
+    for (int j = tid; j < 256; j += NT) {
+        tA[j] = bvfix::mulhi64(a.fixtab[j], rf) << 1;
+        tB[j] = a.fixtab[256 + j];
+    }
+    if (tid < 8)
+        asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"((uint32_t)__cvta_generic_to_shared(s_mb + tid)) : "memory");
+    uint32_t parity = 0;
+    const int d = a.d;
+    longlong2* tiles = reinterpret_cast<longlong2*>(a.ws + (int64_t)blockIdx.x * a.ws_stride);
+    for (int64_t blk = blockIdx.x; blk < a.nblk; blk += gridDim.x) {
+        const int64_t b0 = a.bptr[blk], n0 = a.nptr[blk];
+        const int b = (int)(a.bptr[blk + 1] - b0), m = (int)(a.nptr[blk + 1] - n0), m16 = (m + 15) & ~15;
+        const int N = m16 + b, T = fix_tiles(N), TC = (N + 15) >> 4;
+        uint32_t* dig = reinterpret_cast<uint32_t*>(sm);
+        int4* Ld = reinterpret_cast<int4*>(reinterpret_cast<unsigned char*>(sm) + (size_t)(T - 1) * kDigB);
+        FixRs* rsv = reinterpret_cast<FixRs*>(Ld + 16 * kLd + 16);
+        double* px = reinterpret_cast<double*>(rsv + 16);
+        double* yv = px + d * N;
+        int64_t* yfix = reinterpret_cast<int64_t*>(yv);
+        int64_t* piv = yfix + N;
+        int64_t* zrow = piv + N;
+        if (tid == 0) s_ymax = 0;
+        __syncthreads();
+        for (int j = tid; j < 16 * kLd + 16; j += NT)
+            if (j % kLd >= 16) Ld[j] = make_int4(0, 0, 0, 0);
+        unsigned ym = 0;
+        for (int t = tid; t < N; t += NT) {
+            const bool obs = t < m, pad = !obs && t < m16;
+            const int64_t g = obs ? a.nidx[n0 + t] : pad ? 0 : a.pidx[b0 + (t - m16)];
+            for (int k = 0; k < d; ++k)
+                px[k * N + t] = pad ? 0.0 : (obs ? a.locs[(int64_t)k * a.n_obs + g] : a.plocs[(int64_t)k * a.n_star + g]) * inv_range_k(a.th, k);
+            const double y = obs ? a.y[g] * isd : 0.0;  // data row: [y_NN, 0]
+            yv[t] = y;
+            ym = max(ym, (unsigned)__double2hiint(y) & 0x7fffffffu);
+        }
+        ym = __reduce_max_sync(0xffffffffu, ym);
+        if (lane == 0) atomicMax(&s_ymax, ym);
+        __syncthreads();
+        const int ye = (int)(s_ymax >> 20);
+        int E = (ye > 0 ? ye - 1022 : -1021) + kYRoom;
+        const bool valid = D > 0.0 && D < INFINITY && ye != 0x7ff;
+        bool failed = false;
+        for (int pass = 0;; ++pass) {
+            int flags = valid ? 0 : kFail;
+            for (int t = tid; t < N; t += NT) {
+                const double y = pass == 0 ? yv[t] : ldexp((double)yfix[t], E - kYStep - bvfix::kUnitC);
+                yfix[t] = __double2ll_rn(ldexp(y, bvfix::kUnitC - E));
+            }
+            __syncthreads();
+            for (int q = warp; q < ((T * (T + 1)) >> 1); q += NT / 32) {
+                int I, J;
+                tri_rc(q, I, J);
+                if (J >= TC) continue;
+                fix_fill<GEN ? 2 : 0, true>(tiles + q * 128, I, J, m, m16, N, lane, px, d, yfix, &a.th, a.th.nu_code, ratio,
+                                            nullptr, tA, tB, flags);
+            }
+            int stop = __syncthreads_or(flags);
+            if (!stop) stop = fix_panels<NT>(tiles, T, TC, m16 >> 4, N, dig, Ld, rsv, piv, zrow, s_mb, parity, flags);
+            if (!stop) {
+                if (warp == 0) {
+                    float s = 0.0f;
+                    for (int k = lane; k < m16; k += 32) {
+                        const float z = (float)zrow[k] * 1.734723475976807e-18f;  // 2^-59
+                        s = fmaf(z, z, s);
+                    }
+#pragma unroll
+                    for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+                    if (!(s <= 16.0f)) flags |= kOver;
+                }
+                stop = __syncthreads_or(flags);
+            }
+            failed = stop && __syncthreads_or(flags & kFail);
+            if (failed || !stop) break;
+            if (pass == 12) {
+                failed = true;
+                break;
+            }
+            E += kYStep;
+        }
+        const auto entry = [&](int r, int c) {
+            const longlong2 v = tiles[ftile(r >> 4, c >> 4) * 128 + (((c >> 3) & 1) * 2 + ((r >> 3) & 1)) * 32 + 4 * (r & 7) + ((c & 7) >> 1)];
+            return (c & 1) ? v.y : v.x;
+        };
+        const double vs = D * 0x1p-60, ms = ldexp(sqrt(D), E - bvfix::kUnitC);
+        for (int t = tid; t < b; t += NT) {
+            const int g = a.pidx[b0 + t];
+            a.mean[g] = failed ? NAN : -(double)entry(N, m16 + t) * ms;
+            a.var[g] = failed ? NAN : (double)entry(m16 + t, m16 + t) * vs;
+        }
+        if (a.coff) {
+            double* out = a.cov + a.coff[blk];
+            const int TB = (b * (b + 1)) >> 1;
+            for (int f = tid; f < TB; f += NT) {
+                int r, c;
+                tri_rc(f, r, c);
+                out[f] = failed ? NAN : (double)entry(m16 + r, m16 + c) * vs;
             }
         }
         if (tid == 0 && failed) atomicMin(a.fail, (unsigned long long)blk);
@@ -463,10 +588,20 @@ extern "C" int bv_select_pred_neighbors(bv_ctx* c, int32_t m, int64_t* nn_ptr, i
         BV_TRY(bv_select_pred_neighbors_device(c->d_locs, c->n_tot, d, p->d_cent, p->nblk, p->d_nptr, p->d_nidx, amax,
                                                c->stream));
     BV_CUDA(cudaStreamSynchronize(c->stream));
-    // workspace slots for blocks whose matrix does not fit in shared memory
+    // the fixed-point kernel where the largest block allows it; workspace slots, one per CTA
+    int64_t maxF = 0;
+    for (int64_t i = 0; i < p->nblk; ++i)
+        maxF = std::max(maxF, (mi + 15) / 16 * 16 + p->h_bptr[i + 1] - p->h_bptr[i]);
+    // (without conditioning the covariance is the prior's, to FP64's relative accuracy: k_pred)
+    p->fix = mi > 0 && maxF < 4096 && fix_work_bytes((int)maxF, d) <= (size_t)kFixSmemCap;
+    p->max_n = p->fix ? maxF : maxN;
     int smem_n = 0;
     while (pred_doubles(smem_n + 1) * 8 <= (int64_t)kPredSmemCap) ++smem_n;
-    if (maxN > smem_n) {
+    if (p->fix) {
+        p->ws_slots = (int)std::min<int64_t>(p->nblk, 4 * (int64_t)c->num_sms);
+        p->ws_stride = (int64_t)(fix_tile_bytes((int)maxF) / sizeof(double));
+        BV_CUDA(cudaMalloc(&p->d_ws, sizeof(double) * p->ws_stride * p->ws_slots));
+    } else if (maxN > smem_n) {
         int grid = 0;
         BV_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&grid, k_pred<false>, kPredNT, 0));
         p->ws_slots = std::max(1, std::min<int>(grid * c->num_sms, 2 * c->num_sms));
@@ -496,21 +631,19 @@ extern "C" int bv_get_pred_sizes(bv_ctx* c, int64_t* n_star, int64_t* nblk, int6
 static int pred_launch(bv_ctx* c, const DevTheta& th, bool with_cov) {
     PredState* p = c->pred;
     const bool gen = th.nu_code == NU_GENERAL;
-    auto kern = gen ? k_pred<true> : k_pred<false>;
+    auto kern = p->fix ? (gen ? k_pred_fix<true> : k_pred_fix<false>) : (gen ? k_pred<true> : k_pred<false>);
+    const int nt = p->fix ? kPredFixNT : kPredNT;
     if (p->launch_grid[gen] == 0) {
-        int64_t maxN = 0;
-        for (int64_t i = 0; i < p->nblk; ++i)
-            maxN = std::max(maxN, (p->h_nptr[i + 1] - p->h_nptr[i]) + (p->h_bptr[i + 1] - p->h_bptr[i]));
         int smem_n = 0;
         while (pred_doubles(smem_n + 1) * 8 <= (int64_t)kPredSmemCap) ++smem_n;
-        const int64_t nsm = std::min<int64_t>(maxN, smem_n);
-        const size_t smem = (size_t)pred_doubles(nsm) * 8;
-        BV_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kPredSmemCap));
+        const int64_t nsm = std::min<int64_t>(p->max_n, smem_n);
+        const size_t smem = p->fix ? fix_work_bytes((int)p->max_n, c->d) : (size_t)pred_doubles(nsm) * 8;
+        BV_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, p->fix ? kFixSmemCap : (int)kPredSmemCap));
         int per_sm = 0;
-        BV_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, kPredNT, smem));
+        BV_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, nt, smem));
         int64_t grid = std::max(1, per_sm) * (int64_t)c->num_sms;
         grid = std::min<int64_t>(grid, p->nblk);
-        if (maxN > smem_n) grid = std::min<int64_t>(grid, p->ws_slots);
+        if (p->ws_slots > 0) grid = std::min<int64_t>(grid, p->ws_slots);
         p->launch_grid[gen] = std::max<int64_t>(1, grid);
         p->launch_smem = smem;
         p->launch_nsm = (int)nsm;
@@ -541,7 +674,8 @@ static int pred_launch(bv_ctx* c, const DevTheta& th, bool with_cov) {
     a.nblk = p->nblk;
     a.fail = p->d_fail;
     BV_CUDA(cudaMemsetAsync(p->d_fail, 0xff, sizeof(unsigned long long), c->stream));
-    kern<<<(unsigned)grid, kPredNT, smem, c->stream>>>(a);
+    a.fixtab = c->d_fixtab;
+    kern<<<(unsigned)grid, nt, smem, c->stream>>>(a);
     BV_CUDA(cudaGetLastError());
     return BV_OK;
 }

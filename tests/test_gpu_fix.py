@@ -124,3 +124,25 @@ def test_exact_tile_edges(bv, n):
             ll, quad, ld = ctx.exact_loglik(bv.theta(*th))
         want = oracle.exact_loglik(oracle.theta(*th), locs, y)
         assert abs(ll - want) <= 1e-9 * max(1.0, abs(want), quad), (nu, ll, want)
+
+
+@pytest.mark.parametrize("m", [1, 15, 16, 17, 47, 64, 120, 200])
+@pytest.mark.parametrize("nu", [0.5, 2.5, 0.9])
+def test_prediction_tile_edges(bv, m, nu):
+    # the partial elimination with m below, at and above whole panels of 16; white data under a
+    # smooth covariance, so that the data row is rescaled; tau^2 = 1e-3: errors of about
+    # N 2^-53 1e3 of the prior's scale and of the data's
+    n, ns = 500, 60
+    locs, star = synth.locs_uniform(n, 2, 800), synth.locs_uniform(ns, 2, 801)
+    y = synth.normal(800, 20, n)
+    th = (1.0, 0.25, nu, 1e-3)
+    with bv.Context() as ctx:
+        ctx.set_data(locs, y)
+        ctx.set_pred_locations(star)
+        bp, pi = ctx.build_pred_blocks(6, seed=3)
+        nnp, nni = ctx.select_pred_neighbors(m)
+        mean, var, cov = ctx.predict(bv.theta(*th), packed_cov=True)
+    omean, ovar, ocov = oracle.predict(oracle.theta(*th), locs, y, star, bp, pi, nnp, nni, packed_cov=True)
+    np.testing.assert_allclose(mean, omean, rtol=1e-9, atol=1e-9)
+    np.testing.assert_allclose(var, ovar, rtol=1e-9, atol=1e-11)
+    np.testing.assert_allclose(cov, ocov, rtol=1e-9, atol=1e-11)
