@@ -265,6 +265,158 @@ __global__ void __launch_bounds__(kChunk) k_kpp_pick(const double* __restrict__ 
     if (tid < d) cent_t[tid] = locs[(int64_t)tid * n_tot + off + pick];
 }
 
+// All picks of k-means++ in one launch, for sets that fit one cluster's registers: 8 CTAs of
+// 1,024 threads, P consecutive points a thread, so that the order of (CTA, warp, lane, point)
+// is the points' order.  The two launches a pick above cost their latency whatever the work: at n =
+// 20,000 and k = 2,000 the set-up (K-means, neighbours) took 37.0 ms with them and takes 16.7 ms
+// with this kernel.  Here a pick is two cluster barriers: the CTAs exchange their
+// weight sums; the one that holds the target scans its warps' sums and then that warp's lanes,
+// and writes the new centre into every CTA's shared memory.  Weights are whole numbers, so the
+// sums (kept up to date by differences) do not depend on the order of additions.  A point's
+// exact distance is only computed when its FP32 distance to the new centre is below thr, its
+// current distance and the rounding margin.
+constexpr int kKppCtas = 8, kKppMaxP = 5;
+
+template <int P>
+__global__ void __cluster_dims__(kKppCtas, 1, 1) __launch_bounds__(kChunk, 1)
+    k_kpp_all(const double* __restrict__ locs, int64_t n_tot, int64_t off, int64_t n, int d, int s, float amax, uint64_t stream,
+              int64_t k, double* __restrict__ cent) {
+    __shared__ double s_c[3];                          // the newest centre
+    __shared__ unsigned long long s_sum[kKppCtas];     // weight sums of the CTAs
+    __shared__ unsigned long long s_warp[kChunk / 32], s_tot, s_rem;
+    __shared__ int s_w;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int rank = blockIdx.x;  // one cluster
+    const int64_t i0 = ((int64_t)rank * kChunk + tid) * P;
+    float xf[P][3], thr[P];
+    double D2[P];
+    unsigned long long w[P];
+#pragma unroll
+    for (int p = 0; p < P; ++p) {
+        const bool live = i0 + p < n;
+#pragma unroll
+        for (int q = 0; q < 3; ++q) xf[p][q] = live && q < d ? (float)locs[(int64_t)q * n_tot + off + i0 + p] : 0.0f;
+        thr[p] = live ? INFINITY : -1.0f;
+        D2[p] = INFINITY;
+        w[p] = 0;
+    }
+    if (lane == 0) s_warp[warp] = 0;
+    if (tid == 0) s_tot = 0;
+    if (tid < 3) s_c[tid] = tid < d ? cent[tid] : 0.0;
+    __syncthreads();
+    for (int64_t t = 1; t < k; ++t) {
+        const float c0 = (float)s_c[0], c1 = (float)s_c[1], c2 = (float)s_c[2];
+        unsigned long long dw = 0;  // change of the thread's weight (modulo 2^64)
+#pragma unroll
+        for (int p = 0; p < P; ++p) {
+            const float a0 = xf[p][0] - c0, a1 = xf[p][1] - c1, a2 = xf[p][2] - c2;
+            if (!(fmaf(a2, a2, fmaf(a1, a1, a0 * a0)) > thr[p])) {  // (also when FP32 overflows)
+                double x[3], c[3];
+                for (int q = 0; q < d; ++q) {
+                    x[q] = locs[(int64_t)q * n_tot + off + i0 + p];
+                    c[q] = s_c[q];
+                }
+                const double v = d2_exact(x, c, d);
+                if (v < D2[p]) {
+                    D2[p] = v;
+                    const unsigned long long wn = (unsigned long long)ldexp(v, s);
+                    dw += wn - w[p];
+                    w[p] = wn;
+                    const float vf = __double2float_ru(v);
+                    thr[p] = vf + 2.0f * fp32_margin(vf * 1.001f, amax, d);
+                }
+            }
+        }
+        if (__any_sync(0xffffffffu, dw != 0)) {
+            for (int o = 16; o > 0; o >>= 1) dw += __shfl_xor_sync(0xffffffffu, dw, o);
+            if (lane == 0) {
+                s_warp[warp] += dw;
+                atomicAdd(&s_tot, dw);
+            }
+        }
+        __syncthreads();
+        if (tid < kKppCtas) {  // this CTA's sum into CTA tid's table
+            uint32_t ra;
+            const uint32_t la = (uint32_t)__cvta_generic_to_shared(s_sum + rank);
+            asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(ra) : "r"(la), "r"(tid));
+            asm volatile("st.shared::cluster.u64 [%0], %1;" ::"r"(ra), "l"(s_tot) : "memory");
+        }
+        asm volatile("barrier.cluster.arrive.release.aligned;\nbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+        unsigned long long W = 0;
+#pragma unroll
+        for (int q = 0; q < kKppCtas; ++q) W += s_sum[q];
+        const uint64_t r = bv_sm64(stream, (uint64_t)t);
+        int owner = kKppCtas - 1;
+        unsigned long long target = 0, base = 0;
+        int64_t pick = -1;
+        if (W == 0) {
+            pick = (int64_t)__umul64hi(r, (uint64_t)n);
+            owner = (int)(pick / ((int64_t)kChunk * P));
+        } else {
+            target = __umul64hi(r, W);
+            for (int q = 0; q < kKppCtas; ++q) {  // the first CTA whose inclusive sum exceeds the target
+                if (target < base + s_sum[q]) {
+                    owner = q;
+                    break;
+                }
+                base += s_sum[q];
+            }
+        }
+        if (owner == rank) {
+            if (W != 0) {
+                if (warp == 0) {
+                    const unsigned long long v = s_warp[lane];
+                    unsigned long long inc = v;
+                    for (int o = 1; o < 32; o <<= 1) {
+                        const unsigned long long u = __shfl_up_sync(0xffffffffu, inc, o);
+                        if (lane >= o) inc += u;
+                    }
+                    const unsigned long long rem = target - base;
+                    if (rem < inc && rem >= inc - v) {
+                        s_w = lane;
+                        s_rem = rem - (inc - v);
+                    }
+                }
+                __syncthreads();
+                if (warp == s_w) {
+                    unsigned long long v = 0;
+#pragma unroll
+                    for (int p = 0; p < P; ++p) v += w[p];
+                    unsigned long long inc = v;
+                    for (int o = 1; o < 32; o <<= 1) {
+                        const unsigned long long u = __shfl_up_sync(0xffffffffu, inc, o);
+                        if (lane >= o) inc += u;
+                    }
+                    unsigned long long rem = s_rem;
+                    if (rem < inc && rem >= inc - v) {
+                        rem -= inc - v;
+#pragma unroll
+                        for (int p = 0; p < P; ++p) {
+                            if (pick < 0) {
+                                if (rem < w[p]) pick = i0 + p;
+                                else rem -= w[p];
+                            }
+                        }
+                    }
+                }
+            }
+            if (pick >= 0 && (W != 0 || tid == 0)) {  // one thread
+                for (int q = 0; q < d; ++q) {
+                    const double v = locs[(int64_t)q * n_tot + off + pick];
+                    cent[t * d + q] = v;
+                    const uint32_t la = (uint32_t)__cvta_generic_to_shared(s_c + q);
+                    for (int z = 0; z < kKppCtas; ++z) {
+                        uint32_t ra;
+                        asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(ra) : "r"(la), "r"(z));
+                        asm volatile("st.shared::cluster.f64 [%0], %1;" ::"r"(ra), "d"(v) : "memory");
+                    }
+                }
+            }
+        }
+        asm volatile("barrier.cluster.arrive.release.aligned;\nbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+    }
+}
+
 }  // namespace
 
 static int ceil_log2_u64(uint64_t v) {
@@ -337,10 +489,6 @@ int bv_kmeans_device(const double* d_locs, int64_t n_tot, int64_t off, int64_t n
 
     const uint64_t stream = BV_STREAM_KPP(seed);
     const int64_t nchunks = (n + kChunk - 1) / kChunk;
-    double* D2 = nullptr;
-    unsigned long long* csum = nullptr;
-    BV_CUDA(cudaMallocAsync(&D2, sizeof(double) * n, s));
-    BV_CUDA(cudaMallocAsync(&csum, sizeof(unsigned long long) * nchunks, s));
     // first centre
     {
         const uint64_t r0 = bv_sm64(stream, 0);
@@ -349,16 +497,27 @@ int bv_kmeans_device(const double* d_locs, int64_t n_tot, int64_t off, int64_t n
             BV_CUDA(cudaMemcpyAsync(d_cent + q2, d_locs + (int64_t)q2 * n_tot + off + first, sizeof(double),
                                     cudaMemcpyDeviceToDevice, s));
     }
-    for (int64_t t = 1; t < k; ++t) {
-        k_kpp_update<<<(unsigned)nchunks, kChunk, 0, s>>>(d_locs, n_tot, off, n, d, d_cent + (t - 1) * d,
-                                                          t == 1, sc, D2, csum);
+    const int64_t per = (n + kKppCtas * kChunk - 1) / (kKppCtas * kChunk);  // points a thread of the one-launch form
+    if (per <= kKppMaxP) {
+        auto kern = per == 1 ? k_kpp_all<1> : per == 2 ? k_kpp_all<2> : per == 3 ? k_kpp_all<3> : per == 4 ? k_kpp_all<4> : k_kpp_all<5>;
+        kern<<<kKppCtas, kChunk, 0, s>>>(d_locs, n_tot, off, n, d, sc, (float)amax, stream, k, d_cent);
         BV_CUDA(cudaGetLastError());
-        k_kpp_pick<<<1, kChunk, 0, s>>>(d_locs, n_tot, off, n, d, D2, sc, csum, nchunks, stream, t,
-                                        d_cent + t * d);
-        BV_CUDA(cudaGetLastError());
+    } else {
+        double* D2 = nullptr;
+        unsigned long long* csum = nullptr;
+        BV_CUDA(cudaMallocAsync(&D2, sizeof(double) * n, s));
+        BV_CUDA(cudaMallocAsync(&csum, sizeof(unsigned long long) * nchunks, s));
+        for (int64_t t = 1; t < k; ++t) {
+            k_kpp_update<<<(unsigned)nchunks, kChunk, 0, s>>>(d_locs, n_tot, off, n, d, d_cent + (t - 1) * d,
+                                                              t == 1, sc, D2, csum);
+            BV_CUDA(cudaGetLastError());
+            k_kpp_pick<<<1, kChunk, 0, s>>>(d_locs, n_tot, off, n, d, D2, sc, csum, nchunks, stream, t,
+                                            d_cent + t * d);
+            BV_CUDA(cudaGetLastError());
+        }
+        BV_CUDA(cudaFreeAsync(D2, s));
+        BV_CUDA(cudaFreeAsync(csum, s));
     }
-    BV_CUDA(cudaFreeAsync(D2, s));
-    BV_CUDA(cudaFreeAsync(csum, s));
     // Lloyd
     const unsigned gp = (unsigned)((n + 255) / 256);
     for (int it = 0; it < iters; ++it) {

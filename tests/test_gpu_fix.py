@@ -146,3 +146,17 @@ def test_prediction_tile_edges(bv, m, nu):
     np.testing.assert_allclose(mean, omean, rtol=1e-9, atol=1e-9)
     np.testing.assert_allclose(var, ovar, rtol=1e-9, atol=1e-11)
     np.testing.assert_allclose(cov, ocov, rtol=1e-9, atol=1e-11)
+
+
+@pytest.mark.parametrize("n,k,d", [(8192, 40, 2), (8193, 40, 3), (20000, 64, 1), (40960, 24, 2), (40961, 24, 2), (300, 300, 2)])
+def test_kmeans_seeding_forms(bv, n, k, d):
+    # one to five points a thread of the one-launch seeding, its largest set and the first one
+    # beyond, every point a centre, and repeated points (weights of zero): the oracle's blocks
+    locs = synth.locs_uniform(n, d, 900 + d)
+    locs[n // 2:n // 2 + 40] = locs[:40]
+    with bv.Context() as ctx:
+        ctx.set_data(locs)
+        bp, pi = ctx.build_blocks(k, seed=11, iters=2)
+    obp, opi, _ = oracle.build_blocks(locs, k, seed=11, iters=2)
+    np.testing.assert_array_equal(bp, obp)
+    np.testing.assert_array_equal(pi, opi)
