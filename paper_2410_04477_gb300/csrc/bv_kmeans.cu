@@ -58,43 +58,29 @@ __device__ __forceinline__ float fp32_margin(float v, float amax, int d) {
 
 constexpr int kTile = 256;  // centres per shared-memory tile
 
-// Lloyd assignment.  x: SoA FP64 points [d][n_tot] (this dataset's slice at `off`),
-// cent: row-major FP64 centres [k][d].  One thread per point.
+// Lloyd assignment.  x: SoA FP64 points [d][n_tot] (this dataset's slice at `off`), cent:
+// row-major FP64 centres [k][d].  L lanes a point, each with every L-th centre.  One FP32 pass
+// keeps the smallest two distances and the smallest one's centre: unless the second lies within
+// the rounding margin of the first, that centre is the exact minimiser.  The few points where it
+// does are scored exactly over the centres inside the margin.  (Scoring every point's candidates
+// in a second pass over all centres cost 218 us at n = 20,000, k = 2,000, with one lane a point
+// and half of the SMs without a block.)
+template <int L>
 __global__ void __launch_bounds__(256) k_assign(const double* __restrict__ locs, int64_t n_tot,
                                                 int64_t off, int64_t n, int d,
                                                 const double* __restrict__ cent, int64_t k,
                                                 float amax, int32_t* __restrict__ label) {
     __shared__ float4 cf[kTile];
-    const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+    const int part = threadIdx.x % L;
+    const int64_t i = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) / L;
     const bool live = i < n;
     double x[3] = {0.0, 0.0, 0.0};
-    float xf[3] = {0.f, 0.f, 0.f};
     if (live)
-        for (int q = 0; q < d; ++q) {
-            x[q] = locs[(int64_t)q * n_tot + off + i];
-            xf[q] = (float)x[q];
-        }
-    // pass 1: FP32 minimum
-    float best32 = INFINITY;
-    for (int64_t c0 = 0; c0 < k; c0 += kTile) {
-        const int nt = (int)min((int64_t)kTile, k - c0);
-        __syncthreads();
-        for (int t = threadIdx.x; t < nt; t += blockDim.x) {
-            const double* cc = cent + (c0 + t) * d;
-            cf[t] = make_float4((float)cc[0], d > 1 ? (float)cc[1] : 0.f, d > 2 ? (float)cc[2] : 0.f, 0.f);
-        }
-        __syncthreads();
-        for (int t = 0; t < nt; ++t) {
-            const float4 c = cf[t];
-            const float a0 = xf[0] - c.x, a1 = xf[1] - c.y, a2 = xf[2] - c.z;
-            const float v = fmaf(a2, a2, fmaf(a1, a1, a0 * a0));
-            best32 = fminf(best32, v);
-        }
-    }
-    const float thr = best32 + 2.0f * fp32_margin(best32 * 1.001f, amax, d);
-    // pass 2: exact FP64 score of every centre inside the margin; strict < keeps the
-    // lowest index among equal distances because centres are visited in index order
-    double best = INFINITY;
+#pragma unroll
+        for (int q = 0; q < 3; ++q)
+            if (q < d) x[q] = locs[(int64_t)q * n_tot + off + i];
+    const float xf[3] = {(float)x[0], (float)x[1], (float)x[2]};
+    float best32 = INFINITY, second = INFINITY;
     int32_t bi = 0;
     for (int64_t c0 = 0; c0 < k; c0 += kTile) {
         const int nt = (int)min((int64_t)kTile, k - c0);
@@ -104,20 +90,68 @@ __global__ void __launch_bounds__(256) k_assign(const double* __restrict__ locs,
             cf[t] = make_float4((float)cc[0], d > 1 ? (float)cc[1] : 0.f, d > 2 ? (float)cc[2] : 0.f, 0.f);
         }
         __syncthreads();
-        for (int t = 0; t < nt; ++t) {
+#pragma unroll 4
+        for (int t = part; t < nt; t += L) {
             const float4 c = cf[t];
             const float a0 = xf[0] - c.x, a1 = xf[1] - c.y, a2 = xf[2] - c.z;
             const float v = fmaf(a2, a2, fmaf(a1, a1, a0 * a0));
-            if (v <= thr) {
-                const double e = d2_exact(x, cent + (c0 + t) * d, d);
-                if (e < best) {
-                    best = e;
-                    bi = (int32_t)(c0 + t);
-                }
+            second = fminf(second, fmaxf(v, best32));
+            if (v < best32) {
+                best32 = v;
+                bi = (int32_t)(c0 + t);
             }
         }
     }
-    if (live) label[i] = bi;
+#pragma unroll
+    for (int o = 1; o < L; o <<= 1) {
+        const float ob = __shfl_xor_sync(0xffffffffu, best32, o), os = __shfl_xor_sync(0xffffffffu, second, o);
+        const int32_t oi = __shfl_xor_sync(0xffffffffu, bi, o);
+        second = fminf(fminf(second, os), fmaxf(best32, ob));
+        if (ob < best32) {
+            best32 = ob;
+            bi = oi;
+        }
+    }
+    const float thr = best32 + 2.0f * fp32_margin(best32 * 1.001f, amax, d);
+    const bool close = live && !(second > thr);
+    if (__any_sync(0xffffffffu, close)) {
+        // exact FP64 score of every centre inside the margin; the lowest index among equals
+        double best = INFINITY;
+        int32_t be = 0;
+        if (close) {
+            for (int64_t t = part; t < k; t += L) {
+                const double* cc = cent + t * d;
+                const float a0 = xf[0] - (float)cc[0], a1 = xf[1] - (d > 1 ? (float)cc[1] : 0.f),
+                            a2 = xf[2] - (d > 2 ? (float)cc[2] : 0.f);
+                if (fmaf(a2, a2, fmaf(a1, a1, a0 * a0)) <= thr) {
+                    const double e = d2_exact(x, cc, d);
+                    if (e < best) {
+                        best = e;
+                        be = (int32_t)t;
+                    }
+                }
+            }
+        }
+#pragma unroll
+        for (int o = 1; o < L; o <<= 1) {
+            const double ob = __shfl_xor_sync(0xffffffffu, best, o);
+            const int32_t oi = __shfl_xor_sync(0xffffffffu, be, o);
+            if (ob < best || (ob == best && oi < be)) {
+                best = ob;
+                be = oi;
+            }
+        }
+        if (close) bi = best < INFINITY ? be : 0;
+    }
+    if (live && part == 0) label[i] = bi;
+}
+
+// Four lanes a point until every SM has four warps a scheduler with one (the same labels).
+cudaError_t launch_assign(const double* locs, int64_t n_tot, int64_t off, int64_t n, int d, const double* cent, int64_t k,
+                          float amax, int32_t* label, cudaStream_t s) {
+    if (n < 75000) k_assign<4><<<(unsigned)((4 * n + 255) / 256), 256, 0, s>>>(locs, n_tot, off, n, d, cent, k, amax, label);
+    else k_assign<1><<<(unsigned)((n + 255) / 256), 256, 0, s>>>(locs, n_tot, off, n, d, cent, k, amax, label);
+    return cudaGetLastError();
 }
 
 // Exact integer centroid sums.
@@ -281,6 +315,7 @@ template <int P>
 __global__ void __cluster_dims__(kKppCtas, 1, 1) __launch_bounds__(kChunk, 1)
     k_kpp_all(const double* __restrict__ locs, int64_t n_tot, int64_t off, int64_t n, int d, int s, float amax, uint64_t stream,
               int64_t k, double* __restrict__ cent) {
+    extern __shared__ double s_x[];                    // the CTA's points: coordinate q of point i at q kChunk P + i
     __shared__ double s_c[3];                          // the newest centre
     __shared__ unsigned long long s_sum[kKppCtas];     // weight sums of the CTAs
     __shared__ unsigned long long s_warp[kChunk / 32], s_tot, s_rem;
@@ -295,7 +330,11 @@ __global__ void __cluster_dims__(kKppCtas, 1, 1) __launch_bounds__(kChunk, 1)
     for (int p = 0; p < P; ++p) {
         const bool live = i0 + p < n;
 #pragma unroll
-        for (int q = 0; q < 3; ++q) xf[p][q] = live && q < d ? (float)locs[(int64_t)q * n_tot + off + i0 + p] : 0.0f;
+        for (int q = 0; q < 3; ++q) {
+            const double v = live && q < d ? locs[(int64_t)q * n_tot + off + i0 + p] : 0.0;
+            if (q < d) s_x[(q * kChunk + tid) * P + p] = v;
+            xf[p][q] = (float)v;
+        }
         thr[p] = live ? INFINITY : -1.0f;
         D2[p] = INFINITY;
         w[p] = 0;
@@ -311,12 +350,11 @@ __global__ void __cluster_dims__(kKppCtas, 1, 1) __launch_bounds__(kChunk, 1)
         for (int p = 0; p < P; ++p) {
             const float a0 = xf[p][0] - c0, a1 = xf[p][1] - c1, a2 = xf[p][2] - c2;
             if (!(fmaf(a2, a2, fmaf(a1, a1, a0 * a0)) > thr[p])) {  // (also when FP32 overflows)
-                double x[3], c[3];
+                double v = 0.0;  // d2_exact
                 for (int q = 0; q < d; ++q) {
-                    x[q] = locs[(int64_t)q * n_tot + off + i0 + p];
-                    c[q] = s_c[q];
+                    const double df = __dsub_rn(s_x[(q * kChunk + tid) * P + p], s_c[q]);
+                    v = __dadd_rn(v, __dmul_rn(df, df));
                 }
-                const double v = d2_exact(x, c, d);
                 if (v < D2[p]) {
                     D2[p] = v;
                     const unsigned long long wn = (unsigned long long)ldexp(v, s);
@@ -500,7 +538,9 @@ int bv_kmeans_device(const double* d_locs, int64_t n_tot, int64_t off, int64_t n
     const int64_t per = (n + kKppCtas * kChunk - 1) / (kKppCtas * kChunk);  // points a thread of the one-launch form
     if (per <= kKppMaxP) {
         auto kern = per == 1 ? k_kpp_all<1> : per == 2 ? k_kpp_all<2> : per == 3 ? k_kpp_all<3> : per == 4 ? k_kpp_all<4> : k_kpp_all<5>;
-        kern<<<kKppCtas, kChunk, 0, s>>>(d_locs, n_tot, off, n, d, sc, (float)amax, stream, k, d_cent);
+        const size_t sm = sizeof(double) * kChunk * per * d;
+        BV_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
+        kern<<<kKppCtas, kChunk, sm, s>>>(d_locs, n_tot, off, n, d, sc, (float)amax, stream, k, d_cent);
         BV_CUDA(cudaGetLastError());
     } else {
         double* D2 = nullptr;
@@ -519,13 +559,10 @@ int bv_kmeans_device(const double* d_locs, int64_t n_tot, int64_t off, int64_t n
         BV_CUDA(cudaFreeAsync(csum, s));
     }
     // Lloyd
-    const unsigned gp = (unsigned)((n + 255) / 256);
     for (int it = 0; it < iters; ++it) {
-        k_assign<<<gp, 256, 0, s>>>(d_locs, n_tot, off, n, d, d_cent, k, (float)amax, d_label);
-        BV_CUDA(cudaGetLastError());
+        BV_CUDA(launch_assign(d_locs, n_tot, off, n, d, d_cent, k, (float)amax, d_label, s));
         BV_TRY(bv_centroids_device(d_locs, n_tot, off, n, d, d_label, k, q, d_cent, nullptr, s));
     }
-    k_assign<<<gp, 256, 0, s>>>(d_locs, n_tot, off, n, d, d_cent, k, (float)amax, d_label);
-    BV_CUDA(cudaGetLastError());
+    BV_CUDA(launch_assign(d_locs, n_tot, off, n, d, d_cent, k, (float)amax, d_label, s));
     return BV_OK;
 }
