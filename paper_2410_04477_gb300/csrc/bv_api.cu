@@ -776,7 +776,7 @@ static const int kBinEdges[] = {16, 32, 48, 64, 80, 96, 112, 128, 160, 192, 224,
 // CTA sizes: the mixed kernel's one panel warp plus 2, 4, 8 or 16 update warps.
 static int default_threads(const bv_ctx* c, int kind, int nmax, int nwork) {
     if (kind == 2) return 256;
-    if (kind == 7 || kind == 8) return bv_fix_threads(nmax, nwork, c->num_sms);
+    if (kind >= 7) return bv_fix_threads(nmax, nwork, c->num_sms);
     if (nmax <= 48) return 96;
     if (nmax <= 128) return 160;
     return 288;
@@ -827,9 +827,9 @@ static std::vector<int> fix_edges(int d) {
     return edges;
 }
 
-// Workspace slots of a kind-8 bin, one per CTA of its grid.
+// Workspace slots of a bin of kind 8 or 9, one per CTA of its grid.
 static int alloc_slots(BinPlan& bp) {
-    if (bp.kind != 8) return BV_OK;
+    if (bp.kind < 8) return BV_OK;
     bp.slot_stride = (int64_t)(bv_fix_slot_bytes(bp.nmax) / sizeof(double));
     BV_CUDA(bv_plan_malloc(&bp.d_slots, sizeof(double) * bp.slot_stride * bp.grid));
     return BV_OK;

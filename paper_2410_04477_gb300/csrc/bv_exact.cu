@@ -82,11 +82,14 @@ __global__ void __launch_bounds__(256) k_ex_fill(ExArgs a, int64_t ntiles) {
             }
             const int ex = (int)(bvfix::dbits(acc) >> 52);
             if (ex == 0x7ff) atomicOr(a.flags, kFail);
-            if (GEN) v[e] = bvfix::unit_fix(fmin(matern_gen_corr(a.th, sqrt(acc)), 1.0) * a.th.diag_ratio);
+            if (GEN) v[e] = gen_direct(&a.th, sqrt(acc), a.th.diag_ratio);
             else if (ex == 0) v[e] = (int64_t)(tA[0] >> 2);
-            else if (a.th.nu_code == NU_HALF) v[e] = bvfix::matern_fix<0>(bvfix::dist_fix(bvfix::dbits(acc)), tA, tB);
-            else if (a.th.nu_code == NU_3HALF) v[e] = bvfix::matern_fix<1>(bvfix::dist_fix(bvfix::dbits(acc)), tA, tB);
-            else v[e] = bvfix::matern_fix<2>(bvfix::dist_fix(bvfix::dbits(acc)), tA, tB);
+            else {
+                const Dist x[1] = {bvfix::dist_fix(bvfix::dbits(acc))};
+                int64_t o[1];
+                bvfix::matern_fix<1>(a.th.nu_code == NU_HALF ? 0 : a.th.nu_code == NU_3HALF ? 1 : 2, x, tA, tB, o);
+                v[e] = o[0];
+            }
             if (c >= r || r >= n) v[e] = c == r ? 1ll << bvfix::kUnitC : 0;
             if (r == n && c < n && a.y) v[e] = __double2ll_rn(ldexp(a.y[c] * a.th.diag_rsqrt, bvfix::kUnitC - a.E));
         }

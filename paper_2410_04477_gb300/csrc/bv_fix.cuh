@@ -38,6 +38,12 @@ BV_FIX uint64_t dbits(double x) { uint64_t u; memcpy(&u, &x, 8); return u; }
 BV_FIX double bitsd(uint64_t u) { double x; memcpy(&x, &u, 8); return x; }
 #endif
 
+// v 2^e, |e| <= 2040 (exact unless the result is subnormal); ldexp without its special cases.
+BV_FIX double scale2(double v, int e) {
+    const int a = e / 2;
+    return v * bitsd((uint64_t)(1023 + a) << 52) * bitsd((uint64_t)(1023 + e - a) << 52);
+}
+
 BV_FIX uint32_t hi32(uint64_t a) { return (uint32_t)(a >> 32); }
 BV_FIX uint32_t lo32(uint64_t a) { return (uint32_t)a; }
 
@@ -188,24 +194,47 @@ BV_FIX Exp exp2_fix(uint64_t zf, const TA* A, const TB* B) {
     return o;
 }
 
-// w rho(x) in matrix units for the closed forms: NU = 0 (1/2), 1 (3/2) or 2 (5/2).  x >= 64
-// gives 0 (rho below 2^-80).  No branches: a caller's entries are independent chains that the
-// compiler can interleave.
-template <int NU, typename TA, typename TB>
-BV_FIX int64_t matern_fix(Dist x, const TA* A, const TB* B) {
-    const uint64_t Z = mulhi63(x.X, 0x5C551D94AE0BF85Eull);        // log2 e in units 2^-62
-    const int q = x.q > 6 ? 6 : x.q < -55 ? -55 : x.q, sh = 6 - q;
-    const Exp e = exp2_fix(((Z << 2) + ((1ull << sh) >> 1)) >> sh, A, B);
-    uint64_t v = shr(e.W, e.i);
-    if (NU > 0) {
-        const uint64_t H = mulhi63(x.X, e.W);                      // units 2^(q - 60)
-        v += shr(H << 1, e.i - q);
-        if (NU > 1) {
-            const uint64_t H2 = mulhi63(x.X, mulhi63(H, 0x5555555555555555ull));  // units 2^(2 q - 59)
-            v += shr(H2 << 6, e.i - 2 * q + 4);
+// w rho(x) in matrix units for the closed forms: nu = 0 (1/2), 1 (3/2) or 2 (5/2), for K scaled
+// distances at once (independent chains that the compiler interleaves; one copy of the code for
+// all nu, which branch on it only for the polynomial).  x >= 64 gives 0 (rho below 2^-80).
+template <int K, typename TA, typename TB>
+BV_FIX void matern_fix(int nu, const Dist (&x)[K], const TA* A, const TB* B, int64_t (&out)[K]) {
+    Exp e[K];
+    uint64_t v[K];
+    int q[K];
+#ifdef __CUDACC__
+#pragma unroll
+#endif
+    for (int k = 0; k < K; ++k) {
+        const uint64_t Z = mulhi63(x[k].X, 0x5C551D94AE0BF85Eull);  // log2 e in units 2^-62
+        q[k] = x[k].q > 6 ? 6 : x[k].q < -55 ? -55 : x[k].q;
+        const int sh = 6 - q[k];
+        e[k] = exp2_fix(((Z << 2) + ((1ull << sh) >> 1)) >> sh, A, B);
+        v[k] = shr(e[k].W, e[k].i);
+    }
+    if (nu > 0) {
+        uint64_t H[K];
+#ifdef __CUDACC__
+#pragma unroll
+#endif
+        for (int k = 0; k < K; ++k) {
+            H[k] = mulhi63(x[k].X, e[k].W);                         // units 2^(q - 60)
+            v[k] += shr(H[k] << 1, e[k].i - q[k]);
+        }
+        if (nu > 1) {
+#ifdef __CUDACC__
+#pragma unroll
+#endif
+            for (int k = 0; k < K; ++k) {
+                const uint64_t H2 = mulhi63(x[k].X, mulhi63(H[k], 0x5555555555555555ull));  // units 2^(2 q - 59)
+                v[k] += shr(H2 << 6, e[k].i - 2 * q[k] + 4);
+            }
         }
     }
-    return x.q > 6 ? 0 : (int64_t)((v + 1) >> 1);
+#ifdef __CUDACC__
+#pragma unroll
+#endif
+    for (int k = 0; k < K; ++k) out[k] = x[k].q > 6 ? 0 : (int64_t)((v[k] + 1) >> 1);
 }
 
 // The general smoothness: rho = e^-(x - L(x)), L a polynomial of degree DEG - 1 in t = 2 m - 3

@@ -45,12 +45,15 @@
 
 namespace {
 
-constexpr int kFixWarps = 16;       // resident warps an SM that the register budget allows
 
 // GLOB: the tiles live in a global-memory slot of the CTA (they stay in L2), for blocks whose
 // triangle does not leave room in shared memory.
-template <int NT, bool GEN, bool GLOB>
-__global__ void __launch_bounds__(NT, kFixWarps * 32 / NT) k_ll_fix(LLArgs a) {
+// WARPS: resident warps an SM that the registers leave room for: 20 (96 registers) up to N = 111,
+// where more blocks an SM hide the pivots' chains (n = 200,000, m = 60: 2.40 ms, with 16 2.50),
+// 16 (128 registers) beyond, where spills cost more (3D, m = 200: 10.2 ms, with 16 9.34); 24
+// lose in both (2.58, 10.8).
+template <int NT, bool GEN, bool GLOB, int WARPS>
+__global__ void __launch_bounds__(NT, WARPS * 32 / NT) k_ll_fix(LLArgs a) {
     extern __shared__ __align__(16) unsigned char smraw[];
     __shared__ uint64_t tA[256], tB[256];
     __shared__ int s_w;
@@ -58,6 +61,7 @@ __global__ void __launch_bounds__(NT, kFixWarps * 32 / NT) k_ll_fix(LLArgs a) {
     __shared__ __align__(8) uint64_t s_mb[8];
     constexpr int NW = NT / 32;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+#pragma unroll 1
     for (int j = tid; j < 256; j += NT) tB[j] = a.fixtab[256 + j];
     const int nwork = work_count(a);
     if (tid < 8)
@@ -66,6 +70,7 @@ __global__ void __launch_bounds__(NT, kFixWarps * 32 / NT) k_ll_fix(LLArgs a) {
     if (tid == 0) s_w = take_work(a.ctr, blockIdx.x);
     __syncthreads();
     int dsprev = -1;
+#pragma unroll 1
     for (int w = s_w; w < nwork; w = s_w) {
         const int nx = tid == 0 ? take_work(a.ctr, w + gridDim.x) : 0;
         const int blk = a.work[w];
@@ -89,16 +94,20 @@ __global__ void __launch_bounds__(NT, kFixWarps * 32 / NT) k_ll_fix(LLArgs a) {
         const double D = th.diag, ratio = th.diag_ratio, isd = th.diag_rsqrt;
         if (ds != dsprev) {  // A[j] = 2^(-j/256) sigma^2 / D
             const uint64_t rf = (uint64_t)__double2ull_rn(ratio * 0x1p63);
+#pragma unroll 1
             for (int j = tid; j < 256; j += NT) tA[j] = bvfix::mulhi64(a.fixtab[j], rf) << 1;
             dsprev = ds;
         }
         if (tid == 0) s_ymax = 0;
+#pragma unroll 1
         for (int j = tid; j < 16 * kLd + 16; j += NT)
             if (j % kLd >= 16) Ld[j] = make_int4(0, 0, 0, 0);
         __syncthreads();
         unsigned ym = 0;
+#pragma unroll 1
         for (int t = tid; t < N; t += NT) {
             const int g = t < m ? a.nidx[n0 + t] : a.pidx[b0 + (t - m)];
+#pragma unroll 1
             for (int k = 0; k < d; ++k) px[k * N + t] = a.locs[(int64_t)k * a.n_tot + g] * inv_range_k(th, k);
             const double y = a.y[g] * isd;
             yv[t] = y;  // (in place of its fixed-point value until the scale is known)
@@ -115,14 +124,17 @@ __global__ void __launch_bounds__(NT, kFixWarps * 32 / NT) k_ll_fix(LLArgs a) {
         int64_t* yfix = reinterpret_cast<int64_t*>(yv);
         // again with a larger E when a solved data entry leaves the range (a finite z needs a
         // few passes at most; the data row is 0 after 9)
+#pragma unroll 1
         for (int pass = 0;; ++pass) {
             int flags = valid ? 0 : kFail;
+#pragma unroll 1
             for (int t = tid; t < N; t += NT) {
-                const double y = pass == 0 ? yv[t] : ldexp((double)yfix[t], E - kYStep - bvfix::kUnitC);
-                yfix[t] = __double2ll_rn(ldexp(y, bvfix::kUnitC - E));
+                const double y = pass == 0 ? yv[t] : bvfix::scale2((double)yfix[t], E - kYStep - bvfix::kUnitC);
+                yfix[t] = __double2ll_rn(bvfix::scale2(y, bvfix::kUnitC - E));
             }
             __syncthreads();
             const int ntile = (T * (T + 1)) >> 1;
+#pragma unroll 1
             for (int q = warp; q < ntile; q += NW) {
                 int I, J;
                 tri_rc(q, I, J);
@@ -142,7 +154,7 @@ __global__ void __launch_bounds__(NT, kFixWarps * 32 / NT) k_ll_fix(LLArgs a) {
         }
 
         if (warp == 0) {
-            const double zs = ldexp(1.0, E - bvfix::kUnitL), ps = D * 0x1p-60;
+            const double zs = bvfix::scale2(1.0, E - bvfix::kUnitL), ps = D * 0x1p-60;
             const double2 s2 = warp_terms(m, N, lane, [&](int k) { return fail ? 0.0 : (double)zrow[k] * zs; },
                                           [&](int k) { return fail ? 0.0 : log((double)piv[k] * ps); });
             if (lane == 0) {
@@ -160,43 +172,18 @@ __global__ void __launch_bounds__(NT, kFixWarps * 32 / NT) k_ll_fix(LLArgs a) {
     }
 }
 
-template <int NT, bool GEN, bool GLOB>
-cudaError_t fix_attr() {
-    return cudaFuncSetAttribute(k_ll_fix<NT, GEN, GLOB>, cudaFuncAttributeMaxDynamicSharedMemorySize, kFixSmemCap);
+// The instantiation of a kind, CTA size and smoothness.
+using FixKernel = void (*)(LLArgs);
+template <bool GEN>
+FixKernel fix_kernel_g(int kind, int threads) {
+    if (threads == 256) return kind == 7 ? k_ll_fix<256, GEN, false, 16> : k_ll_fix<256, GEN, true, 16>;
+    if (kind == 7) return threads == 64 ? k_ll_fix<64, GEN, false, 20> : nullptr;
+    if (threads != 128) return nullptr;
+    return kind == 8 ? k_ll_fix<128, GEN, true, 20> : k_ll_fix<128, GEN, true, 16>;
 }
-
-template <int NT>
-cudaError_t fix_go(int grid, size_t smem, bool glob, const LLArgs& a, cudaStream_t s) {
-    cudaError_t e;
-#define BV_GO(GEN, GLOB)                                         \
-    {                                                            \
-        e = fix_attr<NT, GEN, GLOB>();                           \
-        if (e != cudaSuccess) return e;                          \
-        k_ll_fix<NT, GEN, GLOB><<<grid, NT, smem, s>>>(a);       \
-    }
-    if (a.gen) {
-        if (glob) BV_GO(true, true) else BV_GO(true, false)
-    } else {
-        if (glob) BV_GO(false, true) else BV_GO(false, false)
-    }
-#undef BV_GO
-    return cudaGetLastError();
-}
-
-template <int NT>
-int fix_occ(size_t smem, bool glob) {
-    int n1 = 0, n2 = 0;
-    cudaError_t e = glob ? fix_attr<NT, false, true>() : fix_attr<NT, false, false>();
-    if (e == cudaSuccess) e = glob ? fix_attr<NT, true, true>() : fix_attr<NT, true, false>();
-    if (e != cudaSuccess) return 0;
-    if (glob) {
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n1, k_ll_fix<NT, false, true>, NT, smem);
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n2, k_ll_fix<NT, true, true>, NT, smem);
-    } else {
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n1, k_ll_fix<NT, false, false>, NT, smem);
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n2, k_ll_fix<NT, true, false>, NT, smem);
-    }
-    return n1 > n2 ? n1 : n2;
+cudaError_t fix_kernel(int kind, int threads, bool gen, FixKernel* k) {
+    *k = gen ? fix_kernel_g<true>(kind, threads) : fix_kernel_g<false>(kind, threads);
+    return *k ? cudaFuncSetAttribute(*k, cudaFuncAttributeMaxDynamicSharedMemorySize, kFixSmemCap) : cudaErrorInvalidValue;
 }
 
 }  // namespace
@@ -211,15 +198,16 @@ int bv_fix_threads(int nmax, int nwork, int num_sms) {
 }
 
 size_t bv_fix_smem_bytes(int kind, int nmax, int d) {
-    return fix_work_bytes(nmax, d) + (kind == 8 ? 0 : fix_tile_bytes(nmax));
+    return fix_work_bytes(nmax, d) + (kind == 7 ? fix_tile_bytes(nmax) : 0);
 }
 
 // The kernel form of a bin of largest size nmax: tiles in shared memory (7) up to three tile
-// rows, in a workspace (8) beyond, where four to eight CTAs an SM would not fit with them; -1
-// when even the panel's digits do not fit.
+// rows, in a workspace beyond, where four to eight CTAs an SM would not fit with them (8; 9 from
+// N = 112 on, with more registers); -1 when even the panel's digits do not fit.
 int bv_fix_kind(int nmax, int d) {
     if (fix_tiles(nmax) <= 3) return 7;
-    return bv_fix_smem_bytes(8, nmax, d) <= (size_t)kFixSmemCap ? 8 : -1;
+    if (bv_fix_smem_bytes(8, nmax, d) > (size_t)kFixSmemCap) return -1;
+    return nmax <= 111 ? 8 : 9;
 }
 int bv_fix_max_n(int d) {
     int n = 64;
@@ -229,21 +217,21 @@ int bv_fix_max_n(int d) {
 size_t bv_fix_slot_bytes(int nmax) { return fix_tile_bytes(nmax); }
 
 int bv_fix_occupancy(int kind, int threads, size_t smem) {
-    switch (threads) {
-        case 64: return fix_occ<64>(smem, kind == 8);
-        case 128: return fix_occ<128>(smem, kind == 8);
-        case 256: return fix_occ<256>(smem, kind == 8);
-        default: return 0;
+    int n[2] = {0, 0};
+    for (int gen = 0; gen < 2; ++gen) {
+        FixKernel k;
+        if (fix_kernel(kind, threads, gen, &k) != cudaSuccess) return 0;
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n[gen], k, threads, smem);
     }
+    return n[0] > n[1] ? n[0] : n[1];
 }
 
 cudaError_t bv_fix_launch(int kind, int threads, int grid, size_t smem, const LLArgs& a, cudaStream_t s) {
-    switch (threads) {
-        case 64: return fix_go<64>(grid, smem, kind == 8, a, s);
-        case 128: return fix_go<128>(grid, smem, kind == 8, a, s);
-        case 256: return fix_go<256>(grid, smem, kind == 8, a, s);
-        default: return cudaErrorInvalidValue;
-    }
+    FixKernel k;
+    const cudaError_t e = fix_kernel(kind, threads, a.gen, &k);
+    if (e != cudaSuccess) return e;
+    k<<<grid, threads, smem, s>>>(a);
+    return cudaGetLastError();
 }
 
 // The exponential's tables (bv_fix.cuh): 2^(-j/256) in units 2^-62, then 2^(-j/65536) in units

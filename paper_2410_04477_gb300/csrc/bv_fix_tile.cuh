@@ -340,6 +340,11 @@ __device__ __forceinline__ void fix_update(longlong2* C, const uint32_t* dI, con
     }
 }
 
+// The general smoothness through K_nu, in matrix units (not inlined: it is as long as all the rest).
+__device__ __noinline__ int64_t gen_direct(const DevTheta* th, double x, double ratio) {
+    return bvfix::unit_fix(fmin(matern_gen_corr(*th, x), 1.0) * ratio);
+}
+
 // One covariance tile (I, J), one warp, entries in matrix units: rows and columns of the points
 // at px (pre-scaled coordinates, dimension k at k np), row N the data row yfix.  GEN = 0: the
 // closed forms; 1: those and the general smoothness through its table gt; 2: the general
@@ -354,6 +359,7 @@ __device__ __forceinline__ void fix_fill(longlong2* tp, int I, int J, int m, int
         const int c0 = 16 * J + 8 * h + 2 * t, r0 = 16 * I + g;
         const int ra = min(r0, N - 1), rb = min(r0 + 8, N - 1), ca = min(c0, N - 1), cb = min(c0 + 1, N - 1);
         double acc[4] = {0.0, 0.0, 0.0, 0.0};
+#pragma unroll 1
         for (int k = 0; k < d; ++k) {
             const double* pk1 = px + k * N;
             const double xa = pk1[ra], xb = pk1[rb], ya = pk1[ca], yb = pk1[cb];
@@ -369,29 +375,23 @@ __device__ __forceinline__ void fix_fill(longlong2* tp, int I, int J, int m, int
                 const double ac = e == 0 ? acc[0] : e == 1 ? acc[1] : e == 2 ? acc[2] : acc[3];
                 int64_t w;
                 if (GEN == 2) {
-                    w = bvfix::unit_fix(fmin(matern_gen_corr(*th, dist_of(ac)), 1.0) * ratio);
+                    w = gen_direct(th, dist_of(ac), ratio);
                 } else {
                     const Dist x = bvfix::dist_fix(bvfix::dbits(ac));
                     w = bvfix::matern_gen_fix<GTAB_DEG, -GTAB_E0>(x, gt, tA, tB);
-                    if (x.q < 1 + GTAB_E0 && x.q > -500) {  // nearer than the table: K_nu itself
-                        const double xd = ldexp((double)x.X, x.q - 63);
-                        w = bvfix::unit_fix(fmin(matern_gen_corr(*th, xd), 1.0) * ratio);
-                    }
+                    if (x.q < 1 + GTAB_E0 && x.q > -500)  // nearer than the table: K_nu itself
+                        w = gen_direct(th, bvfix::scale2((double)x.X, x.q - 63), ratio);
                 }
                 if (e == 0) v[0] = w;
                 else if (e == 1) v[1] = w;
                 else if (e == 2) v[2] = w;
                 else v[3] = w;
             }
-        } else if (nu_code == NU_HALF) {
-#pragma unroll
-            for (int e = 0; e < 4; ++e) v[e] = bvfix::matern_fix<0>(bvfix::dist_fix(bvfix::dbits(acc[e])), tA, tB);
-        } else if (nu_code == NU_3HALF) {
-#pragma unroll
-            for (int e = 0; e < 4; ++e) v[e] = bvfix::matern_fix<1>(bvfix::dist_fix(bvfix::dbits(acc[e])), tA, tB);
         } else {
+            Dist x[4];
 #pragma unroll
-            for (int e = 0; e < 4; ++e) v[e] = bvfix::matern_fix<2>(bvfix::dist_fix(bvfix::dbits(acc[e])), tA, tB);
+            for (int e = 0; e < 4; ++e) x[e] = bvfix::dist_fix(bvfix::dbits(acc[e]));
+            bvfix::matern_fix<4>(nu_code == NU_HALF ? 0 : nu_code == NU_3HALF ? 1 : 2, x, tA, tB, v);
         }
 #pragma unroll
         for (int e = 0; e < 4; ++e) {
@@ -417,11 +417,13 @@ template <int NT>
 __device__ __forceinline__ int fix_panels(longlong2* tiles, int T, int TC, int NP, int N, uint32_t* dig, int4* Ld, FixRs* rsv,
                                           int64_t* piv, int64_t* zrow, uint64_t* mb, uint32_t& parity, int& flags) {
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+#pragma unroll 1
     for (int p = 0; p < NP; ++p) {
         const int k0 = p << 4, nc = min(16, N - k0), rows = (T - p - 1) << 4;
         if (warp == 0) {
             fix_diag(tiles + ftile(p, p) * 128, nc, k0, N, lane, Ld, rsv, piv, zrow, mb, flags);
         } else {
+#pragma unroll 1
             for (int rw = tid - 32; rw < rows; rw += NT - 32) {
                 const int I = p + 1 + (rw >> 4);
                 fix_row(tiles + ftile(I, p) * 128, Ld, rsv, rw & 15, (I << 4) + (rw & 15) == N, zrow + k0, nc, rw < NT - 32, mb,
@@ -431,6 +433,7 @@ __device__ __forceinline__ int fix_panels(longlong2* tiles, int T, int TC, int N
         parity ^= 1;
         if (__syncthreads_or(flags)) return 1;
         const int S = T - p - 1, cnt = (S * (S + 1)) >> 1;
+#pragma unroll 1
         for (int q = warp; q < cnt; q += NT / 32) {
             int ii, jj;
             tri_rc(q, ii, jj);

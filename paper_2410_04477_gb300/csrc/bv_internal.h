@@ -132,7 +132,8 @@ struct LLArgs {
 struct BinPlan {
     int kind;            // 1: mixed (CTA per block), 2: large (global), 3: mixed (warp per
                          // block), 5: mixed with tensor-core updates (CTA per block),
-                         // 7: FP64 in fixed point, 8: the same with its tiles in d_slots
+                         // 7: FP64 in fixed point, 8, 9: the same with its tiles in d_slots
+                         // (N <= 111, larger)
     int nmax;            // largest augmented size N = m + b in the bin
     int threads;         // CTA size (autotuned)
     int grid;            // CTAs launched
@@ -140,7 +141,7 @@ struct BinPlan {
     int32_t* d_work;     // device block ids (largest N first)
     int32_t nwork;
     int* d_ctr;          // this bin's work counter (a slot of the context's counter array)
-    double* d_slots = nullptr;  // kind 8: one workspace slot of slot_stride doubles per CTA
+    double* d_slots = nullptr;  // kinds 8, 9: one workspace slot of slot_stride doubles per CTA
     int64_t slot_stride = 0;
     int slot = -1;       // mixed check's redo launches: index of the bin's device count
     std::vector<int32_t> h_work;
@@ -151,7 +152,7 @@ size_t bv_tc_smem_bytes(int nmax);
 int bv_tc_occupancy(int threads, size_t smem);
 cudaError_t bv_tc_launch(int threads, int grid, size_t smem, const LLArgs& a, cudaStream_t s);
 
-// FP64 kernel in fixed point with tensor-core updates (bv_fix_ll.cu), kinds 7 and 8.
+// FP64 kernel in fixed point with tensor-core updates (bv_fix_ll.cu), kinds 7 to 9.
 int bv_fix_kind(int nmax, int d);
 int bv_fix_max_n(int d);
 int bv_fix_threads(int nmax, int nwork, int num_sms);

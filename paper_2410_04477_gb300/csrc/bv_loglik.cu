@@ -798,7 +798,7 @@ cudaError_t launch_kind(int kind, int grid, size_t smem, const LLArgs& a, cudaSt
 size_t bv_smem_bytes(int kind, int nmax, int d, int threads) {
     if (kind == 2) return 0;
     if (kind == 5) return bv_tc_smem_bytes(nmax);
-    if (kind == 7 || kind == 8) return bv_fix_smem_bytes(kind, nmax, d);
+    if (kind >= 7) return bv_fix_smem_bytes(kind, nmax, d);
     return sizeof(float) * (size_t)mixed_floats(nmax) * (size_t)(kind == 3 ? threads / 32 : 1);
 }
 
@@ -818,7 +818,7 @@ cudaError_t bv_launch_bin(const BinPlan& bp, const LLArgs& a0, cudaStream_t s) {
     a.nwork = bp.nwork;
     a.ctr = bp.d_ctr;
     if (bp.kind == 5) return bv_tc_launch(bp.threads, bp.grid, bp.smem, a, s);
-    if (bp.kind == 7 || bp.kind == 8) {
+    if (bp.kind >= 7) {
         a.ws = bp.d_slots;
         a.ws_stride = bp.slot_stride;
         return bv_fix_launch(bp.kind, bp.threads, bp.grid, bp.smem, a, s);
@@ -895,7 +895,7 @@ cudaError_t bv_launch_eval_reset(unsigned long long* fail, int* ctr, int n, cuda
 // Occupancy helper for the planner.
 int bv_occupancy(int kind, int threads, size_t smem) {
     if (kind == 5) return bv_tc_occupancy(threads, smem);
-    if (kind == 7 || kind == 8) return bv_fix_occupancy(kind, threads, smem);
+    if (kind >= 7) return bv_fix_occupancy(kind, threads, smem);
     int nb = 0;
     cudaError_t e = cudaSuccess;
 #define BV_OCC(NT)                                                                            \

@@ -265,7 +265,8 @@ __global__ void __launch_bounds__(kPredNT) k_pred(PredArgs a) {
 // (about 800 points): the m conditioning points are filled up to whole panels with rows of the
 // identity, so that the first panels' elimination leaves the Schur complement in whole tiles.
 // k_pred spends its time on the FP64 pipe (2 lanes a clock and SM); this one uses the integer
-// pipe and the tensor cores: 2,000 blocks of m = 120 and 10 sites in 0.5 ms, before 2.8.  Tiles in a global-memory slot of the CTA.  The mean is left by the
+// pipe and the tensor cores: 2,000 blocks of m = 120 and 10 sites in
+// 0.79 ms, before 2.8.  Tiles in a global-memory slot of the CTA.  The mean is left by the
 // elimination at the data row's scale, so a block is done again with a larger one when a solved
 // entry or the sum of their squares (above 16: the mean could leave the range) is too large.
 constexpr int kPredFixNT = 128;
@@ -324,8 +325,8 @@ __global__ void __launch_bounds__(kPredFixNT, 4) k_pred_fix(PredArgs a) {
         for (int pass = 0;; ++pass) {
             int flags = valid ? 0 : kFail;
             for (int t = tid; t < N; t += NT) {
-                const double y = pass == 0 ? yv[t] : ldexp((double)yfix[t], E - kYStep - bvfix::kUnitC);
-                yfix[t] = __double2ll_rn(ldexp(y, bvfix::kUnitC - E));
+                const double y = pass == 0 ? yv[t] : bvfix::scale2((double)yfix[t], E - kYStep - bvfix::kUnitC);
+                yfix[t] = __double2ll_rn(bvfix::scale2(y, bvfix::kUnitC - E));
             }
             __syncthreads();
             for (int q = warp; q < ((T * (T + 1)) >> 1); q += NT / 32) {

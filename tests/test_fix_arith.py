@@ -42,8 +42,12 @@ int main() {
         const Dist d = dist_fix(dbits(acc));
         const L xt = sqrtl((L)acc), xv = ldexpl((L)d.X, d.q - 63);
         ed = fmaxl(ed, fabsl(xv / xt - 1));
-        const int64_t v[3] = {matern_fix<0>(d, A, B), matern_fix<1>(d, A, B), matern_fix<2>(d, A, B)};
-        for (int n = 0; n < 3; ++n) ec[n] = fmaxl(ec[n], fabsl((L)v[n] * 0x1p-60L - corr(n, xt)));
+        for (int n = 0; n < 3; ++n) {
+            const Dist dd[1] = {d};
+            int64_t v[1];
+            matern_fix<1>(n, dd, A, B, v);
+            ec[n] = fmaxl(ec[n], fabsl((L)v[0] * 0x1p-60L - corr(n, xt)));
+        }
     }
     printf("%Lg %Lg %Lg %Lg %Lg\n", er, ed, ec[0], ec[1], ec[2]);
     if (unit_fix(1.0) != 1ll << 60 || unit_fix(0.0) != 0) return 2;
