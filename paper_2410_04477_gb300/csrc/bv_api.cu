@@ -270,6 +270,15 @@ extern "C" int bv_create(bv_ctx** out, int device, void* stream) {
         }();
         e = cudaMemcpy(c->d_fixtab, tab.data(), sizeof(uint64_t) * 512, cudaMemcpyHostToDevice);
     }
+    if (e == cudaSuccess) e = cudaMalloc(&c->d_simtab, bv_sim_table_bytes());
+    if (e == cudaSuccess) {
+        static const std::vector<unsigned char> tab = [] {
+            std::vector<unsigned char> t(bv_sim_table_bytes());
+            bv_sim_table(t.data());
+            return t;
+        }();
+        e = cudaMemcpy(c->d_simtab, tab.data(), tab.size(), cudaMemcpyHostToDevice);
+    }
     if (e != cudaSuccess) {
         bv_record_cuda_error(e, "bv_create", __FILE__, __LINE__);
         bv_destroy(c);
@@ -289,6 +298,7 @@ extern "C" void bv_destroy(bv_ctx* c) {
     dfree(c->d_fail);
     dfree(c->d_wctr);
     dfree(c->d_fixtab);
+    dfree(c->d_simtab);
     dfree(c->d_ws);
     for (auto s : c->side) cudaStreamDestroy(s);
     for (auto e : c->side_ev) cudaEventDestroy(e);

@@ -270,4 +270,74 @@ BV_FIX int64_t unit_fix(double v) {
     return (int64_t)(((b & 0x000FFFFFFFFFFFFFull) | 0x0010000000000000ull) << 8 >> (-k));
 }
 
+// High 64 bits of the signed product a b, up to a unit off (the low x low product is left out);
+// |a|, |b| < 2^63 - 2^31.
+BV_FIX int64_t mulh(int64_t a, int64_t b) {
+    const Bal x = bal(a), y = bal(b);
+    return smad(x.h, y.h, smad(x.h, y.l, smad(x.l, y.h, 0)) >> 32);
+}
+
+// Tables of the Box-Muller pairs: c[j] 2^-15 ~ 1 / (1 + (j + 1/2) / 256) (1 for j = 0, 1/2 for
+// j = 255), with -ln of it -- of its double where j >= kLnHalf -- in units 2^-60, and cosine and
+// sine of (pi / 2) (j + 1/2) / 256 in units 2^-62.
+constexpr int kLnHalf = 106;  // 1 + 106/256: about sqrt(2)
+struct SimTab {
+    uint16_t c[256];
+    int64_t ln[256];
+    int64_t cs[256], sn[256];
+};
+
+// One pair: two uniforms u1 = 1 - k1 2^-53, u2 = k2 2^-53 give rho = sqrt(-2 ln u1) and the
+// angle 2 pi u2.  V = rho^2 in units 2^-56, rho = X 2^(q - 63) (X = 0 for u1 = 1), cs and sn in
+// units 2^-62; all within a few 2^-57.
+struct Pair {
+    uint64_t V, X;
+    int q;
+    int64_t cs, sn;
+};
+BV_FIX Pair pair_fix(uint64_t k1, uint64_t k2, const SimTab& T) {
+    Pair o;
+    {   // -ln u1 = -e ln 2 - ln c^-1 - ln(1 + r), u1 = m 2^e, r = m c - 1, |r| < 2^-7.9
+        const uint64_t U = (1ull << 53) - k1;
+        const int lz = clz64(U);
+        const uint64_t M = U << lz;                      // m 2^63
+        const int j = (int)(M >> 55) & 255;
+        const uint32_t c = T.c[j];
+        const int64_t hi = (int64_t)umad(hi32(M), c, 0) - (1ll << 46);  // (m c - 1) 2^46, top part
+        const int64_t R = (int64_t)((uint64_t)hi << 24) + (int64_t)(umad(lo32(M), c, 0) >> 8);  // r, units 2^-70
+        const float r = (float)(int32_t)(R >> 32) * 3.637978807091713e-12f;     // units 2^-38
+        const float g = fmaf(r, fmaf(r, fmaf(r, -1.0f / 7.0f, 1.0f / 6.0f), -0.2f), 0.25f);
+        const int64_t t1 = 0x1555555555555555ll - ((int64_t)f2i(r * g * 1099511627776.0f) << 22);  // 1/3 - r g, units 2^-62
+        const int64_t t2 = (1ll << 61) - (mulh(R, t1) >> 6);                                       // 1/2 - r t1
+        const int64_t l = (R >> 10) - (mulh(mulh(R, R), t2) >> 14);             // ln(1 + r), units 2^-60
+        const int e = 10 - lz + (j >= kLnHalf);
+        // -e ln 2 in units 2^-58 (up to 2^63.2, unsigned), ln 2 to 4 more bits
+        const uint64_t S = (uint64_t)(-e) * 0x2C5C85FDF473DE6ull + (uint64_t)((-e * 11 + 8) >> 4) - (uint64_t)((T.ln[j] + l + 2) >> 2);
+        o.V = (S + 1) >> 1;                              // 2 (-ln u1) in units 2^-56
+    }
+    {
+        const int sh = clz64(o.V | 1) & ~1;
+        o.q = 4 - (sh >> 1);
+        o.X = o.V ? sqrt_fix(o.V << sh) : 0;
+    }
+    {   // angle (pi / 2) (quarter + f): f's top 8 bits by table, the rest d = (pi / 2) 2^-8 f'
+        const uint64_t A = k2 << 11;
+        const int quarter = (int)(A >> 62), j = (int)(A >> 54) & 255;
+        const int64_t D = mulh((int64_t)((A << 10) ^ (1ull << 63)) >> 1, 0x3243F6A8885A308Dll);  // units 2^-68; pi / 2 in 2^-61
+        const int64_t D2 = mulh(D, D);                   // units 2^-72, < 2^-16.6
+        const float d2 = (float)(int32_t)(D2 >> 26) * 1.4210854715202004e-14f;   // units 2^-46
+        const int64_t c1 = -(D2 >> 7) + (int64_t)f2i(d2 * d2 * fmaf(d2, -1.0f / 720.0f, 1.0f / 24.0f) * 7.378697629483821e19f);  // cos d - 1, 2^-66
+        // d^2 / 6 - d^4 / 120, units 2^-70
+        const int64_t t = (mulh(D2, 0x2AAAAAAAAAAAAAABll) >> 2) - (int64_t)f2i(d2 * d2 * (1.0f / 120.0f) * 1.180591620717411e21f);
+        const int64_t s1 = D - (mulh(D, t) >> 6);        // sin d, units 2^-68
+        const int64_t C = T.cs[j], S = T.sn[j];
+        const int64_t x = C + (mulh(C, c1) >> 2) - (mulh(S, s1) >> 4);
+        const int64_t y = S + (mulh(S, c1) >> 2) + (mulh(C, s1) >> 4);
+        const int64_t a = quarter & 1 ? y : x, b = quarter & 1 ? x : y;
+        o.cs = quarter == 1 || quarter == 2 ? -a : a;
+        o.sn = quarter >= 2 ? -b : b;
+    }
+    return o;
+}
+
 }  // namespace bvfix

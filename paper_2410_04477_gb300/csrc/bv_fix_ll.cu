@@ -242,3 +242,17 @@ void bv_fix_tables(uint64_t* t) {
         t[256 + j] = j ? (uint64_t)(exp2l(-(long double)j / 65536.0L) * 0x1p63L + 0.5L) : (1ull << 63) - 1;
     }
 }
+
+// The Box-Muller pairs' tables (bv_fix.cuh).
+size_t bv_sim_table_bytes() { return sizeof(bvfix::SimTab); }
+void bv_sim_table(void* out) {
+    bvfix::SimTab& t = *static_cast<bvfix::SimTab*>(out);
+    const long double half_pi = 1.570796326794896619231321691639751442L;
+    for (int j = 0; j < 256; ++j) {
+        const long double x = ((long double)j + 0.5L) / 256.0L;
+        t.c[j] = (uint16_t)(j == 0 ? 32768 : j == 255 ? 16384 : (int)(32768.0L / (1.0L + x) + 0.5L));
+        t.ln[j] = (int64_t)floorl(-logl((long double)t.c[j] / 32768.0L * (j >= bvfix::kLnHalf ? 2.0L : 1.0L)) * 0x1p60L + 0.5L);
+        t.cs[j] = (int64_t)(cosl(half_pi * x) * 0x1p62L + 0.5L);
+        t.sn[j] = (int64_t)(sinl(half_pi * x) * 0x1p62L + 0.5L);
+    }
+}

@@ -161,6 +161,8 @@ size_t bv_fix_slot_bytes(int nmax);
 int bv_fix_occupancy(int kind, int threads, size_t smem);
 cudaError_t bv_fix_launch(int kind, int threads, int grid, size_t smem, const LLArgs& a, cudaStream_t s);
 void bv_fix_tables(uint64_t* t);  // 512 values
+size_t bv_sim_table_bytes();
+void bv_sim_table(void* out);
 
 // Launchers (bv_loglik.cu).
 int bv_smem_max_n(int kind, int d);
@@ -297,6 +299,7 @@ struct bv_ctx {
     double* h_out = nullptr;          // pinned, ndata
     DevTheta* d_theta = nullptr;      // ndata
     uint64_t* d_fixtab = nullptr;     // fixed-point exponential tables (bv_fix_tables)
+    unsigned char* d_simtab = nullptr;  // tables of the simulation's normal pairs (bv_sim_table)
     double* d_gtab = nullptr;         // 2 x ndata x BV_GTAB_DOUBLES: general-nu Matern tables, then their fixed-point forms
     std::vector<DevTheta> h_theta;    // ndata (pageable: copies are staged by the driver)
     unsigned long long* h_fail = nullptr;  // pinned

@@ -388,33 +388,48 @@ __global__ void __launch_bounds__(kPredFixNT, 4) k_pred_fix(PredArgs a) {
 // c = j ceil(R/2) + k, and gives z_2k = rho cos(2 pi u2) and z_2k+1 = rho sin(2 pi u2)
 // (the second dropped when 2k + 1 = R).  Because every draw is mu + sd z, the sample mean
 // is mu + sd zbar and the sample variance sd^2 (sum z^2 - R zbar^2) / (R - 1), so one pass
-// accumulating sum z and sum z^2 replaces the two passes over the draws.
+// accumulating sum z and sum z^2 replaces the two passes over the draws; and a whole pair's
+// z^2 sum to rho^2.  The logarithm, root, sine and cosine are taken in fixed point (bv_fix.cuh):
+// in FP64 their 110 operations a pair, at 2 lanes a clock and SM, were the kernel's time.
+// Sums: z in units 2^-50 (rounded: 2^-51 of draws of size 1), rho^2 exactly.
 __global__ void __launch_bounds__(256) k_cond_sim(const double* __restrict__ mean, const double* __restrict__ var,
                                                   const double* __restrict__ ytrue, int64_t n_star, int R,
-                                                  uint64_t stream, double zc, double* __restrict__ lower,
-                                                  double* __restrict__ upper, unsigned long long* covered) {
+                                                  uint64_t stream, double zc, const bvfix::SimTab* __restrict__ tab,
+                                                  double* __restrict__ lower, double* __restrict__ upper,
+                                                  unsigned long long* covered) {
+    __shared__ bvfix::SimTab T;
+    for (int i = threadIdx.x; i < (int)(sizeof(bvfix::SimTab) / 4); i += 256)
+        reinterpret_cast<uint32_t*>(&T)[i] = reinterpret_cast<const uint32_t*>(tab)[i];
+    __syncthreads();
     const int lane = threadIdx.x & 31;
     const int64_t w0 = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
-    const int half = (R + 1) >> 1;
+    const int half = (R + 1) >> 1, whole = R >> 1;
+    const auto pair = [&](uint64_t c) {
+        return bvfix::pair_fix(bv_sm64(stream, 2 * c) >> 11, bv_sm64(stream, 2 * c + 1) >> 11, T);
+    };
     for (int64_t j = w0; j < n_star; j += nw) {
         const uint64_t c0 = (uint64_t)j * (uint64_t)half;
         double s1 = 0.0, s2 = 0.0;
-        for (int k = lane; k < half; k += 32) {
-            const uint64_t c = c0 + (uint64_t)k;
-            const double u1 = 1.0 - (double)(bv_sm64(stream, 2 * c) >> 11) * 0x1p-53;
-            const double u2 = (double)(bv_sm64(stream, 2 * c + 1) >> 11) * 0x1p-53;
-            const double rho = sqrt(-2.0 * log(u1));
-            double sn, cs;
-            sincospi(2.0 * u2, &sn, &cs);
-            const double za = rho * cs;
+        for (int k0 = lane; k0 < whole; k0 += 32 * 256) {  // (256 pairs a lane stay in range)
+            int64_t z = 0;
+            uint64_t vh = 0, vl = 0;
+            const int k1 = min(whole, k0 + 32 * 256);
+            for (int k = k0; k < k1; k += 32) {
+                const bvfix::Pair p = pair(c0 + (uint64_t)k);
+                const int64_t P = bvfix::mulh((int64_t)(p.X >> 1), p.cs + p.sn);  // units 2^(q - 60)
+                z += (P + (1ll << (9 - p.q))) >> (10 - p.q);
+                vh += p.V >> 32;
+                vl += (uint32_t)p.V;
+            }
+            s1 += (double)z * 0x1p-50;
+            s2 += (double)vh * 0x1p-24 + (double)vl * 0x1p-56;
+        }
+        if (half > whole && lane == 0) {  // the last draw of an odd number
+            const bvfix::Pair p = pair(c0 + (uint64_t)whole);
+            const double za = ldexp((double)bvfix::mulh((int64_t)(p.X >> 1), p.cs), p.q - 60);
             s1 += za;
             s2 = fma(za, za, s2);
-            if (2 * k + 1 < R) {
-                const double zb = rho * sn;
-                s1 += zb;
-                s2 = fma(zb, zb, s2);
-            }
         }
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1) {
@@ -711,7 +726,8 @@ extern "C" int bv_cond_sim(bv_ctx* c, int32_t rounds, uint64_t seed, double z_cr
     const int64_t warps = p->n_star;
     const int64_t grid = std::max<int64_t>(1, std::min<int64_t>((warps + 7) / 8, (int64_t)c->num_sms * 8));
     k_cond_sim<<<(unsigned)grid, 256, 0, c->stream>>>(p->d_mean, p->d_var, p->d_ytrue, p->n_star, rounds,
-                                                      BV_STREAM_CSIM(seed), z_crit, p->d_lo, p->d_up, p->d_count);
+                                                      BV_STREAM_CSIM(seed), z_crit, reinterpret_cast<const bvfix::SimTab*>(c->d_simtab),
+                                                      p->d_lo, p->d_up, p->d_count);
     BV_CUDA(cudaGetLastError());
     unsigned long long cnt = 0;
     BV_CUDA(cudaMemcpyAsync(&cnt, p->d_count, sizeof(cnt), cudaMemcpyDeviceToHost, c->stream));
