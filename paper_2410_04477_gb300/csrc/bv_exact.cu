@@ -5,13 +5,15 @@
 // The (n+1) x (n+1) augmented matrix [[Sigma, .], [y^T, .]], divided by the diagonal D =
 // sigma^2 + tau^2, in the fixed-point form of bv_fix_tile.cuh: packed lower 16 x 16 tiles of
 // 64-bit entries, products of factor entries on the tensor cores through their digits.  At n =
-// 8,000 26.8 ms; FP64 arithmetic, 2 lanes a clock and SM, took 188.7 ms (n^3 / 3 operations at
+// 8,000 22.0 ms; FP64 arithmetic, 2 lanes a clock and SM, took 188.7 ms (n^3 / 3 operations at
 // 72% of its peak).  Right-looking by panels of 64 columns (four tiles), three launches a panel:
 //   k_ex_diag    the 64 x 64 diagonal block, one CTA
 //   k_ex_rows    the rows below it, 32 of them a warp: four solves against the 16 x 16
 //                diagonal tiles with the updates between them, and the rows' digits
 //   k_ex_update  A_IJ -= sum over the panel's four tiles of L_I L_J^T, a CTA per 64 x 64 block,
-//                the sums of a block kept in registers so that it is read and written once
+//                the sums of a block kept in registers so that it is read and written once;
+//                the next panel's block column first, so that its diagonal block and rows run
+//                on a stream of higher priority beside the update of the rest
 // The factor's row n is z = L^-1 y, so y^T Sigma^-1 y = |z|^2 and log|Sigma| is the sum of the
 // pivots' logarithms.  The data row is scaled by a power of two; should a solved entry leave
 // the fixed-point range, the factorisation is done again with a larger one.
@@ -194,14 +196,22 @@ __global__ void __launch_bounds__(128) k_ex_rows(ExArgs a, int P) {
     if (flags) atomicOr(a.flags, flags);
 }
 
-// Trailing 64 x 64 block (bi, bj): warp w has tile row w / 2 and two tile columns of it.
-__global__ void __launch_bounds__(256, 2) k_ex_update(ExArgs a, int P) {
+// Trailing 64 x 64 blocks (bi, bj), bj <= bi: those of block column j0 (first) or all beyond it.
+// Warp w has tile row w / 2 and two tile columns of the block.
+__global__ void __launch_bounds__(256, 2) k_ex_update(ExArgs a, int P, int j0, bool first) {
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int64_t f = blockIdx.x;
-    int64_t x = (int64_t)((sqrt(8.0 * (double)f + 1.0) - 1.0) * 0.5);
-    while ((x + 1) * (x + 2) / 2 <= f) ++x;
-    while (x * (x + 1) / 2 > f) --x;
-    const int bi = P + 1 + (int)x, bj = P + 1 + (int)(f - x * (x + 1) / 2);
+    int bi, bj;
+    if (first) {
+        bi = j0 + (int)f;
+        bj = j0;
+    } else {
+        int64_t x = (int64_t)((sqrt(8.0 * (double)f + 1.0) - 1.0) * 0.5);
+        while ((x + 1) * (x + 2) / 2 <= f) ++x;
+        while (x * (x + 1) / 2 > f) --x;
+        bi = j0 + 1 + (int)x;
+        bj = j0 + 1 + (int)(f - x * (x + 1) / 2);
+    }
     const int I = kP * bi + (warp >> 1), J0 = kP * bj + 2 * (warp & 1), tc = min(kP, a.TC - kP * P);
     if (I >= a.T || J0 > I || J0 >= a.TC) return;
     const bool two = J0 + 1 <= I && J0 + 1 < a.TC;
@@ -269,13 +279,20 @@ __global__ void __launch_bounds__(256) k_exact_terms(const int64_t* piv, const i
     }
 }
 
-// The call's device memory, taken from the stream's pool and given back on every path.
+// The call's device memory, taken from the stream's pool, and its second stream, given back on
+// every path: the second stream's work is waited for before the memory goes.
 struct ExBuf {
-    cudaStream_t s;
+    cudaStream_t s, hi = nullptr;
+    cudaEvent_t ready = nullptr, rest = nullptr;  // on s: a panel's rows are wanted; the rest is updated
+    cudaEvent_t rows = nullptr;                   // on hi: a panel's rows and digits are there
     void* p = nullptr;
     explicit ExBuf(cudaStream_t st) : s(st) {}
     ~ExBuf() {
+        if (hi) cudaStreamSynchronize(hi);
         if (p) cudaFreeAsync(p, s);
+        for (cudaEvent_t e : {ready, rest, rows})
+            if (e) cudaEventDestroy(e);
+        if (hi) cudaStreamDestroy(hi);
     }
 };
 
@@ -304,7 +321,7 @@ extern "C" int bv_exact_loglik(bv_ctx* c, const bv_theta* theta, int32_t use_y, 
     const int64_t ntiles = (int64_t)a.T * (a.T + 1) / 2;
     // one allocation: tiles | row digits | factors, roots and digits of the diagonal block |
     // pivots | data row | terms, flags, largest |y|
-    const size_t szA = (size_t)ntiles * kTileB, szD = (size_t)a.T * kP * kDigB, szL = kP * kLdN * sizeof(int4);
+    const size_t szA = (size_t)ntiles * kTileB, szD1 = (size_t)a.T * kP * kDigB, szD = 2 * szD1, szL = kP * kLdN * sizeof(int4);
     const size_t szR = kP * 16 * sizeof(FixRs), szE = 6 * kDigB, szN = (size_t)a.TC * 16 * sizeof(int64_t);
     ExBuf buf(st);
     BV_CUDA(cudaMallocAsync(&buf.p, szA + szD + szL + szR + szE + 2 * szN + 32, st));
@@ -325,6 +342,13 @@ extern "C" int bv_exact_loglik(bv_ctx* c, const bv_theta* theta, int32_t use_y, 
     a.flags = reinterpret_cast<int*>(terms + 2);
     BV_CUDA(cudaMemsetAsync(a.Ld, 0, szL + szR + szE + 2 * szN + 32, st));
     BV_CUDA(cudaFuncSetAttribute(k_ex_rows, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kRowsSmem));
+    uint32_t* const dig0 = a.dig;
+    {
+        int lo = 0, hi = 0;
+        BV_CUDA(cudaDeviceGetStreamPriorityRange(&lo, &hi));
+        BV_CUDA(cudaStreamCreateWithPriority(&buf.hi, cudaStreamNonBlocking, hi));
+        for (cudaEvent_t* e : {&buf.ready, &buf.rest, &buf.rows}) BV_CUDA(cudaEventCreateWithFlags(e, cudaEventDisableTiming));
+    }
     int E = 0;
     if (use_y) {
         k_ex_ymax<<<(unsigned)std::min<int64_t>((n + 255) / 256, c->num_sms), 256, 0, st>>>(c->d_y, n, th.diag_rsqrt,
@@ -344,15 +368,27 @@ extern "C" int bv_exact_loglik(bv_ctx* c, const bv_theta* theta, int32_t use_y, 
         if (th.nu_code == NU_GENERAL) k_ex_fill<true><<<fg, 256, 0, st>>>(a, ntiles);
         else k_ex_fill<false><<<fg, 256, 0, st>>>(a, ntiles);
         BV_CUDA(cudaGetLastError());
+        BV_CUDA(cudaEventRecord(buf.ready, st));
+        BV_CUDA(cudaStreamWaitEvent(buf.hi, buf.ready, 0));
         for (int P = 0; P < np; ++P) {
-            k_ex_diag<<<1, 128, 0, st>>>(a, P);
+            // hi: the panel (its block column is up to date), then the next block column, which
+            // the rest of panel P - 1's update has to have passed; st: the rest of this panel's
+            // update.  The digits of two panels are in use at a time.
+            a.dig = dig0 + (P & 1) * (szD1 / 4);
+            k_ex_diag<<<1, 128, 0, buf.hi>>>(a, P);
             const int64_t strips = a.T - (int64_t)kP * (P + 1), m = nb - P - 1;
-            if (strips > 0) {
-                k_ex_rows<<<(unsigned)((strips + 7) / 8), 128, kRowsSmem, st>>>(a, P);
-                k_ex_update<<<(unsigned)(m * (m + 1) / 2), 256, 0, st>>>(a, P);
-            }
+            if (strips <= 0) break;
+            k_ex_rows<<<(unsigned)((strips + 7) / 8), 128, kRowsSmem, buf.hi>>>(a, P);
+            BV_CUDA(cudaEventRecord(buf.rows, buf.hi));
+            BV_CUDA(cudaStreamWaitEvent(st, buf.rows, 0));
+            if (P > 0) BV_CUDA(cudaStreamWaitEvent(buf.hi, buf.rest, 0));
+            k_ex_update<<<(unsigned)m, 256, 0, buf.hi>>>(a, P, P + 1, true);
+            if (m > 1) k_ex_update<<<(unsigned)(m * (m - 1) / 2), 256, 0, st>>>(a, P, P + 1, false);
+            BV_CUDA(cudaEventRecord(buf.rest, st));
         }
         BV_CUDA(cudaGetLastError());
+        BV_CUDA(cudaEventRecord(buf.rows, buf.hi));
+        BV_CUDA(cudaStreamWaitEvent(st, buf.rows, 0));
         k_exact_terms<<<1, 256, 0, st>>>(a.piv, a.zrow, n, th.diag * 0x1p-60, ldexp(1.0, E - bvfix::kUnitL), terms);
         BV_CUDA(cudaGetLastError());
         BV_CUDA(cudaMemcpyAsync(&h, terms, sizeof(double) * 2 + sizeof(int), cudaMemcpyDeviceToHost, st));
