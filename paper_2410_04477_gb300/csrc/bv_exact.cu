@@ -5,7 +5,7 @@
 // The (n+1) x (n+1) augmented matrix [[Sigma, .], [y^T, .]], divided by the diagonal D =
 // sigma^2 + tau^2, in the fixed-point form of bv_fix_tile.cuh: packed lower 16 x 16 tiles of
 // 64-bit entries, products of factor entries on the tensor cores through their digits.  At n =
-// 8,000 22.0 ms; FP64 arithmetic, 2 lanes a clock and SM, took 188.7 ms (n^3 / 3 operations at
+// 8,000 21.8 ms; FP64 arithmetic, 2 lanes a clock and SM, took 188.7 ms (n^3 / 3 operations at
 // 72% of its peak).  Right-looking by panels of 64 columns (four tiles), three launches a panel:
 //   k_ex_diag    the 64 x 64 diagonal block, one CTA
 //   k_ex_rows    the rows below it, 32 of them a warp: four solves against the 16 x 16

@@ -23,16 +23,17 @@
 // Against a 113-bit factorisation of the same scaled coordinates, the blocks' ell errs by
 // 8.4e-13 (RMS; n = 20,000, m = 60, nu = 3/2, tau^2 = 1e-4), FP64 arithmetic by 2.8e-12; at m =
 // 113 by 4.9e-13 against 1.9e-12.  Time of an evaluation, FP64 arithmetic and this kernel:
-//   n = 200,000, m = 60 (N about 70)        5.04 ms   2.60 ms
-//   n = 36,931, m = 113                     3.64      1.20
-//   n = 100,000, 3D, m = 200                42.4      9.60
-//   n = 50,000, blocks of 1, m = 30         2.36      1.64
-//   n = 100,000, m = 60, nu = 1.2           4.92      2.38
+//   n = 200,000, m = 60 (N about 70)        5.04 ms   2.40 ms
+//   n = 36,931, m = 113                     3.64      1.16
+//   n = 100,000, 3D, m = 200                42.4      9.35
+//   n = 50,000, blocks of 1, m = 30         2.36      1.54
+//   n = 100,000, m = 60, nu = 1.2           4.92      2.20
 //   n = 2,000, m = 30                       0.122     0.094
-// What bounds it: up to N about 100 the latency of the pivots' chain (a tile's 16 pivots take
-// some 13,000 clocks, in which the other warps follow one pair of columns behind) with four to
-// eight blocks an SM; beyond, instruction issue, shared by the covariance, the panel rows and
-// the sums of digit products, the tensor cores themselves being busy a tenth of the time.
+// What bounds it: for few blocks the pivots' chain (a tile's 16 pivots take some 12,000 clocks,
+// in which the other warps follow two columns behind); else instruction issue and fetch, shared
+// by the covariance, the panel rows and the sums of digit products, with the tensor cores busy
+// for a twentieth of the time at N about 70.  More warps an SM, and starting a panel's chain
+// beside the update before it, were measured and lose; halving the code gained 3 to 4%.
 #include <cuda_runtime.h>
 #include <math.h>
 #include <stdint.h>

@@ -134,7 +134,7 @@ __device__ __forceinline__ void fix_diag(const longlong2* tile, int nc, int k0, 
         for (int s = 0; s < 2; ++s) {
             const int c = 2 * k + s;
             const bool on = c < nc;
-            const int64_t p0 = shfl64(dg + (int64_t)((uint64_t)(int64_t)bvfix::f2i(df) << 2), c);
+            const int64_t p0 = shfl64(bvfix::smad(bvfix::f2i(df), 4, dg), c);
             const bool bad = on && p0 <= kPivMin;
             const int64_t p = p0 > kPivMin ? p0 : 1;
             const bvfix::Rsq rs = bvfix::rsqrt_fix(p);
@@ -146,7 +146,7 @@ __device__ __forceinline__ void fix_diag(const longlong2* tile, int nc, int k0, 
                     bvfix::msub(a[q], fc[q], -f.h, -f.hf, -f.lf, l.x, __int_as_float(l.y), __int_as_float(l.z));
                 }
             }
-            const int64_t v = shfl64(a[0] + (int64_t)((uint64_t)(int64_t)bvfix::f2i(fc[0]) << 2), r + 16 * s);
+            const int64_t v = shfl64(bvfix::smad(bvfix::f2i(fc[0]), 4, a[0]), r + 16 * s);
             const int64_t x = fix_scale(v, rb, rs.e);
             f = bvfix::fac(x);
             bvfix::msub(dg, df, -f.h, -f.hf, -f.lf, f.h, f.hf, f.lf);
@@ -187,7 +187,7 @@ __device__ __forceinline__ void fix_row4(int64_t* a, float* fc, int c0, const in
 #pragma unroll 1
     for (int c = c0; c < c0 + 4; ++c) {
         if (wait && !(c & 1) && !pair_wait(mb + (c >> 1), parity)) flags |= kFail;
-        const int64_t v = a[0] + (int64_t)((uint64_t)(int64_t)bvfix::f2i(fc[0]) << 2);
+        const int64_t v = bvfix::smad(bvfix::f2i(fc[0]), 4, a[0]);
         const FixRs rs = rsv[c];
         const int64_t x = fix_scale(v, rs.r, rs.e);
         const Fac f = bvfix::fac(x);
@@ -256,40 +256,42 @@ __device__ __forceinline__ void fix_row(const longlong2* tile, const int4* Ld, c
     }
 }
 
-// The sum of the digit products of one entry (orders 0 .. 5: units 2^-18 .. 2^-68; f6: the
-// middle pair of order 6) in matrix units.  FAST: the FP32 whole numbers become integers by
-// adding 1.5 2^23 (their low bits), a quarter of a clock each instead of a conversion's two;
-// right while all are below 2^22 in size, else *wide shows bits above.
+// The sum of the digit products of one entry (orders 0 .. 5: units 2^-18 .. 2^-68; f6: what is
+// added in units of order 5) in matrix units.  FAST: the FP32 whole numbers f become integers
+// kB + f by adding 1.5 2^23 (a quarter of a clock each, a conversion takes two); right while all
+// are below 2^22 in size, else *wide shows bits above.  Orders 0 and 1 are that small by the
+// rows' norms (at most 1, and 16 entries of 0.71 in the data row), so only the others are looked
+// at.  The weights are multiply-adds on the FMA pipe, the offsets kB one constant: the ALU is
+// what bounds the update.
 template <bool FAST>
-__device__ __forceinline__ int64_t digit_sum(const float (&f)[kDig], int f6, uint32_t& wide) {
+__device__ __forceinline__ int64_t digit_sum(const float (&f)[kDig], uint32_t f6, uint32_t& wide) {
     constexpr uint32_t kB = 0x4B400000u;
-    uint32_t i[kDig];
+    constexpr uint64_t kOff = 0ull - (((uint64_t)kB << 22) + ((uint64_t)kB << 12) + ((uint64_t)kB << 2) + (kB >> 8));
+    uint32_t u[kDig];
 #pragma unroll
     for (int k = 0; k < kDig; ++k) {
-        if (FAST) {
-            const uint32_t u = __float_as_uint(f[k] + 12582912.0f);
-            wide |= u ^ 0x4B000000u;
-            i[k] = u - kB;
-        } else {
-            i[k] = (uint32_t)__float2int_rn(f[k]);
-        }
+        u[k] = FAST ? __float_as_uint(f[k] + 12582912.0f) : kB + (uint32_t)__float2int_rn(f[k]);
+        if (FAST && k > 1) wide |= u[k] ^ 0x4B000000u;
     }
-    // orders 0 and 1 (below 2^18 and 2^21) have weights 2^42 and 2^32: the high word alone
-    const uint32_t top = (i[0] << 10) + i[1];
-    const int low = (int)(i[4] << 2) + (((int)i[5] + (f6 >> 10)) >> 8);
-    const int64_t mid = bvfix::smad((int)i[2], 1 << 22, bvfix::smad((int)i[3], 1 << 12, low));
-    return mid + (int64_t)((uint64_t)top << 32);
+    // orders 0 and 1 have weights 2^42 and 2^32: the high word alone
+    const uint32_t top = (u[0] << 10) + u[1] - ((kB << 10) + kB);
+    const uint64_t mid = bvfix::umad(u[2], 1u << 22, bvfix::umad(u[3], 1u << 12, bvfix::umad(u[4], 4u, bvfix::umad((u[5] + f6) >> 8, 1u, kOff))));
+    return (int64_t)(mid + ((uint64_t)top << 32));
 }
 
 template <bool FAST>
-__device__ __forceinline__ bool digit_sums(int64_t (&o)[4], const float (&acc)[kDig][4], const float (&a6)[4]) {
-    uint32_t wide = 0;
+__device__ __forceinline__ bool digit_sums(int64_t (&o)[4], const float (&acc)[kDig][4], const float (&a6)[4], bool diag) {
+    uint32_t wide = 0, f6[4] = {0, 0, 0, 0};
+    if (diag) {
+#pragma unroll
+        for (int e = 0; e < 4; ++e) f6[e] = (uint32_t)(__float2int_rn(a6[e]) >> 10);
+    }
 #pragma unroll
     for (int e = 0; e < 4; ++e) {
         float f[kDig];
 #pragma unroll
         for (int k = 0; k < kDig; ++k) f[k] = acc[k][e];
-        o[e] = digit_sum<FAST>(f, __float2int_rn(a6[e]), wide);
+        o[e] = digit_sum<FAST>(f, f6[e], wide);
     }
     return !FAST || !__any_sync(0xffffffffu, wide >= 0x800000u);
 }
@@ -319,7 +321,7 @@ __device__ __forceinline__ void digit_dot(int64_t (&o)[4], const uint2 (&A)[kDig
         for (int k = s; k < kDig; ++k) mma_f16(acc[k], A[k - s][0], A[k - s][1], B);
         if (s == 3 && diag) mma_f16(a6, A[3][0], A[3][1], B);
     }
-    if (!digit_sums<true>(o, acc, a6)) digit_sums<false>(o, acc, a6);
+    if (!digit_sums<true>(o, acc, a6, diag)) digit_sums<false>(o, acc, a6, diag);
 }
 
 // C -= L_I L_J^T for one tile, one warp; dI, dJ: the tiles' digits.
