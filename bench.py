@@ -34,17 +34,19 @@ sys.path.insert(0, ROOT)
 from paper_2410_04477_gb300 import synth  # noqa: E402
 
 UNIT = "evals/s"
-FP64_PEAK_TFLOPS = 1.25  # nominal GB300 FP64 (vector and tensor), used as the ALU roofline
+# FP64-accurate products through 10-bit digits: 21 FP16 products each, exact in FP32 sums, so
+# the roofline is the measured dense FP16/BF16 tensor rate over 21 (the FP64 pipe itself: 1.25)
+DIGIT_PAIRS, BF16_TFLOPS = 21, 1930.3
+FP64_PEAK_TFLOPS = BF16_TFLOPS / DIGIT_PAIRS
+FP64_PEAK_SOURCE = ("measured dense BF16 GEMM, 1930 TFLOP/s, over the 21 digit products of an FP64-accurate one "
+                    "(the FP64 pipe: 1.25 TFLOP/s nominal)")
 SM_COUNT, FP32_LANES, SM_MAX_MHZ = 152, 128, 2070.0
 FP32_PEAK_TFLOPS = SM_COUNT * FP32_LANES * 2 * SM_MAX_MHZ * 1e6 / 1e12  # 80.5 at max clock
 
 # DRAM bytes (read + write) of one evaluation's likelihood-kernel launches, summed over
 # the size bins, from an ncu capture (dram__bytes_read.sum + dram__bytes_write.sum);
-# reported as roofline.traffic for these workloads and precisions only.
-NCU_TRAFFIC = {("c2_m60", "fp64"): 636_160 + 10_996_224 + 2_597_376 + 40_704 + 36_864 + 34_816,
-               # config 3: the main bin's 5,937,920 bytes at n-scale 0.05 (4,974 of its 99,949
-               # blocks; the other bins hold 51 blocks), times 20
-               ("c3", "fp64"): 20 * 5_937_920}
+# reported as roofline.traffic for the workloads and precisions captured.
+NCU_TRAFFIC = {}
 
 WORKLOADS = {
     # batched plain FP64: 2e5 uniform points, bc 2e4, m 60 / 120, y from BV at m=400
@@ -612,10 +614,10 @@ def run_pred(args, w, log):
            "h2d_bytes_per_step": int((~hold).sum()) * 8, "d2h_bytes_per_step": n_star * 8 * 4 + 16}
     mean_pred = statistics.mean(pred_ms) / 1e3
     achieved = flops / mean_pred / 1e12
-    roof = {"bound": "alu", "kernel": "k_pred (one launch: covariance + partial augmented Cholesky of every "
+    roof = {"bound": "tensor", "kernel": "k_pred_fix (one launch: covariance + partial augmented Cholesky of every "
             "prediction block)", "achieved": achieved, "peak": FP64_PEAK_TFLOPS, "unit": "TFLOP/s",
             "frac": achieved / FP64_PEAK_TFLOPS, "traffic": None,
-            "peak_source": "nominal GB300 FP64 1.25 TFLOP/s (no FP64 entry in MEASURED_PEAKS.json; probe 1.19)",
+            "peak_source": FP64_PEAK_SOURCE,
             "flops_per_launch": flops, "cov_entries_per_launch": cov_evals}
     cpu = None
     if not args.no_cpu and rank == 0 and ws == 1:
@@ -692,10 +694,10 @@ def run_kl(args, w, log):
     tot_ms = max_over_ranks(float(sum(ms)))
     value = ws * args.steps / (tot_ms / 1e3)
     achieved = flops / (statistics.mean(ms) / 1e3) / 1e12
-    roof = {"bound": "alu", "kernel": "k_update + k_trsm + k_potrf (tiled dense Cholesky, one exact evaluation)",
+    roof = {"bound": "tensor", "kernel": "k_ex_diag + k_ex_rows + k_ex_update (tiled dense Cholesky, one exact evaluation)",
             "achieved": achieved, "peak": FP64_PEAK_TFLOPS, "unit": "TFLOP/s", "frac": achieved / FP64_PEAK_TFLOPS,
             "traffic": None, "flops_per_launch_sequence": flops,
-            "peak_source": "nominal GB300 FP64 1.25 TFLOP/s (no FP64 entry in MEASURED_PEAKS.json; probe 1.19)"}
+            "peak_source": FP64_PEAK_SOURCE}
     # end to end: observations up, ell down, through the public call
     y = synth.normal(w["seed"], 20, n)
     t0 = time.perf_counter()
@@ -858,14 +860,14 @@ def main():
            "d2h_bytes_per_step": 8 * nd}
 
     achieved = info["flops"] / (mean_ms / 1e3) / 1e12
-    roof = {"bound": "alu", "kernel": "k_ll_fp64 (all size bins) + reduction, one evaluation",
+    roof = {"bound": "tensor", "kernel": "k_ll_fix (all size bins) + reduction, one evaluation",
             "achieved": achieved, "peak": FP64_PEAK_TFLOPS, "unit": "TFLOP/s",
             "frac": achieved / FP64_PEAK_TFLOPS, "traffic": NCU_TRAFFIC.get((args.workload, args.precision)),
             "traffic_unit": "bytes per evaluation (ncu dram__bytes_read.sum + dram__bytes_write.sum)",
-            "peak_source": "nominal GB300 FP64 1.25 TFLOP/s (no FP64 entry in MEASURED_PEAKS.json; probe 1.19)",
+            "peak_source": FP64_PEAK_SOURCE,
             "flops_per_eval": info["flops"], "cov_entries_per_eval": info["cov_entries"]}
     if prec == bv.BV_MIXED:
-        roof.update(kernel="k_ll_mixed (all size bins) + reduction, one evaluation", peak=FP32_PEAK_TFLOPS,
+        roof.update(bound="alu", kernel="k_ll_mixed (all size bins) + reduction, one evaluation", peak=FP32_PEAK_TFLOPS,
                     frac=achieved / FP32_PEAK_TFLOPS,
                     peak_source="FP32 FMA: 152 SMs x 128 lanes x 2 x 2070 MHz (probe 69.5 at ~1.99 GHz)")
 
