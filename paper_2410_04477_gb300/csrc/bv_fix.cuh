@@ -63,15 +63,16 @@ BV_FIX int64_t smad(int32_t a, int32_t b, int64_t c) { return (int64_t)((uint64_
 BV_FIX uint64_t umad(uint32_t a, uint32_t b, uint64_t c) { return (uint64_t)a * b + c; }
 #endif
 
-// High 64 bits of a b, up to 2 units low (the low x low product is left out); a, b < 2^63,
-// so that the two middle products sum without a carry: three multiply-adds.
+// High 64 bits of a b within 2 units, without bias (the low x low product is left out and the
+// middle one cut off, 0.75 units on average, which are added); a, b < 2^63, so that the two
+// middle products sum without a carry: three multiply-adds.
 BV_FIX uint64_t mulhi63(uint64_t a, uint64_t b) {
-    const uint64_t mid = umad(hi32(a), lo32(b), umad(lo32(a), hi32(b), 0));
+    const uint64_t mid = umad(hi32(a), lo32(b), umad(lo32(a), hi32(b), 0xC0000000ull));
     return umad(hi32(a), hi32(b), hi32(mid));
 }
 // The same for any a, b.
 BV_FIX uint64_t mulhi64(uint64_t a, uint64_t b) {
-    const uint64_t p = umad(hi32(a), lo32(b), 0), q = umad(lo32(a), hi32(b), 0);
+    const uint64_t p = umad(hi32(a), lo32(b), 0xA0000000ull), q = umad(lo32(a), hi32(b), 0xA0000000ull);
     return umad(hi32(a), hi32(b), hi32(p)) + hi32(q);
 }
 
@@ -189,7 +190,7 @@ BV_FIX Exp exp2_fix(uint64_t zf, const TA* A, const TB* B) {
     const uint64_t E = r - ((uint64_t)(uint32_t)q2 << 14);
     const uint64_t P = mulhi63(A[(zf >> 49) & 255], B[(zf >> 41) & 255]);
     Exp o;
-    o.W = P - (mulhi63(P, E) >> 14);
+    o.W = P - ((mulhi63(P, E) + 8192) >> 14);
     o.i = (int)(zf >> 57);
     return o;
 }

@@ -270,7 +270,9 @@ __device__ __forceinline__ int64_t digit_sum(const float (&f)[kDig], uint32_t f6
     uint32_t u[kDig];
 #pragma unroll
     for (int k = 0; k < kDig; ++k) {
-        u[k] = FAST ? __float_as_uint(f[k] + 12582912.0f) : kB + (uint32_t)__float2int_rn(f[k]);
+        // (order 5 with half of the 2^8 that it is cut by: rounded)
+        u[k] = FAST ? __float_as_uint(f[k] + (k == 5 ? 12583040.0f : 12582912.0f))
+                    : kB + (uint32_t)__float2int_rn(f[k]) + (k == 5 ? 128u : 0u);
         if (FAST && k > 1) wide |= u[k] ^ 0x4B000000u;
     }
     // orders 0 and 1 have weights 2^42 and 2^32: the high word alone

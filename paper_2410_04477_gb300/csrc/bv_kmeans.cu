@@ -30,6 +30,7 @@
 #include <algorithm>
 #include <vector>
 
+#include "bv_fix.cuh"
 #include "bv_internal.h"
 
 namespace {
@@ -62,9 +63,9 @@ constexpr int kTile = 256;  // centres per shared-memory tile
 // row-major FP64 centres [k][d].  L lanes a point, each with every L-th centre.  One FP32 pass
 // keeps the smallest two distances and the smallest one's centre: unless the second lies within
 // the rounding margin of the first, that centre is the exact minimiser.  The few points where it
-// does are scored exactly over the centres inside the margin.  (Scoring every point's candidates
-// in a second pass over all centres cost 218 us at n = 20,000, k = 2,000, with one lane a point
-// and half of the SMs without a block.)
+// does are scored exactly over the centres inside the margin.  76 us at n = 20,000, k = 2,000;
+// scoring every point's candidates in a second pass over all centres, with one lane a point and
+// half of the SMs without a block, took 218 us.
 template <int L>
 __global__ void __launch_bounds__(256) k_assign(const double* __restrict__ locs, int64_t n_tot,
                                                 int64_t off, int64_t n, int d,
@@ -301,14 +302,14 @@ __global__ void __launch_bounds__(kChunk) k_kpp_pick(const double* __restrict__ 
 
 // All picks of k-means++ in one launch, for sets that fit one cluster's registers: 8 CTAs of
 // 1,024 threads, P consecutive points a thread, so that the order of (CTA, warp, lane, point)
-// is the points' order.  The two launches a pick above cost their latency whatever the work: at n =
-// 20,000 and k = 2,000 the set-up (K-means, neighbours) took 37.0 ms with them and takes 16.7 ms
-// with this kernel.  Here a pick is two cluster barriers: the CTAs exchange their
-// weight sums; the one that holds the target scans its warps' sums and then that warp's lanes,
-// and writes the new centre into every CTA's shared memory.  Weights are whole numbers, so the
-// sums (kept up to date by differences) do not depend on the order of additions.  A point's
-// exact distance is only computed when its FP32 distance to the new centre is below thr, its
-// current distance and the rounding margin.
+// is the points' order.  The two launches a pick above cost their latency whatever the work: at
+// n = 20,000 and k = 2,000 the set-up (K-means, neighbours) took 37.0 ms with them, and takes
+// 13.2 ms with this kernel (8.4 ms) and the assignment above.  Here a pick is two cluster
+// barriers: the CTAs exchange their weight sums; the one that holds the target scans its warps'
+// sums and then that warp's lanes, and writes the new centre into every CTA's shared memory.
+// Weights are whole numbers, so the sums (kept up to date by differences) do not depend on the
+// order of additions.  A point's exact distance is only computed when its FP32 distance to the
+// new centre is not above thr, its current distance and the rounding margin.
 constexpr int kKppCtas = 8, kKppMaxP = 5;
 
 template <int P>
@@ -345,6 +346,7 @@ __global__ void __cluster_dims__(kKppCtas, 1, 1) __launch_bounds__(kChunk, 1)
     __syncthreads();
     for (int64_t t = 1; t < k; ++t) {
         const float c0 = (float)s_c[0], c1 = (float)s_c[1], c2 = (float)s_c[2];
+        const uint64_t r = bv_sm64(stream, (uint64_t)t);
         unsigned long long dw = 0;  // change of the thread's weight (modulo 2^64)
 #pragma unroll
         for (int p = 0; p < P; ++p) {
@@ -357,7 +359,7 @@ __global__ void __cluster_dims__(kKppCtas, 1, 1) __launch_bounds__(kChunk, 1)
                 }
                 if (v < D2[p]) {
                     D2[p] = v;
-                    const unsigned long long wn = (unsigned long long)ldexp(v, s);
+                    const unsigned long long wn = (unsigned long long)bvfix::scale2(v, s);  // as ldexp: exact, or below 1
                     dw += wn - w[p];
                     w[p] = wn;
                     const float vf = __double2float_ru(v);
@@ -383,7 +385,6 @@ __global__ void __cluster_dims__(kKppCtas, 1, 1) __launch_bounds__(kChunk, 1)
         unsigned long long W = 0;
 #pragma unroll
         for (int q = 0; q < kKppCtas; ++q) W += s_sum[q];
-        const uint64_t r = bv_sm64(stream, (uint64_t)t);
         int owner = kKppCtas - 1;
         unsigned long long target = 0, base = 0;
         int64_t pick = -1;
@@ -440,7 +441,7 @@ __global__ void __cluster_dims__(kKppCtas, 1, 1) __launch_bounds__(kChunk, 1)
             }
             if (pick >= 0 && (W != 0 || tid == 0)) {  // one thread
                 for (int q = 0; q < d; ++q) {
-                    const double v = locs[(int64_t)q * n_tot + off + pick];
+                    const double v = s_x[q * kChunk * P + (int)(pick - (int64_t)rank * kChunk * P)];  // a point of this CTA
                     cent[t * d + q] = v;
                     const uint32_t la = (uint32_t)__cvta_generic_to_shared(s_c + q);
                     for (int z = 0; z < kKppCtas; ++z) {
