@@ -312,6 +312,14 @@ __global__ void __launch_bounds__(kChunk) k_kpp_pick(const double* __restrict__ 
 // new centre is not above thr, its current distance and the rounding margin.
 constexpr int kKppCtas = 8, kKppMaxP = 5;
 
+// Barrier of all the cluster's threads, releasing and acquiring their writes to its shared memory.
+// The .aligned form needs a converged warp, which a branch taken by some of its lanes does not
+// leave by itself.
+__device__ __forceinline__ void cluster_sync() {
+    __syncwarp();
+    asm volatile("barrier.cluster.arrive.release.aligned;\nbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+
 template <int P>
 __global__ void __cluster_dims__(kKppCtas, 1, 1) __launch_bounds__(kChunk, 1)
     k_kpp_all(const double* __restrict__ locs, int64_t n_tot, int64_t off, int64_t n, int d, int s, float amax, uint64_t stream,
@@ -343,7 +351,7 @@ __global__ void __cluster_dims__(kKppCtas, 1, 1) __launch_bounds__(kChunk, 1)
     if (lane == 0) s_warp[warp] = 0;
     if (tid == 0) s_tot = 0;
     if (tid < 3) s_c[tid] = tid < d ? cent[tid] : 0.0;
-    __syncthreads();
+    cluster_sync();  // (another CTA's shared memory may be written once that CTA is known to run)
     for (int64_t t = 1; t < k; ++t) {
         const float c0 = (float)s_c[0], c1 = (float)s_c[1], c2 = (float)s_c[2];
         const uint64_t r = bv_sm64(stream, (uint64_t)t);
@@ -381,7 +389,7 @@ __global__ void __cluster_dims__(kKppCtas, 1, 1) __launch_bounds__(kChunk, 1)
             asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(ra) : "r"(la), "r"(tid));
             asm volatile("st.shared::cluster.u64 [%0], %1;" ::"r"(ra), "l"(s_tot) : "memory");
         }
-        asm volatile("barrier.cluster.arrive.release.aligned;\nbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+        cluster_sync();
         unsigned long long W = 0;
 #pragma unroll
         for (int q = 0; q < kKppCtas; ++q) W += s_sum[q];
@@ -452,7 +460,7 @@ __global__ void __cluster_dims__(kKppCtas, 1, 1) __launch_bounds__(kChunk, 1)
                 }
             }
         }
-        asm volatile("barrier.cluster.arrive.release.aligned;\nbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+        cluster_sync();
     }
 }
 
