@@ -112,6 +112,14 @@ BV_FIX void msub(int64_t& a, float& c, int32_t nxh, float nxhf, float nxlf, int3
     c = fmaf(nxlf, yhf, c);
 }
 
+// a - x^2 in matrix units for a factor entry x = h 2^29 + l, rounded: h h, 2 h l and l l (to 14 bits
+// of l) in whole numbers.  In FP32, as in msub, the cross term of an x near 1 errs by up to 2^-55,
+// and l l, left out, raises every pivot by 2^-63.6 a column.
+BV_FIX int64_t sub_square(int64_t a, int64_t x, int32_t h) {
+    const int32_t l = (int32_t)((uint32_t)x << 3) >> 3, lq = l >> 15;
+    return smad(-h, h, a) - (smad(h, l, smad(lq, lq, 1ll << 27)) >> 28);
+}
+
 // 1 / sqrt(P), P = p 2^-60, for p in [1, 2^60]: r 2^(e - 62) with r in [2^62, 2^63) and e >= 0,
 // within 2^-59 relative and exact for P = 1.  The hardware seed's mantissa Y (24 bits, error
 // 2^-22) takes a Newton step with the second-order term in fixed point, which cubes its error.

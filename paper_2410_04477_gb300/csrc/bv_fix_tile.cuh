@@ -100,7 +100,8 @@ __device__ __forceinline__ bool pair_wait(uint64_t* mb, uint32_t parity) {
 
 // Factor the diagonal tile of a panel (columns k0 .. k0 + nc - 1), one warp: lane r + 16 h
 // holds row r, columns of parity h, and the row's diagonal entry.  What bounds it is the chain
-// from one pivot to the next, which needs the diagonal entry alone (d -= x^2, no exchange);
+// from one pivot to the next, which needs the diagonal entry alone (d -= x^2, no exchange; a
+// whole-number product, which has no conversions in the chain and no rounding of the cross term);
 // the updates of the other columns by column c are done in the shadow of column c + 1's
 // reciprocal square root.  Two columns a turn and the registers moved down by one, so that the
 // code stays small: unrolled over the 16 columns, this and the row loop below ran at the rate
@@ -118,7 +119,6 @@ __device__ __forceinline__ void fix_diag(const longlong2* tile, int nc, int k0, 
         fc[q] = 0.0f;
     }
     int64_t dg;
-    float df = 0.0f;
     {
         const longlong2 v = tile[(r >> 3) * 96 + 4 * (r & 7) + ((r & 7) >> 1)];
         dg = (r & 1) ? v.y : v.x;
@@ -134,7 +134,7 @@ __device__ __forceinline__ void fix_diag(const longlong2* tile, int nc, int k0, 
         for (int s = 0; s < 2; ++s) {
             const int c = 2 * k + s;
             const bool on = c < nc;
-            const int64_t p0 = shfl64(bvfix::smad(bvfix::f2i(df), 4, dg), c);
+            const int64_t p0 = shfl64(dg, c);
             const bool bad = on && p0 <= kPivMin;
             const int64_t p = p0 > kPivMin ? p0 : 1;
             const bvfix::Rsq rs = bvfix::rsqrt_fix(p);
@@ -149,7 +149,7 @@ __device__ __forceinline__ void fix_diag(const longlong2* tile, int nc, int k0, 
             const int64_t v = shfl64(bvfix::smad(bvfix::f2i(fc[0]), 4, a[0]), r + 16 * s);
             const int64_t x = fix_scale(v, rb, rs.e);
             f = bvfix::fac(x);
-            bvfix::msub(dg, df, -f.h, -f.hf, -f.lf, f.h, f.hf, f.lf);
+            dg = bvfix::sub_square(dg, x, f.h);
             if (par == 0) {
                 Ld[c * kLd + r] = make_int4(f.h, __float_as_int(f.hf), __float_as_int(f.lf), 0);
                 if (r == ry && on) {
