@@ -13,6 +13,7 @@
 #include <string>
 #include <vector>
 
+#include "bv_fix.cuh"
 #include "bv_internal.h"
 
 // ------------------------------------------------------------------------------------
@@ -776,7 +777,7 @@ int bv_theta_to_dev(const bv_theta* t, int d, DevTheta* o) {
     o->diag_lo_f = (float)((o->sigma2 + o->nugget) - (double)d32);
     for (int k = 0; k < 3; ++k) o->inv_range_f[k] = (float)o->inv_range[k];
     o->diag = o->sigma2 + o->nugget;
-    o->diag_ratio = o->sigma2 / o->diag;
+    o->diag_ratio = o->diag < INFINITY ? bvfix::ratio63(o->sigma2, o->diag) : 0;
     o->diag_rsqrt = 1.0 / std::sqrt(o->diag);
     return BV_OK;
 }

@@ -58,8 +58,7 @@ struct ExArgs {
 template <bool GEN>
 __global__ void __launch_bounds__(256) k_ex_fill(ExArgs a, int64_t ntiles) {
     __shared__ uint64_t tA[256], tB[256];
-    const uint64_t rf = (uint64_t)__double2ull_rn(a.th.diag_ratio * 0x1p63);
-    tA[threadIdx.x] = bvfix::mulhi64(a.fixtab[threadIdx.x], rf) << 1;
+    tA[threadIdx.x] = bvfix::mulhi64(a.fixtab[threadIdx.x], a.th.diag_ratio) << 1;
     tB[threadIdx.x] = a.fixtab[256 + threadIdx.x];
     __syncthreads();
     const int lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3;

@@ -8,12 +8,12 @@
 // with an absolute error of 2^-60 or less, where FP64 arithmetic leaves 2^-54 on values
 // near 1.
 #pragma once
+#include <math.h>
 #include <stdint.h>
 
 #ifdef __CUDACC__
 #define BV_FIX __device__ __forceinline__
 #else  // host build of the arithmetic's own test
-#include <math.h>
 #include <string.h>
 #define BV_FIX static inline
 #endif
@@ -87,6 +87,28 @@ BV_FIX Bal bal(int64_t v) {
     b.h = (int32_t)(((uint64_t)v + 0x80000000ull) >> 32);
     return b;
 }
+// a / b in units 2^-63, rounded, for finite 0 < a <= b (host).  A rounding of sigma^2 / D to FP64's
+// 53 bits would be up to 64 units of 2^-60, of one sign in every covariance entry of a dataset.
+inline uint64_t ratio63(double a, double b) {
+    int ea = 0, eb = 0;
+    unsigned __int128 rem = (uint64_t)ldexp(frexp(a, &ea), 53);
+    const uint64_t den = (uint64_t)ldexp(frexp(b, &eb), 53);
+    uint64_t q = rem >= den ? 1 : 0;
+    rem -= q ? den : 0;
+    const int bits = 63 + ea - eb;  // (<= 63: a <= b)
+    if (bits < -1) return 0;
+    if (bits < 0) return q;         // a / b in [2^-65, 2^-63), rounded at 2^-64
+    for (int i = 0; i < bits; ++i) {
+        rem <<= 1;
+        q <<= 1;
+        if (rem >= den) {
+            rem -= den;
+            ++q;
+        }
+    }
+    return q + (2 * rem >= den ? 1 : 0);
+}
+
 // Scales: matrix entries and Schur complements in units of 2^-60 (kUnitC), factor entries in
 // units of 2^-59 (kUnitL).
 constexpr int kUnitC = 60, kUnitL = 59;

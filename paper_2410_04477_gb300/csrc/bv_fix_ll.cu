@@ -92,11 +92,11 @@ __global__ void __launch_bounds__(NT, WARPS * 32 / NT) k_ll_fix(LLArgs a) {
         int64_t* piv = reinterpret_cast<int64_t*>(yv + N);
         int64_t* zrow = piv + N;
 
-        const double D = th.diag, ratio = th.diag_ratio, isd = th.diag_rsqrt;
+        const double D = th.diag, isd = th.diag_rsqrt;
+        const uint64_t ratio = th.diag_ratio;
         if (ds != dsprev) {  // A[j] = 2^(-j/256) sigma^2 / D
-            const uint64_t rf = (uint64_t)__double2ull_rn(ratio * 0x1p63);
 #pragma unroll 1
-            for (int j = tid; j < 256; j += NT) tA[j] = bvfix::mulhi64(a.fixtab[j], rf) << 1;
+            for (int j = tid; j < 256; j += NT) tA[j] = bvfix::mulhi64(a.fixtab[j], ratio) << 1;
             dsprev = ds;
         }
         if (tid == 0) s_ymax = 0;
@@ -118,7 +118,7 @@ __global__ void __launch_bounds__(NT, WARPS * 32 / NT) k_ll_fix(LLArgs a) {
         if (lane == 0) atomicMax(&s_ymax, ym);
         __syncthreads();
         const int ye = (int)(s_ymax >> 20);
-        const bool valid = D > 0.0 && D < INFINITY && ratio >= 0.0 && ratio <= 1.0 && ye != 0x7ff;
+        const bool valid = D > 0.0 && D < INFINITY && ye != 0x7ff;
         int E = (ye > 0 ? ye - 1022 : -1021) + kYRoom;  // |y| 2^-E < 2^-kYRoom
 
         bool fail = false;

@@ -345,8 +345,9 @@ __device__ __forceinline__ void fix_update(longlong2* C, const uint32_t* dI, con
 }
 
 // The general smoothness through K_nu, in matrix units (not inlined: it is as long as all the rest).
-__device__ __noinline__ int64_t gen_direct(const DevTheta* th, double x, double ratio) {
-    return bvfix::unit_fix(fmin(matern_gen_corr(*th, x), 1.0) * ratio);
+__device__ __noinline__ int64_t gen_direct(const DevTheta* th, double x, uint64_t ratio) {
+    const uint64_t rho = (uint64_t)bvfix::unit_fix(fmin(matern_gen_corr(*th, x), 1.0)) << 3;
+    return (int64_t)((bvfix::mulhi64(rho, ratio) + 2) >> 2);
 }
 
 // One covariance tile (I, J), one warp, entries in matrix units: rows and columns of the points
@@ -355,7 +356,7 @@ __device__ __noinline__ int64_t gen_direct(const DevTheta* th, double x, double 
 // smoothness through K_nu itself.  PAD: rows m .. m16 - 1 are no points but rows of the identity.
 template <int GEN, bool PAD>
 __device__ __forceinline__ void fix_fill(longlong2* tp, int I, int J, int m, int m16, int N, int lane, const double* px, int d,
-                                         const int64_t* yfix, const DevTheta* th, int nu_code, double ratio, const int64_t* gt,
+                                         const int64_t* yfix, const DevTheta* th, int nu_code, uint64_t ratio, const int64_t* gt,
                                          const uint64_t* tA, const uint64_t* tB, int& flags) {
     const int g = lane >> 2, t = lane & 3;
 #pragma unroll 1

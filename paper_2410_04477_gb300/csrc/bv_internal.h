@@ -66,9 +66,11 @@ struct DevTheta {
     // (added to every pivot, so that the FP32 factor is that of the exact diagonal)
     float sigma2_f, nugget_f, inv_range_f[3];
     float diag_lo_f;
-    // normalised covariance of the fixed-point kernel: D = sigma^2 + tau^2, sigma^2 / D and
-    // 1 / sqrt(D)
-    double diag, diag_ratio, diag_rsqrt;
+    // normalised covariance of the fixed-point kernels: D = sigma^2 + tau^2 (rounded, as every
+    // kernel's diagonal is), sigma^2 / D in units 2^-63 and 1 / sqrt(D)
+    double diag;
+    uint64_t diag_ratio;
+    double diag_rsqrt;
 };
 
 // Constants of the table-driven FP64 exponential (Tang, "Table-driven implementation of

@@ -278,10 +278,10 @@ __global__ void __launch_bounds__(kPredFixNT, 4) k_pred_fix(PredArgs a) {
     __shared__ unsigned s_ymax;
     __shared__ __align__(8) uint64_t s_mb[8];
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    const double D = a.th.diag, ratio = a.th.diag_ratio, isd = a.th.diag_rsqrt;
-    const uint64_t rf = (uint64_t)__double2ull_rn(ratio * 0x1p63);
+    const double D = a.th.diag, isd = a.th.diag_rsqrt;
+    const uint64_t ratio = a.th.diag_ratio;
     for (int j = tid; j < 256; j += NT) {
-        tA[j] = bvfix::mulhi64(a.fixtab[j], rf) << 1;
+        tA[j] = bvfix::mulhi64(a.fixtab[j], ratio) << 1;
         tB[j] = a.fixtab[256 + j];
     }
     if (tid < 8)
