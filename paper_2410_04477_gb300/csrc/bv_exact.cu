@@ -16,7 +16,7 @@
 //                on a stream of higher priority beside the update of the rest
 // The factor's row n is z = L^-1 y, so y^T Sigma^-1 y = |z|^2 and log|Sigma| is the sum of the
 // pivots' logarithms.  The data row is scaled by a power of two; should a solved entry leave
-// the fixed-point range, the factorisation is done again with a larger one.
+// the fixed-point range, or the squares sum to more than 16, the factorisation is done again with a larger one.
 #include <cuda_runtime.h>
 #include <math.h>
 #include <stdint.h>
@@ -131,11 +131,11 @@ __global__ void __launch_bounds__(128) k_ex_diag(ExArgs a, int P) {
         const int64_t k0 = 16ll * (I0 + p);
         const int nc = (int)min((int64_t)16, a.n - k0), rows = (tr - p - 1) << 4, ry = (int)min(a.n - k0, (int64_t)1 << 20);
         if (warp == 0) {
-            fix_diag(tiles + ftile(p, p) * 128, nc, 0, ry, lane, Ld, rsv, a.piv + k0, a.zrow + k0, mb, flags);
+            fix_diag(tiles + ftile(p, p) * 128, nc, 0, ry, 1, lane, Ld, rsv, a.piv + k0, a.zrow + k0, mb, flags);
         } else if (tid - 32 < rows) {
             const int rw = tid - 32, i = p + 1 + (rw >> 4);
-            fix_row(tiles + ftile(i, p) * 128, Ld, rsv, rw & 15, 16 * (i - p) + (rw & 15) == ry, a.zrow + k0, nc, true, mb,
-                    p & 1, dig + (rw >> 4) * (kDigB / 4), flags);
+            fix_row(tiles + ftile(i, p) * 128, Ld, rsv, rw & 15, 16 * (i - p) + (rw & 15) == ry, 1, a.zrow + k0, nc, true,
+                    mb, p & 1, dig + (rw >> 4) * (kDigB / 4), flags);
         }
         __syncthreads();
         for (int j = tid; j < kLdN; j += 128) a.Ld[p * kLdN + j] = Ld[j];
@@ -179,7 +179,7 @@ __global__ void __launch_bounds__(128) k_ex_rows(ExArgs a, int P) {
         const int64_t k0 = 16ll * (I0 + s);
         const int nc = (int)min((int64_t)16, a.n - k0);
         if ((lane >> 4) < nI)
-            fix_row(a.A + etile(I, I0 + s), Ld + s * kLdN, rsv + s * 16, lane & 15, 16ll * I + (lane & 15) == a.n, a.zrow + k0,
+            fix_row(a.A + etile(I, I0 + s), Ld + s * kLdN, rsv + s * 16, lane & 15, 16ll * I + (lane & 15) == a.n, 1, a.zrow + k0,
                     nc, false, nullptr, 0, dw + (lane >> 4) * (kDigB / 4), flags);
         __syncwarp();
         for (int i = 0; i < nI; ++i) {
@@ -356,7 +356,7 @@ extern "C" int bv_exact_loglik(bv_ctx* c, const bv_theta* theta, int32_t use_y, 
         BV_CUDA(cudaMemcpyAsync(&h.ymax, a.flags + 1, sizeof(unsigned), cudaMemcpyDeviceToHost, st));
         BV_CUDA(cudaStreamSynchronize(st));
         const int ye = (int)(h.ymax >> 20);
-        E = (ye > 0 ? ye - 1022 : -1021) + kYRoom;
+        E = (ye > 0 ? ye - 1022 : -1021) + kYRoom + 1;
     }
     const bool valid = th.diag > 0.0 && th.diag < INFINITY && (int)(h.ymax >> 20) != 0x7ff;
     const int np = (a.TC + kP - 1) / kP, nb = (a.T + kP - 1) / kP;
@@ -392,6 +392,10 @@ extern "C" int bv_exact_loglik(bv_ctx* c, const bv_theta* theta, int32_t use_y, 
         BV_CUDA(cudaGetLastError());
         BV_CUDA(cudaMemcpyAsync(&h, terms, sizeof(double) * 2 + sizeof(int), cudaMemcpyDeviceToHost, st));
         BV_CUDA(cudaStreamSynchronize(st));
+        // the data row's Schur complements are below 2^-5 + |z| in units of 2^E sqrt(D); while the
+        // squares sum to at most 16 none has left the range of +-8 (an entry that had would have
+        // come after entries whose squares sum to more)
+        if (!(h.term[1] <= ldexp(16.0, 2 * E))) h.flags |= kOver;
         if (!(h.flags & kOver) || (h.flags & kFail) || pass == 12) break;
         E += kYStep;
     }

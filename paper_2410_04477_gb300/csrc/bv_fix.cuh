@@ -142,6 +142,16 @@ BV_FIX int64_t sub_square(int64_t a, int64_t x, int32_t h) {
     return smad(-h, h, a) - (smad(h, l, smad(lq, lq, 1ll << 27)) >> 28);
 }
 
+// Largest size of a solved data entry, as a power of two: below 2^-row_limit(N).  A row of the
+// factor has a norm of at most 1, so the data row's Schur complements stay below 2^-5 + sqrt(N)
+// 2^-row_limit(N) < 4.1, in the range of +-8 of a 64-bit entry in matrix units (and entries below
+// 1/2 keep the digits' sums in range).
+BV_FIX int row_limit(int n) {
+    int g = 1;
+    while (n > 16 << (2 * g)) ++g;
+    return g;
+}
+
 // 1 / sqrt(P), P = p 2^-60, for p in [1, 2^60]: r 2^(e - 62) with r in [2^62, 2^63) and e >= 0,
 // within 2^-59 relative and exact for P = 1.  The hardware seed's mantissa Y (24 bits, error
 // 2^-22) takes a Newton step with the second-order term in fixed point, which cubes its error.

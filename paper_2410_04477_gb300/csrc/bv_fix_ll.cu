@@ -119,7 +119,7 @@ __global__ void __launch_bounds__(NT, WARPS * 32 / NT) k_ll_fix(LLArgs a) {
         __syncthreads();
         const int ye = (int)(s_ymax >> 20);
         const bool valid = D > 0.0 && D < INFINITY && ye != 0x7ff;
-        int E = (ye > 0 ? ye - 1022 : -1021) + kYRoom;  // |y| 2^-E < 2^-kYRoom
+        int E = (ye > 0 ? ye - 1022 : -1021) + kYRoom + bvfix::row_limit(N);
 
         bool fail = false;
         int64_t* yfix = reinterpret_cast<int64_t*>(yv);

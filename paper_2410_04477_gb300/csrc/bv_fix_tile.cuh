@@ -25,8 +25,9 @@ constexpr int kDig = 6;        // digits of a factor entry
 constexpr int kLd = 24;            // entries of a diagonal factor's column (16, then zeros)
 constexpr int kDigB = kDig * 512;  // bytes of a tile's digits
 constexpr int kFail = 1, kOver = 2;  // a thread's findings about the block
-// The data row's headroom: |y| / sqrt(D) < 2^-kYRoom at first, 2^-kYStep less a pass after.
-constexpr int kYRoom = 5, kYStep = 8;
+// The data row's headroom: |y| / sqrt(D) < 2^-(kYRoom + row_limit(N)) at first, so that a solved entry
+// may be 2^kYRoom / 2 of the largest |y| / sqrt(D), and 2^-kYStep less a pass after.
+constexpr int kYRoom = 4, kYStep = 8;
 // A pivot of at most this (2^-54 of the diagonal, below one FP64 rounding of it) counts as not
 // positive: what a singular matrix leaves is noise of this size, of either sign.
 constexpr int64_t kPivMin = 64;
@@ -71,7 +72,8 @@ struct __align__(16) FixRs {
     int pad;
 };
 
-__device__ __forceinline__ bool out_of_range(int64_t v, int e) { return ((v < 0 ? -v : v) >> (59 - e)) != 0; }
+// A solved data entry x = v 2^e r, r in [1, 2), is below 2^-lim when v 2^e is below half of that.
+__device__ __forceinline__ bool out_of_range(int64_t v, int e, int lim) { return ((v < 0 ? -v : v) >> (59 - lim - e)) != 0; }
 
 // The diagonal factor in shared memory: column c's entries L[j][c] at c kLd + j.  The loops
 // below read past j = 15, where the row loop needs zeros.
@@ -107,7 +109,7 @@ __device__ __forceinline__ bool pair_wait(uint64_t* mb, uint32_t parity) {
 // code stays small: unrolled over the 16 columns, this and the row loop below ran at the rate
 // of instruction fetches (10,000 clocks a tile and a row pass).  The pivots and the data row's
 // entries (row N, if it lies in the tile) are stored.
-__device__ __forceinline__ void fix_diag(const longlong2* tile, int nc, int k0, int N, int lane, int4* Ld, FixRs* rsv,
+__device__ __forceinline__ void fix_diag(const longlong2* tile, int nc, int k0, int N, int lim, int lane, int4* Ld, FixRs* rsv,
                                          int64_t* piv, int64_t* zrow, uint64_t* mb, int& flags) {
     const int r = lane & 15, par = lane >> 4;
     int64_t a[8];  // columns 2 (k + q) + par in turn k
@@ -154,7 +156,7 @@ __device__ __forceinline__ void fix_diag(const longlong2* tile, int nc, int k0, 
                 Ld[c * kLd + r] = make_int4(f.h, __float_as_int(f.hf), __float_as_int(f.lf), 0);
                 if (r == ry && on) {
                     zrow[k0 + c] = x;
-                    if (out_of_range(v, rs.e)) flags |= kOver;
+                    if (out_of_range(v, rs.e, lim)) flags |= kOver;
                 }
             }
             if (lane == 0) {
@@ -183,7 +185,7 @@ __device__ __forceinline__ void fix_diag(const longlong2* tile, int nc, int k0, 
 // wait, the columns come in pairs from the warp at work on the diagonal tile.
 template <int W>
 __device__ __forceinline__ void fix_row4(int64_t* a, float* fc, int c0, const int4* Ld, const FixRs* rsv, bool yrow,
-                                         int64_t* z, int nc, bool wait, uint64_t* mb, uint32_t parity, int& flags) {
+                                         int lim, int64_t* z, int nc, bool wait, uint64_t* mb, uint32_t parity, int& flags) {
 #pragma unroll 1
     for (int c = c0; c < c0 + 4; ++c) {
         if (wait && !(c & 1) && !pair_wait(mb + (c >> 1), parity)) flags |= kFail;
@@ -203,14 +205,14 @@ __device__ __forceinline__ void fix_row4(int64_t* a, float* fc, int c0, const in
         fc[W - 1] = 0.0f;
         if (yrow && c < nc) {
             z[c] = x;
-            if (out_of_range(v, rs.e)) flags |= kOver;
+            if (out_of_range(v, rs.e, lim)) flags |= kOver;
         }
     }
 }
 
 // One row of the panel below the diagonal tile: x L^T = a, then its digits.
-__device__ __forceinline__ void fix_row(const longlong2* tile, const int4* Ld, const FixRs* rsv, int r, bool yrow, int64_t* z,
-                                        int nc, bool wait, uint64_t* mb, uint32_t parity, uint32_t* dig, int& flags) {
+__device__ __forceinline__ void fix_row(const longlong2* tile, const int4* Ld, const FixRs* rsv, int r, bool yrow, int lim,
+                                        int64_t* z, int nc, bool wait, uint64_t* mb, uint32_t parity, uint32_t* dig, int& flags) {
     const int g = r & 7, rr = r >> 3;
     int64_t a[16];
     float fc[16];
@@ -221,10 +223,10 @@ __device__ __forceinline__ void fix_row(const longlong2* tile, const int4* Ld, c
         a[2 * q + 1] = v.y;
         fc[2 * q] = fc[2 * q + 1] = 0.0f;
     }
-    fix_row4<16>(a, fc, 0, Ld, rsv, yrow, z, nc, wait, mb, parity, flags);   // a: columns 4 .. 15, x of 0 .. 3
-    fix_row4<12>(a, fc, 4, Ld, rsv, yrow, z, nc, wait, mb, parity, flags);   // columns 8 .. 15, x of 4 .. 7, 0 .. 3
-    fix_row4<8>(a, fc, 8, Ld, rsv, yrow, z, nc, wait, mb, parity, flags);
-    fix_row4<4>(a, fc, 12, Ld, rsv, yrow, z, nc, wait, mb, parity, flags);   // x of 12 .. 15, 8 .. 11, 4 .. 7, 0 .. 3
+    fix_row4<16>(a, fc, 0, Ld, rsv, yrow, lim, z, nc, wait, mb, parity, flags);   // a: columns 4 .. 15, x of 0 .. 3
+    fix_row4<12>(a, fc, 4, Ld, rsv, yrow, lim, z, nc, wait, mb, parity, flags);   // columns 8 .. 15, x of 4 .. 7, 0 .. 3
+    fix_row4<8>(a, fc, 8, Ld, rsv, yrow, lim, z, nc, wait, mb, parity, flags);
+    fix_row4<4>(a, fc, 12, Ld, rsv, yrow, lim, z, nc, wait, mb, parity, flags);   // x of 12 .. 15, 8 .. 11, 4 .. 7, 0 .. 3
     // digits: x + 512 sum 2^10k has the digits plus 512 in six ten-bit fields; 1024 + field
     // is the FP16 number 0x6400 + field.  Word i of a row: columns 2 i, 2 i + 1 (the order of
     // the columns inside a product's sum is free).
@@ -259,9 +261,11 @@ __device__ __forceinline__ void fix_row(const longlong2* tile, const int4* Ld, c
 // The sum of the digit products of one entry (orders 0 .. 5: units 2^-18 .. 2^-68; f6: what is
 // added in units of order 5) in matrix units.  FAST: the FP32 whole numbers f become integers
 // kB + f by adding 1.5 2^23 (a quarter of a clock each, a conversion takes two); right while all
-// are below 2^22 in size, else *wide shows bits above.  Orders 0 and 1 are that small by the
-// rows' norms (at most 1, and 16 entries of 0.71 in the data row), so only the others are looked
-// at.  The weights are multiply-adds on the FMA pipe, the offsets kB one constant: the ALU is
+// are below 2^22 in size, else *wide shows bits above.  Orders 0 and 1 are that small: of two rows
+// of norm 1 (first digits of norm 514 with their rounding, second ones up to 512 each) at most
+// 514^2 and 2 x 512 x 4 x 514 < 2^21.1; of a row and the data row, whose entries are below 1/2 (first
+// digits up to 256), at most 4 x 256 x 514 and 16 x 256 x 512 + 512 x 4 x 514 < 2^21.6.  So only the
+// others are looked at.  The weights are multiply-adds on the FMA pipe, the offsets kB one constant: the ALU is
 // what bounds the update.
 template <bool FAST>
 __device__ __forceinline__ int64_t digit_sum(const float (&f)[kDig], uint32_t f6, uint32_t& wide) {
@@ -421,18 +425,18 @@ __device__ __forceinline__ void fix_fill(longlong2* tp, int I, int J, int m, int
 template <int NT>
 __device__ __forceinline__ int fix_panels(longlong2* tiles, int T, int TC, int NP, int N, uint32_t* dig, int4* Ld, FixRs* rsv,
                                           int64_t* piv, int64_t* zrow, uint64_t* mb, uint32_t& parity, int& flags) {
-    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, lim = bvfix::row_limit(N);
 #pragma unroll 1
     for (int p = 0; p < NP; ++p) {
         const int k0 = p << 4, nc = min(16, N - k0), rows = (T - p - 1) << 4;
         if (warp == 0) {
-            fix_diag(tiles + ftile(p, p) * 128, nc, k0, N, lane, Ld, rsv, piv, zrow, mb, flags);
+            fix_diag(tiles + ftile(p, p) * 128, nc, k0, N, lim, lane, Ld, rsv, piv, zrow, mb, flags);
         } else {
 #pragma unroll 1
             for (int rw = tid - 32; rw < rows; rw += NT - 32) {
                 const int I = p + 1 + (rw >> 4);
-                fix_row(tiles + ftile(I, p) * 128, Ld, rsv, rw & 15, (I << 4) + (rw & 15) == N, zrow + k0, nc, rw < NT - 32, mb,
-                        parity, dig + (rw >> 4) * (kDigB / 4), flags);
+                fix_row(tiles + ftile(I, p) * 128, Ld, rsv, rw & 15, (I << 4) + (rw & 15) == N, lim, zrow + k0, nc, rw < NT - 32,
+                        mb, parity, dig + (rw >> 4) * (kDigB / 4), flags);
             }
         }
         parity ^= 1;

@@ -267,8 +267,7 @@ __global__ void __launch_bounds__(kPredNT) k_pred(PredArgs a) {
 // k_pred spends its time on the FP64 pipe (2 lanes a clock and SM); this one uses the integer
 // pipe and the tensor cores: 2,000 blocks of m = 120 and 10 sites in
 // 0.79 ms, before 2.8.  Tiles in a global-memory slot of the CTA.  The mean is left by the
-// elimination at the data row's scale, so a block is done again with a larger one when a solved
-// entry or the sum of their squares (above 16: the mean could leave the range) is too large.
+// elimination at the data row's scale; the limit of its solved entries keeps it in range.
 constexpr int kPredFixNT = 128;
 template <bool GEN>
 __global__ void __launch_bounds__(kPredFixNT, 4) k_pred_fix(PredArgs a) {
@@ -319,7 +318,7 @@ __global__ void __launch_bounds__(kPredFixNT, 4) k_pred_fix(PredArgs a) {
         if (lane == 0) atomicMax(&s_ymax, ym);
         __syncthreads();
         const int ye = (int)(s_ymax >> 20);
-        int E = (ye > 0 ? ye - 1022 : -1021) + kYRoom;
+        int E = (ye > 0 ? ye - 1022 : -1021) + kYRoom + bvfix::row_limit(N);
         const bool valid = D > 0.0 && D < INFINITY && ye != 0x7ff;
         bool failed = false;
         for (int pass = 0;; ++pass) {
@@ -338,19 +337,6 @@ __global__ void __launch_bounds__(kPredFixNT, 4) k_pred_fix(PredArgs a) {
             }
             int stop = __syncthreads_or(flags);
             if (!stop) stop = fix_panels<NT>(tiles, T, TC, m16 >> 4, N, dig, Ld, rsv, piv, zrow, s_mb, parity, flags);
-            if (!stop) {
-                if (warp == 0) {
-                    float s = 0.0f;
-                    for (int k = lane; k < m16; k += 32) {
-                        const float z = (float)zrow[k] * 1.734723475976807e-18f;  // 2^-59
-                        s = fmaf(z, z, s);
-                    }
-#pragma unroll
-                    for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-                    if (!(s <= 16.0f)) flags |= kOver;
-                }
-                stop = __syncthreads_or(flags);
-            }
             failed = stop && __syncthreads_or(flags & kFail);
             if (failed || !stop) break;
             if (pass == 12) {
