@@ -30,6 +30,7 @@
 
 namespace {
 
+constexpr int kExStep = 8, kExPasses = 13;                // the data row's scalings (a pass each)
 constexpr int kP = 4;                                     // tiles of a panel
 constexpr int kLdN = 16 * kLd + 16;                       // entries of a tile's factor in memory
 
@@ -396,8 +397,8 @@ extern "C" int bv_exact_loglik(bv_ctx* c, const bv_theta* theta, int32_t use_y, 
         // squares sum to at most 16 none has left the range of +-8 (an entry that had would have
         // come after entries whose squares sum to more)
         if (!(h.term[1] <= ldexp(16.0, 2 * E))) h.flags |= kOver;
-        if (!(h.flags & kOver) || (h.flags & kFail) || pass == 12) break;
-        E += kYStep;
+        if (!(h.flags & kOver) || (h.flags & kFail) || pass + 1 == kExPasses) break;
+        E += kExStep;
     }
     if (!valid || h.flags) {
         if (out_loglik) *out_loglik = -INFINITY;

@@ -16,9 +16,9 @@
 //                <= 5 are taken (the pairs of order 4 and 5, five and six to a sum, could
 //                round in the last bit only on sums that real digits do not reach, by one
 //                unit of 2^-58); what is left out is below 2^-57 of 1.
-// The data row is scaled by a power of two so that |y| / sqrt(D) stays below 2^-5; if a
-// solved entry leaves the range, the block is done again with a larger power (an outlier
-// more than 2^5 conditional standard deviations above the largest observation).
+// The data row is scaled by a power of two that leaves solved entries room for 16 times the
+// largest |y| / sqrt(D); where one is larger (the parameters are far from the data's), the row is
+// scaled further and the panel solved again.
 //
 // Against a 113-bit factorisation of the same scaled coordinates, the blocks' ell errs by
 // 8.4e-13 (RMS; n = 20,000, m = 60, nu = 3/2, tau^2 = 1e-4), FP64 arithmetic by 2.8e-12; at m =
@@ -121,37 +121,25 @@ __global__ void __launch_bounds__(NT, WARPS * 32 / NT) k_ll_fix(LLArgs a) {
         const bool valid = D > 0.0 && D < INFINITY && ye != 0x7ff;
         int E = (ye > 0 ? ye - 1022 : -1021) + kYRoom + bvfix::row_limit(N);
 
-        bool fail = false;
         int64_t* yfix = reinterpret_cast<int64_t*>(yv);
-        // again with a larger E when a solved data entry leaves the range (a finite z needs a
-        // few passes at most; the data row is 0 after 9)
+        int flags = valid ? 0 : kFail;
 #pragma unroll 1
-        for (int pass = 0;; ++pass) {
-            int flags = valid ? 0 : kFail;
+        for (int t = tid; t < N; t += NT) yfix[t] = __double2ll_rn(bvfix::scale2(yv[t], bvfix::kUnitC - E));
+        __syncthreads();
+        const int ntile = (T * (T + 1)) >> 1;
 #pragma unroll 1
-            for (int t = tid; t < N; t += NT) {
-                const double y = pass == 0 ? yv[t] : bvfix::scale2((double)yfix[t], E - kYStep - bvfix::kUnitC);
-                yfix[t] = __double2ll_rn(bvfix::scale2(y, bvfix::kUnitC - E));
-            }
-            __syncthreads();
-            const int ntile = (T * (T + 1)) >> 1;
-#pragma unroll 1
-            for (int q = warp; q < ntile; q += NW) {
-                int I, J;
-                tri_rc(q, I, J);
-                if (J >= TC) continue;
-                fix_fill<GEN ? 1 : 0, false>(tiles + q * 128, I, J, N, N, N, lane, px, d, yfix, a.theta + ds, th.nu_code, ratio,
-                                             a.gtabi + (int64_t)ds * GTAB_SIZE, tA, tB, flags);
-            }
-            int stop = __syncthreads_or(flags);
-            if (!stop) stop = fix_panels<NT>(tiles, T, TC, TC, N, dig, Ld, rsv, piv, zrow, s_mb, parity, flags);
-            fail = stop && __syncthreads_or(flags & kFail);
-            if (fail || !stop) break;
-            if (pass == 12) {
-                fail = true;
-                break;
-            }
-            E += kYStep;
+        for (int q = warp; q < ntile; q += NW) {
+            int I, J;
+            tri_rc(q, I, J);
+            if (J >= TC) continue;
+            fix_fill<GEN ? 1 : 0, false>(tiles + q * 128, I, J, N, N, N, lane, px, d, yfix, a.theta + ds, th.nu_code, ratio,
+                                         a.gtabi + (int64_t)ds * GTAB_SIZE, tA, tB, flags);
+        }
+        bool fail = __syncthreads_or(flags);
+        if (!fail) {
+            const int scaled = fix_panels<NT>(tiles, T, TC, TC, N, dig, Ld, rsv, piv, zrow, s_mb, parity);
+            fail = scaled < 0;
+            E += kYStep * scaled;
         }
 
         if (warp == 0) {

@@ -26,8 +26,9 @@ constexpr int kLd = 24;            // entries of a diagonal factor's column (16,
 constexpr int kDigB = kDig * 512;  // bytes of a tile's digits
 constexpr int kFail = 1, kOver = 2;  // a thread's findings about the block
 // The data row's headroom: |y| / sqrt(D) < 2^-(kYRoom + row_limit(N)) at first, so that a solved entry
-// may be 2^kYRoom / 2 of the largest |y| / sqrt(D), and 2^-kYStep less a pass after.
-constexpr int kYRoom = 4, kYStep = 8;
+// may be 2^kYRoom / 2 of the largest |y| / sqrt(D).  When one is larger, the row is scaled down by
+// 2^kYStep, kYMax times at most (beyond any ratio that the pivots leave).
+constexpr int kYRoom = 5, kYStep = 8, kYMax = 16;
 // A pivot of at most this (2^-54 of the diagonal, below one FP64 rounding of it) counts as not
 // positive: what a singular matrix leaves is noise of this size, of either sign.
 constexpr int64_t kPivMin = 64;
@@ -417,18 +418,40 @@ __device__ __forceinline__ void fix_fill(longlong2* tp, int I, int J, int m, int
     }
 }
 
+__device__ __forceinline__ int64_t y_step(int64_t v) { return (v + (1ll << (kYStep - 1))) >> kYStep; }
+
+// The data row (row N) from tile column p on, and the solved entries of the columns before, times
+// 2^-kYStep.
+template <int NT>
+__device__ __noinline__ void fix_rescale(longlong2* tiles, int p, int TC, int N, int64_t* zrow) {
+    const int tid = threadIdx.x, I = N >> 4, r = N & 15;
+    const int cnt = (min(I + 1, TC) - p) << 3;
+#pragma unroll 1
+    for (int i = tid; i < cnt; i += NT) {
+        const int q = i & 7;
+        longlong2* e = tiles + ftile(I, p + (i >> 3)) * 128 + ((q >> 2) * 2 + (r >> 3)) * 32 + 4 * (r & 7) + (q & 3);
+        const longlong2 v = *e;
+        *e = make_longlong2(y_step(v.x), y_step(v.y));
+    }
+#pragma unroll 1
+    for (int k = tid; k < 16 * p; k += NT) zrow[k] = y_step(zrow[k]);
+}
+
 // Eliminate the first NP panels of 16 columns of the T x T tiles (rows 0 .. N, row N the data
 // row; TC tile columns of points) by one CTA.  Warp 0 factors a panel's diagonal tile; the
 // other warps follow it, two columns behind, on the rows below, one row a thread (rows beyond
-// one a thread, in the largest blocks, after that); then all update the trailing tiles.  Ends
-// at a bad pivot or a data entry out of range: non-zero then, each thread's findings in flags.
+// one a thread, in the largest blocks, after that); then all update the trailing tiles.  A data
+// entry out of range scales the data row down and the panel, whose tiles are as they were, is
+// solved again.  Returns the scalings, or -1 at a bad pivot (or more than kYMax scalings).
 template <int NT>
 __device__ __forceinline__ int fix_panels(longlong2* tiles, int T, int TC, int NP, int N, uint32_t* dig, int4* Ld, FixRs* rsv,
-                                          int64_t* piv, int64_t* zrow, uint64_t* mb, uint32_t& parity, int& flags) {
+                                          int64_t* piv, int64_t* zrow, uint64_t* mb, uint32_t& parity) {
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, lim = bvfix::row_limit(N);
+    int scaled = 0;
 #pragma unroll 1
     for (int p = 0; p < NP; ++p) {
         const int k0 = p << 4, nc = min(16, N - k0), rows = (T - p - 1) << 4;
+        int flags = 0;
         if (warp == 0) {
             fix_diag(tiles + ftile(p, p) * 128, nc, k0, N, lim, lane, Ld, rsv, piv, zrow, mb, flags);
         } else {
@@ -440,7 +463,12 @@ __device__ __forceinline__ int fix_panels(longlong2* tiles, int T, int TC, int N
             }
         }
         parity ^= 1;
-        if (__syncthreads_or(flags)) return 1;
+        if (__syncthreads_or(flags)) {
+            if (__syncthreads_or(flags & kFail) || ++scaled > kYMax) return -1;
+            fix_rescale<NT>(tiles, p--, TC, N, zrow);
+            __syncthreads();
+            continue;
+        }
         const int S = T - p - 1, cnt = (S * (S + 1)) >> 1;
 #pragma unroll 1
         for (int q = warp; q < cnt; q += NT / 32) {
@@ -452,7 +480,7 @@ __device__ __forceinline__ int fix_panels(longlong2* tiles, int T, int TC, int N
         }
         __syncthreads();
     }
-    return 0;
+    return scaled;
 }
 
 }  // namespace

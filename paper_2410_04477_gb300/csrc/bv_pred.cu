@@ -320,30 +320,21 @@ __global__ void __launch_bounds__(kPredFixNT, 4) k_pred_fix(PredArgs a) {
         const int ye = (int)(s_ymax >> 20);
         int E = (ye > 0 ? ye - 1022 : -1021) + kYRoom + bvfix::row_limit(N);
         const bool valid = D > 0.0 && D < INFINITY && ye != 0x7ff;
-        bool failed = false;
-        for (int pass = 0;; ++pass) {
-            int flags = valid ? 0 : kFail;
-            for (int t = tid; t < N; t += NT) {
-                const double y = pass == 0 ? yv[t] : bvfix::scale2((double)yfix[t], E - kYStep - bvfix::kUnitC);
-                yfix[t] = __double2ll_rn(bvfix::scale2(y, bvfix::kUnitC - E));
-            }
-            __syncthreads();
-            for (int q = warp; q < ((T * (T + 1)) >> 1); q += NT / 32) {
-                int I, J;
-                tri_rc(q, I, J);
-                if (J >= TC) continue;
-                fix_fill<GEN ? 2 : 0, true>(tiles + q * 128, I, J, m, m16, N, lane, px, d, yfix, &a.th, a.th.nu_code, ratio,
-                                            nullptr, tA, tB, flags);
-            }
-            int stop = __syncthreads_or(flags);
-            if (!stop) stop = fix_panels<NT>(tiles, T, TC, m16 >> 4, N, dig, Ld, rsv, piv, zrow, s_mb, parity, flags);
-            failed = stop && __syncthreads_or(flags & kFail);
-            if (failed || !stop) break;
-            if (pass == 12) {
-                failed = true;
-                break;
-            }
-            E += kYStep;
+        int flags = valid ? 0 : kFail;
+        for (int t = tid; t < N; t += NT) yfix[t] = __double2ll_rn(bvfix::scale2(yv[t], bvfix::kUnitC - E));
+        __syncthreads();
+        for (int q = warp; q < ((T * (T + 1)) >> 1); q += NT / 32) {
+            int I, J;
+            tri_rc(q, I, J);
+            if (J >= TC) continue;
+            fix_fill<GEN ? 2 : 0, true>(tiles + q * 128, I, J, m, m16, N, lane, px, d, yfix, &a.th, a.th.nu_code, ratio, nullptr,
+                                        tA, tB, flags);
+        }
+        bool failed = __syncthreads_or(flags);
+        if (!failed) {
+            const int scaled = fix_panels<NT>(tiles, T, TC, m16 >> 4, N, dig, Ld, rsv, piv, zrow, s_mb, parity);
+            failed = scaled < 0;
+            E += kYStep * scaled;
         }
         const auto entry = [&](int r, int c) {
             const longlong2 v = tiles[ftile(r >> 4, c >> 4) * 128 + (((c >> 3) & 1) * 2 + ((r >> 3) & 1)) * 32 + 4 * (r & 7) + ((c & 7) >> 1)];
