@@ -423,7 +423,7 @@ __device__ __forceinline__ int64_t y_step(int64_t v) { return (v + (1ll << (kYSt
 // The data row (row N) from tile column p on, and the solved entries of the columns before, times
 // 2^-kYStep.
 template <int NT>
-__device__ __noinline__ void fix_rescale(longlong2* tiles, int p, int TC, int N, int64_t* zrow) {
+__device__ __forceinline__ void fix_rescale(longlong2* tiles, int p, int TC, int N, int64_t* zrow) {
     const int tid = threadIdx.x, I = N >> 4, r = N & 15;
     const int cnt = (min(I + 1, TC) - p) << 3;
 #pragma unroll 1
