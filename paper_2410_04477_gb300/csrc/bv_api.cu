@@ -787,7 +787,7 @@ static const int kBinEdges[] = {16, 32, 48, 64, 80, 96, 112, 128, 160, 192, 224,
 // CTA sizes: the mixed kernel's one panel warp plus 2, 4, 8 or 16 update warps.
 static int default_threads(const bv_ctx* c, int kind, int nmax, int nwork) {
     if (kind == 2) return 256;
-    if (kind >= 7) return bv_fix_threads(nmax, nwork, c->num_sms);
+    if (kind >= 7) return bv_fix_threads(kind, nmax, nwork, c->num_sms);
     if (nmax <= 48) return 96;
     if (nmax <= 128) return 160;
     return 288;
@@ -923,7 +923,7 @@ static int build_check(bv_ctx* c, const std::vector<int>& Nof) {
         int nmax = 0;
         for (int32_t i : all[b]) nmax = std::max(nmax, Nof[i]);
         bp.nmax = nmax;
-        bp.kind = b < edges.size() ? bv_fix_kind(nmax, c->d) : 2;
+        bp.kind = b < edges.size() ? bv_fix_kind(nmax, (int)c->nblk, c->num_sms, c->d) : 2;
         // redo launch: the whole bin's capacity, count from the device
         bp.nwork = (int32_t)all[b].size();
         bp.threads = default_threads(c, bp.kind, bp.nmax, bp.nwork);
@@ -1035,7 +1035,7 @@ int bv_ensure_plan(bv_ctx* c, int prec) {
         BinPlan bp;
         bp.d_ctr = nullptr;
         bp.nmax = Nof[L.front()];
-        bp.kind = b >= edges.size() ? 2 : fix ? bv_fix_kind(bp.nmax, c->d) : 1;
+        bp.kind = b >= edges.size() ? 2 : fix ? bv_fix_kind(bp.nmax, (int)c->nblk, c->num_sms, c->d) : 1;
         bp.nwork = (int32_t)L.size();
         bp.threads = default_threads(c, bp.kind, bp.nmax, bp.nwork);
         bp.h_work = L;
@@ -1119,7 +1119,12 @@ static int autotune(bv_ctx* c, int prec) {
                             c->stream));
     BV_CUDA(bv_launch_fail_reset(c->d_fail, c->stream));
     for (auto& bp : c->plan[prec]) {
-        if (bp.kind != 1) continue;  // one form each
+        if (bp.kind != 1) {  // one form each
+            if (getenv("BV_LOG_PLAN"))
+                fprintf(stderr, "[bv plan] prec %d bin nmax %d nwork %d -> kind %d threads %d grid %d smem %zu\n", prec, bp.nmax,
+                        bp.nwork, bp.kind, bp.threads, bp.grid, bp.smem);
+            continue;
+        }
         // candidates: CTA per block with 1 panel warp + 2/4/8/16 update warps; up to N = 128
         // also a warp per block with 2/4/8 warps per CTA; from N = 64 on also the tensor-core
         // kernel.  BV_KERNEL_FORM=cta, =warp or =tc restricts the choice to one form where it

@@ -132,7 +132,7 @@ __global__ void __launch_bounds__(128) k_ex_diag(ExArgs a, int P) {
         const int64_t k0 = 16ll * (I0 + p);
         const int nc = (int)min((int64_t)16, a.n - k0), rows = (tr - p - 1) << 4, ry = (int)min(a.n - k0, (int64_t)1 << 20);
         if (warp == 0) {
-            fix_diag(tiles + ftile(p, p) * 128, nc, 0, ry, 1, lane, Ld, rsv, a.piv + k0, a.zrow + k0, mb, flags);
+            fix_diag<false>(tiles + ftile(p, p) * 128, nc, 0, ry, 1, lane, Ld, rsv, a.piv + k0, a.zrow + k0, mb, flags);
         } else if (tid - 32 < rows) {
             const int rw = tid - 32, i = p + 1 + (rw >> 4);
             fix_row(tiles + ftile(i, p) * 128, Ld, rsv, rw & 15, 16 * (i - p) + (rw & 15) == ry, 1, a.zrow + k0, nc, true,

@@ -56,14 +56,17 @@ namespace {
 template <int NT, bool GEN, bool GLOB, int WARPS>
 __global__ void __launch_bounds__(NT, WARPS * 32 / NT) k_ll_fix(LLArgs a) {
     extern __shared__ __align__(16) unsigned char smraw[];
-    __shared__ uint64_t tA[256], tB[256];
+    __shared__ uint64_t tA[256], tBs[NT == 32 ? 1 : 256];  // (one-warp CTAs: as many as fit count more)
     __shared__ int s_w;
     __shared__ unsigned s_ymax;  // largest high word of |y| / sqrt(D)
     __shared__ __align__(8) uint64_t s_mb[8];
     constexpr int NW = NT / 32;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    if (NT > 32) {
 #pragma unroll 1
-    for (int j = tid; j < 256; j += NT) tB[j] = a.fixtab[256 + j];
+        for (int j = tid; j < 256; j += NT) tBs[j] = a.fixtab[256 + j];
+    }
+    const uint64_t* tB = NT > 32 ? tBs : a.fixtab + 256;
     const int nwork = work_count(a);
     if (tid < 8)
         asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"((uint32_t)__cvta_generic_to_shared(s_mb + tid)) : "memory");
@@ -132,7 +135,7 @@ __global__ void __launch_bounds__(NT, WARPS * 32 / NT) k_ll_fix(LLArgs a) {
             int I, J;
             tri_rc(q, I, J);
             if (J >= TC) continue;
-            fix_fill<GEN ? 1 : 0, false>(tiles + q * 128, I, J, N, N, N, lane, px, d, yfix, a.theta + ds, th.nu_code, ratio,
+            fix_fill<GEN ? 1 : 0, false, NT == 32>(tiles + q * 128, I, J, N, N, N, lane, px, d, yfix, a.theta + ds, th.nu_code, ratio,
                                          a.gtabi + (int64_t)ds * GTAB_SIZE, tA, tB, flags);
         }
         bool fail = __syncthreads_or(flags);
@@ -167,6 +170,7 @@ template <bool GEN>
 FixKernel fix_kernel_g(int kind, int threads) {
     if (threads == 256) return kind == 7 ? k_ll_fix<256, GEN, false, 16> : k_ll_fix<256, GEN, true, 16>;
     if (kind == 7) return threads == 64 ? k_ll_fix<64, GEN, false, 20> : nullptr;
+    if (threads == 32) return k_ll_fix<32, GEN, true, 20>;
     if (threads != 128) return nullptr;
     return kind == 8 ? k_ll_fix<128, GEN, true, 20> : k_ll_fix<128, GEN, true, 16>;
 }
@@ -177,30 +181,39 @@ cudaError_t fix_kernel(int kind, int threads, bool gen, FixKernel* k) {
 
 }  // namespace
 
-// CTA size: one warp for the diagonal tiles, the others for the rows below, with which four
-// warps cover blocks up to N = 111 in one pass.  Blocks of up to three tile rows take two
-// warps, large ones eight.  A bin of few blocks (two an SM) takes eight as well: there a
-// block's latency counts, not the SM's rate.
-int bv_fix_threads(int nmax, int nwork, int num_sms) {
-    if (nwork <= 2 * num_sms) return 256;
-    return nmax <= 47 ? 64 : nmax <= 239 ? 128 : 256;
+// CTA size: one warp for the diagonal tiles, the others for the rows below, with which four warps cover
+// blocks up to N = 111 in one pass and large ones take eight.  A bin of few blocks (two an SM) takes eight
+// as well: there a block's latency counts, not the SM's rate.  Up to three tile rows with tiles in the
+// workspace (8): one warp for everything, up to 20 of them an SM.
+int bv_fix_threads(int kind, int nmax, int nwork, int num_sms) {
+    if (kind == 7) return nwork <= 2 * num_sms ? 256 : 64;
+    if (fix_tiles(nmax) <= 3) return 32;
+    return nwork > 2 * num_sms && nmax <= 239 ? 128 : 256;
 }
 
 size_t bv_fix_smem_bytes(int kind, int nmax, int d) {
     return fix_work_bytes(nmax, d) + (kind == 7 ? fix_tile_bytes(nmax) : 0);
 }
 
-// The kernel form of a bin of largest size nmax: tiles in shared memory (7) up to three tile
-// rows, in a workspace beyond, where four to eight CTAs an SM would not fit with them (8; 9 from
-// N = 112 on, with more registers); -1 when even the panel's digits do not fit.
-int bv_fix_kind(int nmax, int d) {
-    if (fix_tiles(nmax) <= 3) return 7;
+// The kernel form of a bin of largest size nmax: -1 when even the panel's digits do not fit; tiles in a
+// workspace (8; 9 from N = 112 on, with more registers), or, up to three tile rows, in shared memory (7)
+// when the evaluation has few blocks in all (total): then latency counts, and one kernel for all small
+// bins, since fetching a kernel's code takes some 13 us.  Many small blocks go to one-warp CTAs, since a
+// second warp mostly waits on the pivots and as many CTAs do not fit with their tiles: 50,000 blocks of N =
+// 8, 11, 18, 24, 31, 36, 47 take 0.37, 0.43, 1.00, 1.13, 1.25, 2.10, 2.40 ms (two warps and tiles in
+// shared memory: 0.74, 0.74, 1.50, 1.51, 1.53, 2.67, 2.69; FP64, a warp a block: 0.46, 0.59, 0.97, 1.45,
+// 2.18, 2.84, 4.78).  With fewer blocks an SM the second warp helps: up to 8 for N <= 24 (1,000 blocks of N
+// = 21: 105 us a call either way), some 20 beyond (3,000 blocks of N = 31: 160 us with one, 141 with two;
+// 2,000 of N = 47: 208 and 171).
+int bv_fix_kind(int nmax, int total, int num_sms, int d) {
+    const int T = fix_tiles(nmax);
+    if (T <= 3) return total <= (T == 1 ? 2 : nmax <= 24 ? 8 : 21) * num_sms ? 7 : 8;
     if (bv_fix_smem_bytes(8, nmax, d) > (size_t)kFixSmemCap) return -1;
     return nmax <= 111 ? 8 : 9;
 }
 int bv_fix_max_n(int d) {
     int n = 64;
-    while (bv_fix_kind(n + 1, d) > 0) ++n;
+    while (bv_fix_kind(n + 1, 0, 0, d) > 0) ++n;
     return n;
 }
 size_t bv_fix_slot_bytes(int nmax) { return fix_tile_bytes(nmax); }

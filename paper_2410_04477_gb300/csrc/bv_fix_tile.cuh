@@ -109,7 +109,10 @@ __device__ __forceinline__ bool pair_wait(uint64_t* mb, uint32_t parity) {
 // reciprocal square root.  Two columns a turn and the registers moved down by one, so that the
 // code stays small: unrolled over the 16 columns, this and the row loop below ran at the rate
 // of instruction fetches (10,000 clocks a tile and a row pass).  The pivots and the data row's
-// entries (row N, if it lies in the tile) are stored.
+// entries (row N, if it lies in the tile) are stored.  PART (the one-warp CTAs, in which nobody waits):
+// a last panel's columns beyond nc are left out; elsewhere the loop's known length is worth more (1.3%
+// at N = 47).
+template <bool PART>
 __device__ __forceinline__ void fix_diag(const longlong2* tile, int nc, int k0, int N, int lim, int lane, int4* Ld, FixRs* rsv,
                                          int64_t* piv, int64_t* zrow, uint64_t* mb, int& flags) {
     const int r = lane & 15, par = lane >> 4;
@@ -131,8 +134,9 @@ __device__ __forceinline__ void fix_diag(const longlong2* tile, int nc, int k0, 
     f.h = 0;
     f.hf = f.lf = 0.0f;
     const int4* lp = Ld;  // the column last factored
+    const int kend = PART ? (nc + 1) >> 1 : 8;
 #pragma unroll 1
-    for (int k = 0; k < 8; ++k) {
+    for (int k = 0; k < kend; ++k) {
 #pragma unroll
         for (int s = 0; s < 2; ++s) {
             const int c = 2 * k + s;
@@ -172,7 +176,7 @@ __device__ __forceinline__ void fix_diag(const longlong2* tile, int nc, int k0, 
             __syncwarp();
             lp = Ld + c * kLd + 2 * (k + s);
         }
-        pair_ready(mb + k, lane);  // (after the columns' __syncwarp)
+        if (!PART) pair_ready(mb + k, lane);  // (after the columns' __syncwarp)
 #pragma unroll
         for (int q = 0; q < 7; ++q) {
             a[q] = a[q + 1];
@@ -355,28 +359,49 @@ __device__ __noinline__ int64_t gen_direct(const DevTheta* th, double x, uint64_
     return (int64_t)((bvfix::mulhi64(rho, ratio) + 2) >> 2);
 }
 
+// What a tile (I, J) holds beside pairs of points, the data row and the identity, in the quarters s of
+// the mask: rows 8 (s & 1) .., columns 8 (s >> 1) ...
+__device__ __forceinline__ void fill_rest(longlong2* tp, int I, int J, int mask, int N, int lane, const int64_t* yfix) {
+#pragma unroll 1
+    for (int s = 0; s < 4; ++s) {
+        if (!(mask >> s & 1)) continue;
+        const int r = 16 * I + (lane >> 2) + 8 * (s & 1), c = 16 * J + 8 * (s >> 1) + 2 * (lane & 3);
+        int64_t v[2];
+#pragma unroll
+        for (int e = 0; e < 2; ++e) v[e] = r == N && c + e < N ? yfix[c + e] : c + e == r ? 1ll << bvfix::kUnitC : 0;
+        tp[s * 32 + lane] = make_longlong2(v[0], v[1]);
+    }
+}
+
 // One covariance tile (I, J), one warp, entries in matrix units: rows and columns of the points
 // at px (pre-scaled coordinates, dimension k at k np), row N the data row yfix.  GEN = 0: the
 // closed forms; 1: those and the general smoothness through its table gt; 2: the general
 // smoothness through K_nu itself.  PAD: rows m .. m16 - 1 are no points but rows of the identity.
-template <int GEN, bool PAD>
+// PART: as in fix_diag.
+template <int GEN, bool PAD, bool PART>
 __device__ __forceinline__ void fix_fill(longlong2* tp, int I, int J, int m, int m16, int N, int lane, const double* px, int d,
                                          const int64_t* yfix, const DevTheta* th, int nu_code, uint64_t ratio, const int64_t* gt,
                                          const uint64_t* tA, const uint64_t* tB, int& flags) {
     const int g = lane >> 2, t = lane & 3;
+    // Column halves: entries (g + 8 i, c0 + e), four chains.  PART: a tile row of the data row alone takes
+    // no pass, one of at most eight rows a single pass over them (both halves), and a half without
+    // points none.
+    const bool top = PART && 16 * I + 8 > N;
+    const int hend = !PART ? 2 : 16 * I >= N ? 0 : top || 16 * J + 8 >= N ? 1 : 2;
 #pragma unroll 1
-    for (int h = 0; h < 2; ++h) {  // column halves: entries (g + 8 i, c0 + e), four chains
-        const int c0 = 16 * J + 8 * h + 2 * t, r0 = 16 * I + g;
-        const int ra = min(r0, N - 1), rb = min(r0 + 8, N - 1), ca = min(c0, N - 1), cb = min(c0 + 1, N - 1);
+    for (int h = 0; h < hend; ++h) {
+        const int c0 = 16 * J + 8 * h + 2 * t, r0 = 16 * I + g, c1 = top ? c0 + 8 : c0, r1 = top ? r0 : r0 + 8;
+        const int ra = min(r0, N - 1), rb = min(r1, N - 1);
+        const int ca = min(c0, N - 1), cb = min(c0 + 1, N - 1), cc = min(c1, N - 1), cd = min(c1 + 1, N - 1);
         double acc[4] = {0.0, 0.0, 0.0, 0.0};
 #pragma unroll 1
         for (int k = 0; k < d; ++k) {
             const double* pk1 = px + k * N;
-            const double xa = pk1[ra], xb = pk1[rb], ya = pk1[ca], yb = pk1[cb];
+            const double xa = pk1[ra], xb = pk1[rb], ya = pk1[ca], yb = pk1[cb], yc = pk1[cc], yd = pk1[cd];
             acc[0] = fma(xa - ya, xa - ya, acc[0]);
             acc[1] = fma(xa - yb, xa - yb, acc[1]);
-            acc[2] = fma(xb - ya, xb - ya, acc[2]);
-            acc[3] = fma(xb - yb, xb - yb, acc[3]);
+            acc[2] = fma(xb - yc, xb - yc, acc[2]);
+            acc[3] = fma(xb - yd, xb - yd, acc[3]);
         }
         int64_t v[4];
         if (GEN && nu_code == NU_GENERAL) {
@@ -405,7 +430,7 @@ __device__ __forceinline__ void fix_fill(longlong2* tp, int I, int J, int m, int
         }
 #pragma unroll
         for (int e = 0; e < 4; ++e) {
-            const int r = r0 + 8 * (e >> 1), c = c0 + (e & 1);
+            const int r = e < 2 ? r0 : r1, c = (e < 2 ? c0 : c1) + (e & 1);
             const int ex = (int)(bvfix::dbits(acc[e]) >> 52);
             if (ex == 0x7ff) flags |= kFail;
             if (ex == 0) v[e] = (int64_t)(tA[0] >> 2);
@@ -414,8 +439,9 @@ __device__ __forceinline__ void fix_fill(longlong2* tp, int I, int J, int m, int
             if (r == N && c < N) v[e] = yfix[c];
         }
         tp[(2 * h) * 32 + lane] = make_longlong2(v[0], v[1]);
-        tp[(2 * h + 1) * 32 + lane] = make_longlong2(v[2], v[3]);
+        tp[(top ? 2 : 2 * h + 1) * 32 + lane] = make_longlong2(v[2], v[3]);
     }
+    if (PART && hend < 2) fill_rest(tp, I, J, hend == 0 ? 15 : top ? 10 : 12, N, lane, yfix);
 }
 
 __device__ __forceinline__ int64_t y_step(int64_t v) { return (v + (1ll << (kYStep - 1))) >> kYStep; }
@@ -440,7 +466,7 @@ __device__ __forceinline__ void fix_rescale(longlong2* tiles, int p, int TC, int
 // Eliminate the first NP panels of 16 columns of the T x T tiles (rows 0 .. N, row N the data
 // row; TC tile columns of points) by one CTA.  Warp 0 factors a panel's diagonal tile; the
 // other warps follow it, two columns behind, on the rows below, one row a thread (rows beyond
-// one a thread, in the largest blocks, after that); then all update the trailing tiles.  A data
+// one a thread, in the largest blocks, after that; a CTA of one warp does them after the tile); then all update the trailing tiles.  A data
 // entry out of range scales the data row down and the panel, whose tiles are as they were, is
 // solved again.  Returns the scalings, or -1 at a bad pivot (or more than kYMax scalings).
 template <int NT>
@@ -452,8 +478,16 @@ __device__ __forceinline__ int fix_panels(longlong2* tiles, int T, int TC, int N
     for (int p = 0; p < NP; ++p) {
         const int k0 = p << 4, nc = min(16, N - k0), rows = (T - p - 1) << 4;
         int flags = 0;
-        if (warp == 0) {
-            fix_diag(tiles + ftile(p, p) * 128, nc, k0, N, lim, lane, Ld, rsv, piv, zrow, mb, flags);
+        if (NT == 32) {
+            fix_diag<true>(tiles + ftile(p, p) * 128, nc, k0, N, lim, lane, Ld, rsv, piv, zrow, mb, flags);
+#pragma unroll 1
+            for (int rw = lane; rw < rows; rw += 32) {
+                const int I = p + 1 + (rw >> 4);
+                fix_row(tiles + ftile(I, p) * 128, Ld, rsv, rw & 15, (I << 4) + (rw & 15) == N, lim, zrow + k0, nc, false, mb,
+                        parity, dig + (rw >> 4) * (kDigB / 4), flags);
+            }
+        } else if (warp == 0) {
+            fix_diag<false>(tiles + ftile(p, p) * 128, nc, k0, N, lim, lane, Ld, rsv, piv, zrow, mb, flags);
         } else {
 #pragma unroll 1
             for (int rw = tid - 32; rw < rows; rw += NT - 32) {

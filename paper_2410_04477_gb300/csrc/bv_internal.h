@@ -155,9 +155,9 @@ int bv_tc_occupancy(int threads, size_t smem);
 cudaError_t bv_tc_launch(int threads, int grid, size_t smem, const LLArgs& a, cudaStream_t s);
 
 // FP64 kernel in fixed point with tensor-core updates (bv_fix_ll.cu), kinds 7 to 9.
-int bv_fix_kind(int nmax, int d);
+int bv_fix_kind(int nmax, int total, int num_sms, int d);
 int bv_fix_max_n(int d);
-int bv_fix_threads(int nmax, int nwork, int num_sms);
+int bv_fix_threads(int kind, int nmax, int nwork, int num_sms);
 size_t bv_fix_smem_bytes(int kind, int nmax, int d);
 size_t bv_fix_slot_bytes(int nmax);
 int bv_fix_occupancy(int kind, int threads, size_t smem);

@@ -327,7 +327,7 @@ __global__ void __launch_bounds__(kPredFixNT, 4) k_pred_fix(PredArgs a) {
             int I, J;
             tri_rc(q, I, J);
             if (J >= TC) continue;
-            fix_fill<GEN ? 2 : 0, true>(tiles + q * 128, I, J, m, m16, N, lane, px, d, yfix, &a.th, a.th.nu_code, ratio, nullptr,
+            fix_fill<GEN ? 2 : 0, true, false>(tiles + q * 128, I, J, m, m16, N, lane, px, d, yfix, &a.th, a.th.nu_code, ratio, nullptr,
                                         tA, tB, flags);
         }
         bool failed = __syncthreads_or(flags);
