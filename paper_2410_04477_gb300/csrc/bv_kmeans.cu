@@ -547,8 +547,10 @@ int bv_kmeans_device(const double* d_locs, int64_t n_tot, int64_t off, int64_t n
     const int64_t per = (n + kKppCtas * kChunk - 1) / (kKppCtas * kChunk);  // points a thread of the one-launch form
     if (per <= kKppMaxP) {
         auto kern = per == 1 ? k_kpp_all<1> : per == 2 ? k_kpp_all<2> : per == 3 ? k_kpp_all<3> : per == 4 ? k_kpp_all<4> : k_kpp_all<5>;
+        // (the attribute is the kernel's, not the call's: the same for all dimensions, so that calls of
+        // several threads do not take it from one another)
         const size_t sm = sizeof(double) * kChunk * per * d;
-        BV_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
+        BV_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(sizeof(double) * kChunk * per * 3)));
         kern<<<kKppCtas, kChunk, sm, s>>>(d_locs, n_tot, off, n, d, sc, (float)amax, stream, k, d_cent);
         BV_CUDA(cudaGetLastError());
     } else {
