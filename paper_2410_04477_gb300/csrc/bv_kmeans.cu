@@ -26,6 +26,8 @@
 #include <cuda_runtime.h>
 #include <math.h>
 #include <stdint.h>
+#include <stdlib.h>
+#include <string.h>
 
 #include <algorithm>
 #include <vector>
@@ -466,6 +468,28 @@ __global__ void __cluster_dims__(kKppCtas, 1, 1) __launch_bounds__(kChunk, 1)
 
 }  // namespace
 
+// Whether a cluster of the one-launch seeding can be placed on this device (a part of one may have no eight
+// SMs of a cluster's size, or not the shared memory).  BV_FAULT_CLUSTER says no, for tests.
+template <class K>
+static bool kpp_cluster_fits(K kern, size_t smem) {
+    const char* f = getenv("BV_FAULT_CLUSTER");
+    if (f && *f && strcmp(f, "0") != 0) return false;
+    if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess) {
+        cudaGetLastError();
+        return false;
+    }
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(kKppCtas);
+    cfg.blockDim = dim3(kChunk);
+    cfg.dynamicSmemBytes = smem;
+    int n = 0;
+    if (cudaOccupancyMaxActiveClusters(&n, kern, &cfg) != cudaSuccess) {
+        cudaGetLastError();
+        return false;
+    }
+    return n > 0;
+}
+
 static int ceil_log2_u64(uint64_t v) {
     int e = 0;
     while (e < 64 && ((uint64_t)1 << e) < v) ++e;
@@ -545,12 +569,11 @@ int bv_kmeans_device(const double* d_locs, int64_t n_tot, int64_t off, int64_t n
                                     cudaMemcpyDeviceToDevice, s));
     }
     const int64_t per = (n + kKppCtas * kChunk - 1) / (kKppCtas * kChunk);  // points a thread of the one-launch form
-    if (per <= kKppMaxP) {
-        auto kern = per == 1 ? k_kpp_all<1> : per == 2 ? k_kpp_all<2> : per == 3 ? k_kpp_all<3> : per == 4 ? k_kpp_all<4> : k_kpp_all<5>;
-        // (the attribute is the kernel's, not the call's: the same for all dimensions, so that calls of
-        // several threads do not take it from one another)
+    // (the shared-memory limit is the kernel's, not the call's: the same for all dimensions, so that calls
+    // of several threads do not take it from one another)
+    auto kern = per == 1 ? k_kpp_all<1> : per == 2 ? k_kpp_all<2> : per == 3 ? k_kpp_all<3> : per == 4 ? k_kpp_all<4> : k_kpp_all<5>;
+    if (per <= kKppMaxP && kpp_cluster_fits(kern, sizeof(double) * kChunk * per * 3)) {
         const size_t sm = sizeof(double) * kChunk * per * d;
-        BV_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(sizeof(double) * kChunk * per * 3)));
         kern<<<kKppCtas, kChunk, sm, s>>>(d_locs, n_tot, off, n, d, sc, (float)amax, stream, k, d_cent);
         BV_CUDA(cudaGetLastError());
     } else {
