@@ -414,7 +414,7 @@ __device__ __forceinline__ void fix_fill(longlong2* tp, int I, int J, int m, int
                 } else {
                     const Dist x = bvfix::dist_fix(bvfix::dbits(ac));
                     w = bvfix::matern_gen_fix<GTAB_DEG, -GTAB_E0>(x, gt, tA, tB);
-                    if (x.q < 1 + GTAB_E0 && x.q > -500)  // nearer than the table: K_nu itself
+                    if (x.q < 1 + GTAB_E0 && x.q > -511)  // nearer than the table, and not 0: K_nu itself
                         w = gen_direct(th, bvfix::scale2((double)x.X, x.q - 63), ratio);
                 }
                 if (e == 0) v[0] = w;
