@@ -368,7 +368,8 @@ __global__ void __launch_bounds__(kPredFixNT, 4) k_pred_fix(PredArgs a) {
 // accumulating sum z and sum z^2 replaces the two passes over the draws; and a whole pair's
 // z^2 sum to rho^2.  The logarithm, root, sine and cosine are taken in fixed point (bv_fix.cuh):
 // in FP64 their 110 operations a pair, at 2 lanes a clock and SM, were the kernel's time.
-// Sums: z in units 2^-50 (rounded: 2^-51 of draws of size 1), rho^2 exactly.
+// Sums: z in units 2^-54, so that a pair is rounded by 2^-55 (FP64 rounds draws of size 1 by 2^-54);
+// rho^2, itself within 2^-57, exactly.
 __global__ void __launch_bounds__(256) k_cond_sim(const double* __restrict__ mean, const double* __restrict__ var,
                                                   const double* __restrict__ ytrue, int64_t n_star, int R,
                                                   uint64_t stream, double zc, const bvfix::SimTab* __restrict__ tab,
@@ -388,18 +389,18 @@ __global__ void __launch_bounds__(256) k_cond_sim(const double* __restrict__ mea
     for (int64_t j = w0; j < n_star; j += nw) {
         const uint64_t c0 = (uint64_t)j * (uint64_t)half;
         double s1 = 0.0, s2 = 0.0;
-        for (int k0 = lane; k0 < whole; k0 += 32 * 256) {  // (256 pairs a lane stay in range)
+        for (int k0 = lane; k0 < whole; k0 += 32 * 16) {  // (16 pairs a lane stay in range: 16 x 12.2 < 2^8)
             int64_t z = 0;
             uint64_t vh = 0, vl = 0;
-            const int k1 = min(whole, k0 + 32 * 256);
+            const int k1 = min(whole, k0 + 32 * 16);
             for (int k = k0; k < k1; k += 32) {
                 const bvfix::Pair p = pair(c0 + (uint64_t)k);
                 const int64_t P = bvfix::mulh((int64_t)(p.X >> 1), p.cs + p.sn);  // units 2^(q - 60)
-                z += (P + (1ll << (9 - p.q))) >> (10 - p.q);
+                z += (P + (1ll << (5 - p.q))) >> (6 - p.q);
                 vh += p.V >> 32;
                 vl += (uint32_t)p.V;
             }
-            s1 += (double)z * 0x1p-50;
+            s1 += (double)z * 0x1p-54;
             s2 += (double)vh * 0x1p-24 + (double)vl * 0x1p-56;
         }
         if (half > whole && lane == 0) {  // the last draw of an odd number
