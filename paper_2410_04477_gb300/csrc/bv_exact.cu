@@ -84,7 +84,7 @@ __global__ void __launch_bounds__(256) k_ex_fill(ExArgs a, int64_t ntiles) {
             }
             const int ex = (int)(bvfix::dbits(acc) >> 52);
             if ((ex & 0x7ff) == 0x7ff && a.th.nu_code != NU_HALF) atomicOr(a.flags, kFail);  // (as in fix_fill)
-            if (GEN) v[e] = gen_direct(&a.th, sqrt(acc), a.th.diag_ratio);
+            if (GEN) v[e] = c < r && r < n ? gen_direct(&a.th, sqrt(acc), a.th.diag_ratio) : 0;
             else if (ex == 0) v[e] = (int64_t)(tA[0] >> 2);
             else {
                 const Dist x[1] = {bvfix::dist_fix(bvfix::dbits(acc))};

@@ -135,7 +135,7 @@ __global__ void __launch_bounds__(NT, WARPS * 32 / NT) k_ll_fix(LLArgs a) {
             int I, J;
             tri_rc(q, I, J);
             if (J >= TC) continue;
-            fix_fill<GEN ? 1 : 0, false, NT == 32>(tiles + q * 128, I, J, N, N, N, lane, px, d, yfix, a.theta + ds, th.nu_code, ratio,
+            fix_fill<GEN, false, NT == 32>(tiles + q * 128, I, J, N, N, N, lane, px, d, yfix, a.theta + ds, th.nu_code, ratio,
                                          a.gtabi + (int64_t)ds * GTAB_SIZE, tA, tB, flags);
         }
         bool fail = __syncthreads_or(flags);

@@ -374,11 +374,10 @@ __device__ __forceinline__ void fill_rest(longlong2* tp, int I, int J, int mask,
 }
 
 // One covariance tile (I, J), one warp, entries in matrix units: rows and columns of the points
-// at px (pre-scaled coordinates, dimension k at k np), row N the data row yfix.  GEN = 0: the
-// closed forms; 1: those and the general smoothness through its table gt; 2: the general
-// smoothness through K_nu itself.  PAD: rows m .. m16 - 1 are no points but rows of the identity.
+// at px (pre-scaled coordinates, dimension k at k np), row N the data row yfix.  GEN: the
+// general smoothness beside the closed forms, through its table gt.  PAD: rows m .. m16 - 1 are no points but rows of the identity.
 // PART: as in fix_diag.
-template <int GEN, bool PAD, bool PART>
+template <bool GEN, bool PAD, bool PART>
 __device__ __forceinline__ void fix_fill(longlong2* tp, int I, int J, int m, int m16, int N, int lane, const double* px, int d,
                                          const int64_t* yfix, const DevTheta* th, int nu_code, uint64_t ratio, const int64_t* gt,
                                          const uint64_t* tA, const uint64_t* tB, int& flags) {
@@ -408,15 +407,10 @@ __device__ __forceinline__ void fix_fill(longlong2* tp, int I, int J, int m, int
 #pragma unroll 1
             for (int e = 0; e < 4; ++e) {
                 const double ac = e == 0 ? acc[0] : e == 1 ? acc[1] : e == 2 ? acc[2] : acc[3];
-                int64_t w;
-                if (GEN == 2) {
-                    w = gen_direct(th, dist_of(ac), ratio);
-                } else {
-                    const Dist x = bvfix::dist_fix(bvfix::dbits(ac));
-                    w = bvfix::matern_gen_fix<GTAB_DEG, -GTAB_E0>(x, gt, tA, tB);
-                    if (x.q < 1 + GTAB_E0 && x.q > -511)  // nearer than the table, and not 0: K_nu itself
-                        w = gen_direct(th, bvfix::scale2((double)x.X, x.q - 63), ratio);
-                }
+                const Dist x = bvfix::dist_fix(bvfix::dbits(ac));
+                int64_t w = bvfix::matern_gen_fix<GTAB_DEG, -GTAB_E0>(x, gt, tA, tB);
+                if (x.q < 1 + GTAB_E0 && x.q > -511)  // nearer than the table, and not 0: K_nu itself
+                    w = gen_direct(th, bvfix::scale2((double)x.X, x.q - 63), ratio);
                 if (e == 0) v[0] = w;
                 else if (e == 1) v[1] = w;
                 else if (e == 2) v[2] = w;

@@ -269,6 +269,10 @@ __global__ void __launch_bounds__(kPredNT) k_pred(PredArgs a) {
 // 0.79 ms, before 2.8.  Tiles in a global-memory slot of the CTA.  The mean is left by the
 // elimination at the data row's scale; the limit of its solved entries keeps it in range.
 constexpr int kPredFixNT = 128;
+// Where the tiles hold columns c and c + 1 (c even, or c - 1 and c) of row r.
+__device__ __forceinline__ int entry_at(int r, int c) {
+    return ftile(r >> 4, c >> 4) * 128 + (((c >> 3) & 1) * 2 + ((r >> 3) & 1)) * 32 + 4 * (r & 7) + ((c & 7) >> 1);
+}
 template <bool GEN>
 __global__ void __launch_bounds__(kPredFixNT, 4) k_pred_fix(PredArgs a) {
     constexpr int NT = kPredFixNT;
@@ -327,8 +331,32 @@ __global__ void __launch_bounds__(kPredFixNT, 4) k_pred_fix(PredArgs a) {
             int I, J;
             tri_rc(q, I, J);
             if (J >= TC) continue;
-            fix_fill<GEN ? 2 : 0, true, false>(tiles + q * 128, I, J, m, m16, N, lane, px, d, yfix, &a.th, a.th.nu_code, ratio, nullptr,
-                                        tA, tB, flags);
+            if (GEN) fill_rest(tiles + q * 128, I, J, 15, N, lane, yfix);
+            else fix_fill<false, true, false>(tiles + q * 128, I, J, m, m16, N, lane, px, d, yfix, &a.th, a.th.nu_code, ratio, nullptr, tA,
+                                          tB, flags);
+        }
+        if (GEN) {
+            // K_nu costs some hundred times a closed form: the pairs of points alone, one a thread (whole
+            // tiles, with the other triangle and the padding, took 4 to 10 times as long up to m = 30)
+            __syncthreads();
+            const int P = m + b;
+            for (int f = tid; f < ((P * (P - 1)) >> 1); f += NT) {
+                int r, c;
+                tri_rc(f, r, c);
+                ++r;
+                r = r < m ? r : m16 + (r - m);
+                c = c < m ? c : m16 + (c - m);
+                double acc = 0.0;
+                for (int k = 0; k < d; ++k) {
+                    const double t = px[k * N + r] - px[k * N + c];
+                    acc = fma(t, t, acc);
+                }
+                if ((__double2hiint(acc) & 0x7ff00000) == 0x7ff00000) flags |= kFail;
+                longlong2* e = tiles + entry_at(r, c);
+                const int64_t v = gen_direct(&a.th, dist_of(acc), ratio);
+                if (c & 1) e->y = v;
+                else e->x = v;
+            }
         }
         bool failed = __syncthreads_or(flags);
         if (!failed) {
@@ -337,7 +365,7 @@ __global__ void __launch_bounds__(kPredFixNT, 4) k_pred_fix(PredArgs a) {
             E += kYStep * scaled;
         }
         const auto entry = [&](int r, int c) {
-            const longlong2 v = tiles[ftile(r >> 4, c >> 4) * 128 + (((c >> 3) & 1) * 2 + ((r >> 3) & 1)) * 32 + 4 * (r & 7) + ((c & 7) >> 1)];
+            const longlong2 v = tiles[entry_at(r, c)];
             return (c & 1) ? v.y : v.x;
         };
         const double vs = D * 0x1p-60, ms = ldexp(sqrt(D), E - bvfix::kUnitC);
