@@ -83,7 +83,8 @@ __global__ void __launch_bounds__(256) k_ex_fill(ExArgs a, int64_t ntiles) {
                 acc = fma(dt, dt, acc);
             }
             const int ex = (int)(bvfix::dbits(acc) >> 52);
-            if ((ex & 0x7ff) == 0x7ff && a.th.nu_code != NU_HALF) atomicOr(a.flags, kFail);  // (as in fix_fill)
+            // a squared distance beyond FP64's range: e^-x and K_nu give 0 there, the other forms have no value
+            if ((ex & 0x7ff) == 0x7ff && a.th.nu_code != NU_HALF && !GEN) atomicOr(a.flags, kFail);
             if (GEN) v[e] = c < r && r < n ? gen_direct(&a.th, sqrt(acc), a.th.diag_ratio) : 0;
             else if (ex == 0) v[e] = (int64_t)(tA[0] >> 2);
             else {

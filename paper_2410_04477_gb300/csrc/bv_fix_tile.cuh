@@ -426,8 +426,7 @@ __device__ __forceinline__ void fix_fill(longlong2* tp, int I, int J, int m, int
         for (int e = 0; e < 4; ++e) {
             const int r = e < 2 ? r0 : r1, c = (e < 2 ? c0 : c1) + (e & 1);
             const int ex = (int)(bvfix::dbits(acc[e]) >> 52);
-            // a squared distance beyond FP64's range: rho = e^-x is 0 (v is), the other forms have no value
-            if ((ex & 0x7ff) == 0x7ff && nu_code != NU_HALF) flags |= kFail;
+            if ((ex & 0x7ff) == 0x7ff) flags |= kFail;  // a squared distance beyond FP64's range
             if (ex == 0) v[e] = (int64_t)(tA[0] >> 2);
             if (PAD && ((r >= m && r < m16) || (c >= m && c < m16))) v[e] = 0;
             if (c >= r || r >= N) v[e] = c == r ? 1ll << bvfix::kUnitC : 0;

@@ -1,5 +1,5 @@
-"""GPU: points whose scaled squared distance leaves FP64's range: at nu = 1/2 their covariance is 0, in
-the block likelihood, the exact one and in prediction, as with a merely large distance."""
+"""GPU: distances at the ends of FP64's range: squares that overflow, and the smallest whose squares are
+normal numbers."""
 import numpy as np
 import pytest
 
@@ -9,36 +9,32 @@ from paper_2410_04477_gb300 import synth
 pytestmark = pytest.mark.gpu
 
 
-def test_overflowing_distances():
+@pytest.mark.parametrize("nu", [0.5, 0.8, 1.5])
+def test_overflowing_distances(nu):
+    # the exact likelihood takes them as a covariance of 0 where the form has that limit (nu = 1/2, K_nu), as
+    # a merely large distance; the polynomial forms are refused, and the block likelihood refuses all
     import torch
     assert torch.cuda.is_available()
     from paper_2410_04477_gb300 import bv
     n = 24
-    locs = synth.locs_uniform(n, 2, 3)
-    near, far = locs.copy(), locs.copy()
+    near = synth.locs_uniform(n, 2, 3)
+    far = near.copy()
     near[-2:] = [[1e4, 0.0], [0.0, -1e4]]          # 1e5 ranges away: the covariance underflows
-    far[-2:] = [[1e200, 0.0], [0.0, -3e201]]       # the squared distance overflows
+    far[-2:] = [[1e200, 0.0], [0.0, -3e201]]
     y = synth.normal(3, 20, n)
-    th = (1.0, 0.1, 0.5, 1e-2)
-    got = []
-    for pts in (near, far):
-        with bv.Context() as ctx:
-            ctx.set_data(pts, y)
-            ctx.set_blocks(np.array([0, n], np.int64), np.arange(n, dtype=np.int32), locs[:1].copy())
-            ctx.select_neighbors(0)
-            got.append((ctx.loglik(bv.theta(*th), bv.BV_FP64), ctx.exact_loglik(bv.theta(*th))[0]))
-    want = oracle.exact_loglik(oracle.theta(*th), near, y)
-    assert got[0] == got[1]
-    np.testing.assert_allclose(got[0], want, rtol=1e-10)
-    # prediction at a far point from all observations: the prior
+    th = (1.0, 0.1, nu, 1e-2)
     with bv.Context() as ctx:
-        ctx.set_data(locs[:20], y[:20])
-        ctx.set_pred_locations(far[-2:])
-        ctx.build_pred_blocks(1, seed=1)
-        ctx.select_pred_neighbors(20)
-        mean, var, _ = ctx.predict(bv.theta(*th))
-    np.testing.assert_allclose(mean, 0.0, atol=1e-12)
-    np.testing.assert_allclose(var, 1.01, rtol=1e-14)
+        ctx.set_data(far, y)
+        ctx.set_blocks(np.array([0, n], np.int64), np.arange(n, dtype=np.int32), far[:1].copy())
+        ctx.select_neighbors(0)
+        with pytest.raises(bv.BVError):
+            ctx.loglik(bv.theta(*th), bv.BV_FP64)
+        if nu == 1.5:
+            with pytest.raises(bv.BVError):
+                ctx.exact_loglik(bv.theta(*th))
+        else:
+            want = oracle.exact_loglik(oracle.theta(*th), near, y)
+            assert abs(ctx.exact_loglik(bv.theta(*th))[0] - want) <= 1e-10 * abs(want)
 
 
 @pytest.mark.parametrize("x", [2.0 ** -499.5, 2.0 ** -503.5, 2.0 ** -508.5])
