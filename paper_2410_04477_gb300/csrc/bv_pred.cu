@@ -614,8 +614,13 @@ extern "C" int bv_select_pred_neighbors(bv_ctx* c, int32_t m, int64_t* nn_ptr, i
     int64_t maxF = 0;
     for (int64_t i = 0; i < p->nblk; ++i)
         maxF = std::max(maxF, (mi + 15) / 16 * 16 + p->h_bptr[i + 1] - p->h_bptr[i]);
-    // (without conditioning the covariance is the prior's, to FP64's relative accuracy: k_pred)
-    p->fix = mi > 0 && maxF < 4096 && fix_work_bytes((int)maxF, d) <= (size_t)kFixSmemCap;
+    // (without conditioning the covariance is the prior's, to FP64's relative accuracy: k_pred; and where
+    // the blocks are small: the fixed-point kernel takes whole panels of 16 neighbours and two tile rows at
+    // least.  20,000 sites, closed form, both sides in us: blocks of one with m = 8 255 (k_pred) and 585, 20 605
+    // and 1,035, 30 1,060 and 1,040, 60 3,920 and 2,310; blocks of 10 with m = 15 125 and 122, 20 152 and 176,
+    // 30 225 and 176.  Equal where a block has some 32 points)
+    p->fix = mi > 0 && (mi * p->nblk + p->n_star) >= 32 * p->nblk && maxF < 4096 &&
+             fix_work_bytes((int)maxF, d) <= (size_t)kFixSmemCap;
     p->max_n = p->fix ? maxF : maxN;
     int smem_n = 0;
     while (pred_doubles(smem_n + 1) * 8 <= (int64_t)kPredSmemCap) ++smem_n;

@@ -62,10 +62,11 @@ def test_pivot_of_coincident_points(tau2, sigma2):
             assert abs(ell - want) <= tol, (nu, ell, want)
             ell = ctx.exact_loglik(bv.theta(sigma2, 0.1, nu, tau2))[0]
             assert abs(ell - want) <= tol, (nu, ell, want)
-    # prediction there: the conditional variance is that pivot
+    # prediction there: the conditional variance is that pivot (with 39 far sites in the block, so that it
+    # takes the fixed-point kernel)
     with bv.Context() as ctx:
         ctx.set_data(locs[:1], np.zeros(1))
-        ctx.set_pred_locations(locs[:1])
+        ctx.set_pred_locations(np.concatenate([locs[:1], locs[:1] + 100.0 * np.arange(1, 40)[:, None]]))
         ctx.build_pred_blocks(1, seed=1)
         ctx.select_pred_neighbors(1)
         for nu in (0.5, 1.5, 2.5, 0.8):
