@@ -828,8 +828,8 @@ static LLArgs make_args(bv_ctx* c) {
 }
 
 // Bin edges of the fixed-point FP64 kernel: a block of N points has (N + 16) / 16 tile rows,
-// so a bin of N = 16 k .. 16 k + 15 holds blocks of one shared-memory footprint; four tile
-// rows to a bin beyond N = 255, where few blocks lie.
+// so a bin of N = 16 k .. 16 k + 15 holds blocks of one footprint; four tile rows to a bin beyond
+// N = 255, where few blocks lie.
 static std::vector<int> fix_edges(int d) {
     const int nsm = bv_fix_max_n(d);
     std::vector<int> edges;
@@ -854,7 +854,7 @@ static int set_grid(bv_ctx* c, BinPlan& bp) {
     }
     const int occ = bv_occupancy(bp.kind, bp.threads, bp.smem);
     if (occ <= 0) return BV_EINTERNAL;
-    const int64_t per_cta = (bp.kind == 3 || bp.kind == 4) ? bp.threads / 32 : 1;  // blocks in flight per CTA
+    const int64_t per_cta = bp.kind == 3 ? bp.threads / 32 : 1;  // blocks in flight per CTA
     bp.grid = (int)std::min<int64_t>((bp.nwork + per_cta - 1) / per_cta, (int64_t)occ * c->num_sms);
     return BV_OK;
 }
@@ -1130,7 +1130,7 @@ static int autotune(bv_ctx* c, int prec) {
         // kernel.  BV_KERNEL_FORM=cta, =warp or =tc restricts the choice to one form where it
         // exists (tests use it to check each kernel against the oracle).
         const char* form = getenv("BV_KERNEL_FORM");
-        const bool only_cta = form && (strcmp(form, "cta") == 0 || strcmp(form, "cta2") == 0);
+        const bool only_cta = form && strcmp(form, "cta") == 0;
         const bool only_warp = form && strcmp(form, "warp") == 0;
         const bool only_tc = form && strcmp(form, "tc") == 0;
         std::vector<std::pair<int, int>> cands;

@@ -79,8 +79,8 @@ struct DevTheta {
 // L1 + L2 = ln2/256, 2^{n/256} = 2^{floor(n/256)} tab[n mod 256].  Filled on the host in
 // long double.
 #define BV_EXP_TAB 256
-// work counters per group of launches (at most 15 shared-memory bins and one global-memory
-// bin each): FP64 bins, mixed bins, the mixed check's FP64 sample bins and its FP64 redo bins
+// work counters per group of launches (FP64 has at most 28 size bins and one of larger blocks, mixed
+// precision 16): FP64 bins, mixed bins, the mixed check's FP64 sample bins and its FP64 redo bins
 #define BV_WCTR_PER_PREC 32
 #define BV_WCTR_GROUPS 4
 struct ExpConsts {
@@ -134,10 +134,10 @@ struct LLArgs {
 struct BinPlan {
     int kind;            // 1: mixed (CTA per block), 2: large (global), 3: mixed (warp per
                          // block), 5: mixed with tensor-core updates (CTA per block),
-                         // 7: FP64 in fixed point, 8, 9: the same with its tiles in d_slots
-                         // (N <= 111, larger)
+                         // 7: FP64 in fixed point, tiles in shared memory (N <= 47), 8, 9:
+                         // the same with its tiles in d_slots (N <= 111, larger)
     int nmax;            // largest augmented size N = m + b in the bin
-    int threads;         // CTA size (autotuned)
+    int threads;         // CTA size (mixed: autotuned)
     int grid;            // CTAs launched
     size_t smem;         // dynamic shared memory bytes
     int32_t* d_work;     // device block ids (largest N first)

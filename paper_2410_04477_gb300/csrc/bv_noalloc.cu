@@ -95,8 +95,8 @@ __global__ void k_na_maxn(const int64_t* bptr, const int64_t* nptr, int64_t bc, 
     atomicMax(w + kMaxNSlot, (unsigned long long)(b + m));
 }
 
-// Same fused algorithm as the library's FP64 shared-memory kernel (augmented Cholesky
-// of [[Sigma^con, Sigma^cross, y_NN], [., Sigma^lk, y_B], [., ., *]]), with theta passed by
+// FP64 arithmetic, the block's packed triangle in shared memory: the augmented Cholesky of
+// [[Sigma^con, Sigma^cross, y_NN], [., Sigma^lk, y_B], [., ., *]], right-looking, with theta passed by
 // value, blocks taken in index order and the per-block results written to the scratch.
 template <int NT>
 __global__ void __launch_bounds__(NT) k_na_ll(const double* __restrict__ locs, int64_t n_tot, int d,
