@@ -53,7 +53,9 @@ typedef enum bv_status {
     BV_EINVAL = 1,    /* invalid argument (size, pointer, theta outside its domain)      */
     BV_ENOMEM = 2,    /* device or host allocation failed                                 */
     BV_ECUDA = 3,     /* a CUDA runtime call failed (bv_last_cuda_error has the text)     */
-    BV_ENOTPD = 4,    /* a block's covariance was not positive definite; ell = -inf       */
+    BV_ENOTPD = 4,    /* a block's covariance was not positive definite; ell = -inf.  A
+                         pivot of at most 2^-54 (sigma^2 + tau^2), less than FP64 resolves
+                         there, counts as not positive                                    */
     BV_ETIMEOUT = 5,  /* reserved: no entry point waits on the device with a time limit,
                          so none returns it; the value stays assigned so that codes keep
                          their meaning                                                    */
@@ -62,7 +64,11 @@ typedef enum bv_status {
 } bv_status;
 
 typedef enum bv_precision {
-    BV_FP64 = 0,  /* every step in FP64                                                    */
+    BV_FP64 = 0,  /* FP64 accuracy: blocks of up to about 900 points in 64-bit fixed point,
+                     larger ones in FP64.  In fixed point covariances, pivots and factor are
+                     held to 2^-60 of sigma^2 + tau^2, and a block's data to 2^-52 or less
+                     of the largest |y| among its points and its conditioning points (an
+                     outlier 1e10 times the rest leaves the others' terms about 1e-6)        */
     BV_MIXED = 1  /* covariance generation, triangular solves and Schur-complement updates
                      in FP32; log-determinant and quadratic form accumulated in FP64; an
                      FP64 check keeps every dataset's relative error within a stated
