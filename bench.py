@@ -34,19 +34,27 @@ sys.path.insert(0, ROOT)
 from paper_2410_04477_gb300 import synth  # noqa: E402
 
 UNIT = "evals/s"
+
+
+def _bf16_tflops():
+    """Dense BF16 GEMM rate of this kind of GPU: as measured beside the repository, else 1930."""
+    try:
+        with open(os.path.join(ROOT, "MEASURED_PEAKS.json")) as f:
+            return float(json.load(f)["bf16_tflops"])
+    except (OSError, KeyError, ValueError):
+        return 1930.3
+
+
 # FP64-accurate products through 10-bit digits: 21 FP16 products each, exact in FP32 sums, so
-# the roofline is the measured dense FP16/BF16 tensor rate over 21 (the FP64 pipe itself: 1.25)
-DIGIT_PAIRS, BF16_TFLOPS = 21, 1930.3
-FP64_PEAK_TFLOPS = BF16_TFLOPS / DIGIT_PAIRS
-FP64_PEAK_SOURCE = ("measured dense BF16 GEMM, 1930 TFLOP/s, over the 21 digit products of an FP64-accurate one "
-                    "(the FP64 pipe: 1.25 TFLOP/s nominal)")
+# the contraction's ceiling is the dense FP16/BF16 tensor rate over 21 (the FP64 pipe itself: 1.25;
+# mma.sync m16n8k16 issues at a third of it by probe, 644 TFLOP/s).  What bounds the kernels is
+# instruction issue around it: the covariance, the panels and the sums of digit products
+DIGIT_PAIRS = 21
+FP64_PEAK_TFLOPS = _bf16_tflops() / DIGIT_PAIRS
+FP64_PEAK_SOURCE = (f"measured dense BF16 GEMM, {FP64_PEAK_TFLOPS * DIGIT_PAIRS:.0f} TFLOP/s, over the 21 digit products of an "
+                    "FP64-accurate one (the FP64 pipe: 1.25 TFLOP/s nominal)")
 SM_COUNT, FP32_LANES, SM_MAX_MHZ = 152, 128, 2070.0
 FP32_PEAK_TFLOPS = SM_COUNT * FP32_LANES * 2 * SM_MAX_MHZ * 1e6 / 1e12  # 80.5 at max clock
-
-# DRAM bytes (read + write) of one evaluation's likelihood-kernel launches, summed over
-# the size bins, from an ncu capture (dram__bytes_read.sum + dram__bytes_write.sum);
-# reported as roofline.traffic for the workloads and precisions captured.
-NCU_TRAFFIC = {}
 
 WORKLOADS = {
     # batched plain FP64: 2e5 uniform points, bc 2e4, m 60 / 120, y from BV at m=400
@@ -614,7 +622,7 @@ def run_pred(args, w, log):
            "h2d_bytes_per_step": int((~hold).sum()) * 8, "d2h_bytes_per_step": n_star * 8 * 4 + 16}
     mean_pred = statistics.mean(pred_ms) / 1e3
     achieved = flops / mean_pred / 1e12
-    roof = {"bound": "tensor", "kernel": "k_pred_fix (one launch: covariance + partial augmented Cholesky of every "
+    roof = {"bound": "issue", "kernel": "k_pred_fix (one launch: covariance + partial augmented Cholesky of every "
             "prediction block)", "achieved": achieved, "peak": FP64_PEAK_TFLOPS, "unit": "TFLOP/s",
             "frac": achieved / FP64_PEAK_TFLOPS, "traffic": None,
             "peak_source": FP64_PEAK_SOURCE,
@@ -694,7 +702,7 @@ def run_kl(args, w, log):
     tot_ms = max_over_ranks(float(sum(ms)))
     value = ws * args.steps / (tot_ms / 1e3)
     achieved = flops / (statistics.mean(ms) / 1e3) / 1e12
-    roof = {"bound": "tensor", "kernel": "k_ex_diag + k_ex_rows + k_ex_update (tiled dense Cholesky, one exact evaluation)",
+    roof = {"bound": "issue", "kernel": "k_ex_diag + k_ex_rows + k_ex_update (tiled dense Cholesky, one exact evaluation)",
             "achieved": achieved, "peak": FP64_PEAK_TFLOPS, "unit": "TFLOP/s", "frac": achieved / FP64_PEAK_TFLOPS,
             "traffic": None, "flops_per_launch_sequence": flops,
             "peak_source": FP64_PEAK_SOURCE}
@@ -860,10 +868,9 @@ def main():
            "d2h_bytes_per_step": 8 * nd}
 
     achieved = info["flops"] / (mean_ms / 1e3) / 1e12
-    roof = {"bound": "tensor", "kernel": "k_ll_fix (all size bins) + reduction, one evaluation",
+    roof = {"bound": "issue", "kernel": "k_ll_fix (all size bins) + reduction, one evaluation",
             "achieved": achieved, "peak": FP64_PEAK_TFLOPS, "unit": "TFLOP/s",
-            "frac": achieved / FP64_PEAK_TFLOPS, "traffic": NCU_TRAFFIC.get((args.workload, args.precision)),
-            "traffic_unit": "bytes per evaluation (ncu dram__bytes_read.sum + dram__bytes_write.sum)",
+            "frac": achieved / FP64_PEAK_TFLOPS, "traffic": None,
             "peak_source": FP64_PEAK_SOURCE,
             "flops_per_eval": info["flops"], "cov_entries_per_eval": info["cov_entries"]}
     if prec == bv.BV_MIXED:

@@ -20,19 +20,20 @@
 // largest |y| / sqrt(D); where one is larger (the parameters are far from the data's), the row is
 // scaled further and the panel solved again.
 //
-// Against a 113-bit factorisation of the same scaled coordinates, the blocks' ell errs by
-// 8.4e-13 (RMS; n = 20,000, m = 60, nu = 3/2, tau^2 = 1e-4), FP64 arithmetic by 2.8e-12; at m =
-// 113 by 4.9e-13 against 1.9e-12.  Time of an evaluation, FP64 arithmetic and this kernel:
-//   n = 200,000, m = 60 (N about 70)        5.04 ms   2.40 ms
-//   n = 36,931, m = 113                     3.64      1.16
-//   n = 100,000, 3D, m = 200                42.4      9.35
-//   n = 50,000, blocks of 1, m = 30         2.36      1.54
-//   n = 100,000, m = 60, nu = 1.2           4.92      2.20
-//   n = 2,000, m = 30                       0.122     0.094
+// Against a 113-bit factorisation of the same scaled coordinates, the quadratic form and the log-
+// determinant err by 2.2e-14 and 2.8e-16 (RMS, relative; n = 4,000, m = 60, nu = 3/2, tau^2 = 1e-4), FP64
+// arithmetic by 1.4e-13 and 2.2e-15; classic Vecchia at m = 30 by 1.9e-14 and 1.4e-16 against 1.3e-13 and
+// 1.1e-14.  Time of an evaluation, FP64 arithmetic and this kernel:
+//   n = 200,000, m = 60 (N about 70)        5.09 ms   2.38 ms
+//   n = 36,931, m = 113                     3.58      1.16
+//   n = 100,000, 3D, m = 200                42.6      9.38
+//   n = 50,000, blocks of 1, m = 30         2.35      1.25
+//   n = 100,000, m = 60, nu = 1.2           4.93      2.25
+//   n = 2,000, m = 30                       0.126     0.096
 // What bounds it: for few blocks the pivots' chain (a tile's 16 pivots take some 12,000 clocks,
 // in which the other warps follow two columns behind); else instruction issue and fetch, shared
 // by the covariance, the panel rows and the sums of digit products, with the tensor cores busy
-// for a twentieth of the time at N about 70.  More warps an SM, and starting a panel's chain
+// for a twentieth of the time at N about 70 and an eightieth at N = 31.  More warps an SM, and starting a panel's chain
 // beside the update before it, were measured and lose; halving the code gained 3 to 4%.
 #include <cuda_runtime.h>
 #include <math.h>
@@ -47,8 +48,8 @@
 namespace {
 
 
-// GLOB: the tiles live in a global-memory slot of the CTA (they stay in L2), for blocks whose
-// triangle does not leave room in shared memory.
+// GLOB: the tiles live in a global-memory slot of the CTA (they stay in L2), where they would not
+// leave room for as many CTAs in shared memory.
 // WARPS: resident warps an SM that the registers leave room for: 20 (96 registers) up to N = 111,
 // where more blocks an SM hide the pivots' chains (n = 200,000, m = 60: 2.40 ms, with 16 2.50),
 // 16 (128 registers) beyond, where spills cost more (3D, m = 200: 10.2 ms, with 16 9.34); 24
@@ -184,7 +185,7 @@ cudaError_t fix_kernel(int kind, int threads, bool gen, FixKernel* k) {
 // CTA size: one warp for the diagonal tiles, the others for the rows below, with which four warps cover
 // blocks up to N = 111 in one pass and large ones take eight.  A bin of few blocks (two an SM) takes eight
 // as well: there a block's latency counts, not the SM's rate.  Up to three tile rows with tiles in the
-// workspace (8): one warp for everything, up to 20 of them an SM.
+// workspace (8): one warp for everything, 16 to 20 of them an SM.
 int bv_fix_threads(int kind, int nmax, int nwork, int num_sms) {
     if (kind == 7) return nwork <= 2 * num_sms ? 256 : 64;
     if (fix_tiles(nmax) <= 3) return 32;

@@ -261,18 +261,19 @@ __global__ void __launch_bounds__(kPredNT) k_pred(PredArgs a) {
     }
 }
 
+// Where the tiles hold entry (r, c), beside the one of column c ^ 1.
+__device__ __forceinline__ int entry_at(int r, int c) {
+    return ftile(r >> 4, c >> 4) * 128 + (((c >> 3) & 1) * 2 + ((r >> 3) & 1)) * 32 + 4 * (r & 7) + ((c & 7) >> 1);
+}
+
 // The same in fixed point (bv_fix_tile.cuh), for blocks whose panel digits fit in shared memory
-// (about 800 points): the m conditioning points are filled up to whole panels with rows of the
+// (about 900 points): the m conditioning points are filled up to whole panels with rows of the
 // identity, so that the first panels' elimination leaves the Schur complement in whole tiles.
 // k_pred spends its time on the FP64 pipe (2 lanes a clock and SM); this one uses the integer
 // pipe and the tensor cores: 2,000 blocks of m = 120 and 10 sites in
 // 0.79 ms, before 2.8.  Tiles in a global-memory slot of the CTA.  The mean is left by the
 // elimination at the data row's scale; the limit of its solved entries keeps it in range.
 constexpr int kPredFixNT = 128;
-// Where the tiles hold columns c and c + 1 (c even, or c - 1 and c) of row r.
-__device__ __forceinline__ int entry_at(int r, int c) {
-    return ftile(r >> 4, c >> 4) * 128 + (((c >> 3) & 1) * 2 + ((r >> 3) & 1)) * 32 + 4 * (r & 7) + ((c & 7) >> 1);
-}
 template <bool GEN>
 __global__ void __launch_bounds__(kPredFixNT, 4) k_pred_fix(PredArgs a) {
     constexpr int NT = kPredFixNT;
